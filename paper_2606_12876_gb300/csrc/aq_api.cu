@@ -107,12 +107,7 @@ aq_status check_ptrs(std::initializer_list<const void*> ps) {
 size_t gemm_ws_bytes(const Dims& d, int tokens) { return aq::gemm_ws_need(d, tokens); }
 
 size_t gemv_ws_bytes(const Dims& d, int batch) {
-    // Partial planes: S per token, or S per book and token for the largest prefix the
-    // table-lookup kernel serves at this batch.
-    size_t planes = (size_t)d.S * (size_t)batch;
-    const int lm = aq::lut_max_m(batch), mt = d.M < lm ? d.M : lm;
-    if (mt > 0 && aq::uses_lut(d, mt, batch)) planes = (size_t)d.S * (size_t)batch * (size_t)mt;
-    return aq::ws_partial_offset(d) + planes * (size_t)d.rows_pad * 4;
+    return aq::ws_partial_offset(d) + aq::gemv_ws_planes(d, batch) * (size_t)d.rows_pad * 4;
 }
 
 }  // namespace

@@ -40,20 +40,20 @@ constexpr size_t kWsStatusBytes = 256;
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline size_t ws_partial_offset(const Dims&) { return kWsStatusBytes; }
 
-// The table-lookup GEMV (2^8-entry books; batch 1 and 2 with prefixes up to kLutMaxM, batch
-// 3..4 with prefixes up to kLutMultiM: their two 64 KiB tables and five or more codebooks
-// leave room for a single code stage; batch 5..8 with prefixes up to kLut8M and fp16 tables,
-// when the layer has at least kLut8MinItems (slice, book, 32-row block) items, about 30 per SM:
-// below that an eight-token table build costs more than the tensor-core kernel's decode)
-// writes one partial plane per (slice, book, token); every other GEMV one per (slice, token).
-constexpr int kLutMaxM = 8, kLutMultiM = 4, kLut8M = 6;
-constexpr long long kLut8MinItems = 4560;
-inline int lut_max_m(int batch) {
-    return batch <= 2 ? kLutMaxM : batch <= 4 ? kLutMultiM : batch <= 8 ? kLut8M : 0;
-}
-inline bool uses_lut(const Dims& d, int m, int batch) {
-    if (d.B != 8 || m > lut_max_m(batch)) return false;
-    return batch <= 4 || (long long)d.S * m * d.RBc >= kLut8MinItems;
+// The table-lookup GEMV (2^8-entry books) serves one and two tokens, and writes one partial plane
+// per (slice, book, token); the 2^16-entry-book kernels write one per (slice, token); the
+// remaining GEMVs (gemv_cw, gemv_lut4) need no partial planes.
+constexpr int kLutMaxBatch = 2;
+
+// Partial planes that a GEMV workspace has room for. The size is part of the interface (callers
+// keep workspaces across releases), so it stays what earlier kernels needed: S planes per token,
+// times the books of the longest prefix up to 8 (batch 1..2), 4 (3..4) or 6 (5..8, for layers of
+// at least 4560 (slice, book, 32-row block) items) for 8-bit codes.
+inline size_t gemv_ws_planes(const Dims& d, int batch) {
+    const int lm = batch <= 2 ? 8 : batch <= 4 ? 4 : batch <= 8 ? 6 : 0, mt = d.M < lm ? d.M : lm;
+    size_t planes = (size_t)d.S * (size_t)batch;
+    if (d.B == 8 && mt > 0 && (batch <= 4 || (long long)d.S * mt * d.RBc >= 4560)) planes *= (size_t)mt;
+    return planes;
 }
 
 // Prefill GEMM workspace: [status block, 256 B: status word at 0, the dense form's weight
@@ -97,6 +97,10 @@ aq_status launch_decode(const Dims& d, int m, const void* planes, const void* bo
 aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* books,
                       const void* scales, const void* x, int x_dt, int batch, void* y,
                       int y_dt, void* ws, cudaStream_t st, const void* y_prev = nullptr);
+// The same for 2..16 tokens with 4- or 8-bit codes in one kernel (gemv_cw.cu).
+aq_status launch_cw(const Dims& d, int m, const void* planes, const void* books, const void* scales,
+                    const void* x, int x_dt, int batch, void* y, int y_dt, const void* y_prev,
+                    cudaStream_t st);
 // aq_gemv_group: n (<= 4) layers sharing x; ws[l] = layer l's workspace region.
 aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* planes,
                             const void* const* books, const void* const* scales, const void* x,

@@ -1,0 +1,436 @@
+// gemv_cw: y = x * W_m^T for 2..16 tokens with 4- and 8-bit codes (the prefix-m reconstruction
+// of Sec. 3.2 / Sec. 5; Y = W X of Sec. 2.2), one kernel per call.
+//
+// By linearity in the books (Sec. 5), x_g . (sum_k C_k[b_k]) = sum_k x_g . C_k[b_k], and a
+// 16-byte codeword is, as it stands, the eight weights of one row and group: it goes straight
+// into the A fragment of a 16-bit tensor-core multiply (mma.sync m16n8k16, fp32 accumulation),
+// with no sum, no conversion and no rounding of weights on the way. In lane 4g + c (g < 8,
+// c < 4) the fragment holds row g (and g + 8), and the four K positions that the lane owns in
+// each of two multiplies are bound to the two halves of the codeword of one group; the K order
+// of a multiply is free, so lane c walks the groups 8c .. 8c+7 of a 256-input slice, one per
+// step, and the B fragment of the step is the same group of the lane's token g: one 16-byte load.
+//
+// Bound: shared-memory wavefronts of the codeword gathers (16 bytes per code; one 16-byte load of
+// a warp is four wavefronts when no two of the eight lanes of a phase meet in a bank group). Each
+// codebook is staged in 2^cshift interleaved copies, lane L reading copy L mod 2^cshift: with
+// eight copies there are no conflicts whatever the codes (a single copy costs about 2.6 times the
+// wavefronts). At 8 codes per clock and SM the gate projection (14336 x 4096, m = 4) cannot take
+// less than 12.6 us; every other unit (issue 34 %, tensor pipe at 16 tokens 50 %) has slack.
+//
+// Work split: a warp's work item is a (32-row block, slice, book); a cluster of kc CTAs (16 warps
+// each) owns whole row blocks, its warps share the row block's (slice, book) units evenly in
+// slice-major order (so a warp's B fragments, 32 or 64 registers, are loaded once per slice), and
+// the warps' accumulators are added in a fixed order in shared memory (and over the cluster
+// through distributed shared memory). So the kernel writes y itself: no partial planes in the
+// workspace and no reduction launch. kc > 1 is for layers with too few row blocks for the SMs.
+//
+// Operand types: books and activations both fp16, or both bf16, are multiplied as they are. fp16
+// books with bf16 activations: every (token, slice) of x is scaled by a power of two that puts
+// its largest |x| in [2^14, 2^15) and rounded to fp16, which is exact for values within 2^29 of
+// the largest, and the slice's sums are scaled back when they are added to the total. bf16 books
+// with fp16 activations: the books are scaled the same way (one power of two for the m books).
+#include "aq_internal.cuh"
+#include "launch.cuh"
+#include "tc_ptx.cuh"
+
+namespace aq {
+namespace {
+
+constexpr int kCwWarps = 16;
+constexpr int kCwThreads = kCwWarps * 32;
+constexpr int kCwPitch = 36;       // floats per token in a warp's sums (4 of padding: no conflicts)
+
+struct CwArgs {
+    const uint8_t* planes;
+    const uint16_t *books, *scales, *x;
+    void* y;
+    const void* y_prev;            // added to the product (refinement), or null
+    int y_dt, scale_dt, m, batch, out, in, ng, rows_pad, RBc, S;
+    int cshift;                    // log2 of the interleaved copies of a codebook
+    int kc, nclusters;             // CTAs per cluster, clusters (row blocks are dealt to them in turn)
+    int static_weights;
+    size_t plane_bytes;
+};
+
+// Shared memory: books [m][2^B][2^cshift] x 16 B, codes 16 warps x 32 rows, the warps' sums (two
+// buffers of [16][8 NT][36] floats), the CTA's sums (two buffers of [8 NT][32]; clusters only).
+constexpr size_t cw_red_floats(int nt) { return (size_t)kCwWarps * 8 * nt * kCwPitch; }
+inline size_t cw_smem_bytes(int B, int m, int cshift, int nt) {
+    return ((size_t)m * 16 << B << cshift) + (size_t)kCwWarps * 32 * unit_bytes(B) +
+           (2 * cw_red_floats(nt) + 2 * 256 * (size_t)nt) * 4;
+}
+
+template <int DT>
+__device__ __forceinline__ void mma16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                      uint32_t b0, uint32_t b1) {
+    if constexpr (DT == AQ_F16)
+        asm(
+            "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+            "{%8, %9}, {%0, %1, %2, %3};"
+            : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+    else
+        asm(
+            "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+            "{%8, %9}, {%0, %1, %2, %3};"
+            : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Eight 16-bit values of type DT times sc (a power of two), as fp16.
+template <int DT>
+__device__ __forceinline__ uint4 scaled_to_f16(const uint4& v, float sc) {
+    float f[8];
+    unpack8<DT>(v, f);
+    return make_uint4(round_pack2<AQ_F16>(f[0] * sc, f[1] * sc), round_pack2<AQ_F16>(f[2] * sc, f[3] * sc),
+                      round_pack2<AQ_F16>(f[4] * sc, f[5] * sc), round_pack2<AQ_F16>(f[6] * sc, f[7] * sc));
+}
+
+template <int DT>
+__device__ __forceinline__ float max_abs8(const uint4& v) {
+    float f[8], mx = 0.0f;
+    unpack8<DT>(v, f);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) mx = fmaxf(mx, fabsf(f[e]));
+    return mx;
+}
+
+// The exponent e that puts mx * 2^-e in [2^14, 2^15); 0 for 0, clamped so that 2^e and 2^-e are floats.
+__device__ __forceinline__ int f16_exponent(float mx) {
+    return mx > 0.0f ? max(-100, min(100, exponent_of(mx) - 14)) : 0;
+}
+
+// The codes of a row's slice unit as stored (position p holds group (p + o) mod 32) in group order.
+template <int B>
+__device__ __forceinline__ void store_unrotated(unsigned char* buf, int row, const uint4 (&raw)[2]) {
+    if constexpr (B == 8) {
+        const uint32_t w[8] = {raw[0].x, raw[0].y, raw[0].z, raw[0].w, raw[1].x, raw[1].y, raw[1].z, raw[1].w};
+        uint32_t u[8];
+        unrotate_codes(w, row, u);
+        // the row's 16-byte halves change places in rows 4..7 of every eight: no bank conflicts
+        const int sw = (row >> 2) & 1;
+        *(uint4*)(buf + row * 32 + sw * 16) = make_uint4(u[0], u[1], u[2], u[3]);
+        *(uint4*)(buf + row * 32 + (sw ^ 1) * 16) = make_uint4(u[4], u[5], u[6], u[7]);
+    } else {
+        const uint32_t w[4] = {raw[0].x, raw[0].y, raw[0].z, raw[0].w};
+        const int r = row & 31, rw = r >> 3, rb = (r & 7) * 4;
+        uint32_t t[4], v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) t[i] = (rw & 1) ? w[(i + 3) & 3] : w[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = (rw & 2) ? t[(i + 2) & 3] : t[i];
+        uint4 u;
+        u.x = rb ? __funnelshift_l(v[3], v[0], rb) : v[0];
+        u.y = rb ? __funnelshift_l(v[0], v[1], rb) : v[1];
+        u.z = rb ? __funnelshift_l(v[1], v[2], rb) : v[2];
+        u.w = rb ? __funnelshift_l(v[2], v[3], rb) : v[3];
+        *(uint4*)(buf + row * 16) = u;
+    }
+}
+
+// The codes of groups 8c .. 8c+7 of a staged row: eight bytes (B = 8) or eight nibbles (B = 4).
+template <int B>
+__device__ __forceinline__ uint2 staged_codes(const unsigned char* buf, int row, int c) {
+    if constexpr (B == 8)
+        return *(const uint2*)(buf + row * 32 + (((c >> 1) ^ ((row >> 2) & 1)) * 16) + (c & 1) * 8);
+    else
+        return make_uint2(*(const uint32_t*)(buf + row * 16 + c * 4), 0u);
+}
+template <int B>
+__device__ __forceinline__ uint32_t code_of(const uint2& w, int j) {
+    if constexpr (B == 8) return prmt(j < 4 ? w.x : w.y, 0u, 0x4440u | (uint32_t)(j & 3));
+    else return (w.x >> (4 * j)) & 15u;
+}
+
+template <int B, int BDT, int XDT, int NT>
+__global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_constant__ CwArgs a) {
+    constexpr int UNIT = unit_bytes(B), NC = 1 << B, NTOK = 8 * NT;
+    constexpr int MDT = BDT == AQ_BF16 && XDT == AQ_BF16 ? AQ_BF16 : AQ_F16;   // operand type
+    constexpr bool kScaleX = XDT != MDT, kScaleB = BDT != MDT;
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ unsigned int s_bmax;
+    uint4* books_s = (uint4*)smem;
+    const int nslot = (a.m * NC) << a.cshift;
+    unsigned char* codes_s = smem + (size_t)nslot * 16;
+    float* red = (float*)(codes_s + kCwWarps * 32 * UNIT);
+    float* csum = red + 2 * cw_red_floats(NT);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = a.kc > 1 ? (int)cluster_rank() : 0;
+    const int cid = (int)blockIdx.x / a.kc;
+
+    // this warp's (slice, book) units u0 .. u1-1 of every row block of the cluster; u = s*m + k
+    const long long U = (long long)a.S * a.m;
+    const int nwarps = kCwWarps * a.kc, gw = rank * kCwWarps + warp;
+    const int u0 = (int)(U * gw / nwarps), u1 = (int)(U * (gw + 1) / nwarps);
+    const int s0 = u0 / a.m, k0 = u0 - s0 * a.m;
+    struct Item {
+        int rb, u, s, k;
+    };
+    auto next_item = [&](Item& it) {
+        if (++it.u == u1) {
+            it = Item{it.rb + a.nclusters, u0, s0, k0};
+        } else if (++it.k == a.m) {
+            it.k = 0;
+            ++it.s;
+        }
+    };
+    uint4 raw[2];
+    auto load_codes = [&](const Item& it) {
+        if (u0 < u1 && it.rb < a.RBc) {
+            const uint8_t* src = a.planes + (size_t)it.k * a.plane_bytes +
+                                 ((size_t)it.s * a.rows_pad + (size_t)it.rb * 32 + lane) * UNIT;
+            raw[0] = ld_stream_v4(src);
+            if constexpr (B == 8) raw[1] = ld_stream_v4(src + 16);
+        }
+    };
+    Item nxt{cid, u0, s0, k0};
+    float bfac = 1.0f;                                   // 2^f of the staged books (kScaleB)
+    auto stage_books = [&]() {
+        if constexpr (kScaleB) {
+            if (tid == 0) s_bmax = 0u;
+            __syncthreads();
+            float mx = 0.0f;
+            for (int i = tid; i < a.m * NC; i += kCwThreads)
+                mx = fmaxf(mx, max_abs8<BDT>(__ldg((const uint4*)a.books + i)));
+            atomicMax(&s_bmax, __float_as_uint(mx));     // non-negative floats order as integers
+            __syncthreads();
+            const int f = f16_exponent(__uint_as_float(s_bmax));
+            bfac = pow2f(f);
+            const float sc = pow2f(-f);
+            for (int i = tid; i < nslot; i += kCwThreads)
+                books_s[i] = scaled_to_f16<BDT>(__ldg((const uint4*)a.books + (i >> a.cshift)), sc);
+        } else {
+#pragma unroll 4
+            for (int i = tid; i < nslot; i += kCwThreads)
+                books_s[i] = __ldg((const uint4*)a.books + (i >> a.cshift));
+        }
+    };
+    if (a.static_weights) {   // read-only weights: requested before the preceding kernel has finished
+        load_codes(nxt);
+        stage_books();
+    }
+    pdl_wait();
+    pdl_launch_dependents();
+    if (!a.static_weights) {
+        load_codes(nxt);
+        stage_books();
+    }
+    __syncthreads();
+
+    const int g = lane >> 2, c = lane & 3;
+    unsigned char* buf = codes_s + warp * 32 * UNIT;
+    const uint32_t mul = 16u << a.cshift;
+    const uint32_t books_u = smem_u32(books_s) + ((uint32_t)(lane & ((1 << a.cshift) - 1)) << 4);
+    uint4 bf[NT][8];                                     // B fragments of slice cur_s
+    float fac[NT][2];                                    // (kScaleX) 2^e of tokens 2c, 2c+1
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) fac[nt][0] = fac[nt][1] = 1.0f;   // a warp without units
+    int cur_s = -1;
+    auto load_b = [&](int s) {
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            const int t = 8 * nt + g;
+            const uint4* src = (const uint4*)(a.x + (size_t)t * a.in) + s * 32 + 8 * c;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                bf[nt][j] = t < a.batch && s * 32 + 8 * c + j < a.ng ? __ldg(src + j) : make_uint4(0u, 0u, 0u, 0u);
+            if constexpr (kScaleX) {
+                float mx = 0.0f;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) mx = fmaxf(mx, max_abs8<XDT>(bf[nt][j]));
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                const int e = f16_exponent(mx);
+                const float sc = pow2f(-e), up = pow2f(e);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) bf[nt][j] = scaled_to_f16<XDT>(bf[nt][j], sc);
+                fac[nt][0] = __shfl_sync(0xffffffffu, up, 8 * c);
+                fac[nt][1] = __shfl_sync(0xffffffffu, up, 8 * c + 4);
+            }
+        }
+        cur_s = s;
+    };
+
+    int pass = 0;
+    for (int rb = cid; rb < a.RBc; rb += a.nclusters, ++pass) {
+        float acc[2][NT][4];
+        // The warps' sums of a pass, added in warp order. Two buffers: a pass's writes meet the sums
+        // that are read two passes earlier, which every thread finished before the last barrier.
+        float* rp = red + (pass & 1) * cw_red_floats(NT);
+        float* mine = rp + (size_t)warp * NTOK * kCwPitch;
+        bool first = true;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.0f;
+        // The accumulators into the warp's sums in shared memory; with kScaleX once per slice, times
+        // the slice's 2^e (added to the earlier slices'), else once at the end of the pass.
+        auto fold = [&]() {
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        float* p = mine + (8 * nt + 2 * c + (e & 1)) * kCwPitch + 16 * mt + 8 * (e >> 1) + g;
+                        if constexpr (kScaleX) {
+                            const float v = acc[mt][nt][e] * fac[nt][e & 1];
+                            *p = first ? v : *p + v;
+                            acc[mt][nt][e] = 0.0f;
+                        } else {
+                            *p = acc[mt][nt][e];
+                        }
+                    }
+            first = false;
+        };
+        for (int u = u0; u < u1; ++u) {
+            const int s = nxt.s, k = nxt.k;
+            store_unrotated<B>(buf, lane, raw);
+            __syncwarp();
+            next_item(nxt);
+            load_codes(nxt);                             // travels while this item is multiplied
+            if (s != cur_s) {
+                if (kScaleX && u > u0) fold();
+                load_b(s);
+            }
+            uint2 cw[4];
+#pragma unroll
+            for (int rr = 0; rr < 4; ++rr) cw[rr] = staged_codes<B>(buf, g + 8 * rr, c);
+            __syncwarp();                                // the buffer may be refilled
+            const uint32_t base = books_u + (uint32_t)k * (NC * mul);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                uint4 w[4];
+#pragma unroll
+                for (int rr = 0; rr < 4; ++rr) w[rr] = lds128(base + code_of<B>(cw[rr], j) * mul);
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) {
+                        mma16<MDT>(acc[mt][nt], w[2 * mt].x, w[2 * mt + 1].x, w[2 * mt].y, w[2 * mt + 1].y,
+                                   bf[nt][j].x, bf[nt][j].y);
+                        mma16<MDT>(acc[mt][nt], w[2 * mt].z, w[2 * mt + 1].z, w[2 * mt].w, w[2 * mt + 1].w,
+                                   bf[nt][j].z, bf[nt][j].w);
+                    }
+            }
+        }
+        fold();
+        __syncthreads();
+        const int i0 = a.kc > 1 ? rank * (32 * NTOK / a.kc) : 0;      // outputs this CTA finishes
+        const int i1 = a.kc > 1 ? i0 + 32 * NTOK / a.kc : 32 * NTOK;
+        float* cs = csum + (pass & 1) * 32 * NTOK;
+        float v = 0.0f;
+        if (tid < 32 * NTOK) {
+#pragma unroll
+            for (int w = 0; w < kCwWarps; ++w) v += rp[((size_t)w * NTOK + (tid >> 5)) * kCwPitch + (tid & 31)];
+            if (a.kc > 1) cs[tid] = v;
+        }
+        if (a.kc > 1) {
+            cluster_sync();
+            v = 0.0f;
+            if (tid >= i0 && tid < i1)
+                for (int r = 0; r < a.kc; ++r) {          // the CTAs' sums, in rank order
+                    float p;
+                    asm volatile("ld.shared::cluster.f32 %0, [%1];"
+                                 : "=f"(p) : "r"(map_to_rank(smem_u32(cs + tid), (uint32_t)r)) : "memory");
+                    v += p;
+                }
+        }
+        const int t = tid >> 5, o = rb * 32 + (tid & 31);
+        if (tid >= i0 && tid < i1 && t < a.batch && o < a.out) {
+            float r = v * bfac * bits_to_f32_rt(a.scales[o], a.scale_dt);
+            const size_t yi = (size_t)t * a.out + o;
+            if (a.y_prev)
+                r = (a.y_dt == AQ_F32 ? ((const float*)a.y_prev)[yi]
+                                      : bits_to_f32_rt(((const uint16_t*)a.y_prev)[yi], a.y_dt)) + r;
+            if (a.y_dt == AQ_F32) ((float*)a.y)[yi] = r;
+            else ((uint16_t*)a.y)[yi] = a.y_dt == AQ_F16 ? f32_to_bits<AQ_F16>(r) : f32_to_bits<AQ_BF16>(r);
+        }
+    }
+    if (a.kc > 1) cluster_sync();   // no CTA leaves while a peer may still read its sums
+}
+
+// Copies of a codebook (log2): eight while they fit next to the sums, else four.
+inline int cw_cshift(int B, int m) { return B == 4 || m <= 4 ? 3 : 2; }
+
+// CTAs per cluster: the split with the smallest estimated time of the busiest cluster, in clocks:
+// passes over its row blocks times the units of a warp (a unit's gathers are 128 wavefronts, plus
+// about 24 of staging, shared by the SM's active warps, or the latency of its eight steps) and the
+// reduction of a pass (with a cluster barrier when kc > 1). Clusters of 2, 4 and 8 that are
+// resident at once: 76, 36 and 16 on 152 SMs.
+inline int cw_cluster(const Dims& d, int m, int sms, int* nclusters) {
+    int best = 1;
+    double best_t = -1.0;
+    for (int kc = 1; kc <= 8; kc *= 2) {
+        int nc = kc == 1 ? sms : kc == 2 ? sms / 2 : kc == 4 ? sms * 9 / 38 : sms * 2 / 19;
+        if (nc > d.RBc) nc = d.RBc;
+        if (nc < 1) nc = 1;
+        const long long U = (long long)d.S * m;
+        const long long units = (U + 16 * kc - 1) / (16 * kc);
+        const long long active = U < 16 * kc ? (U + kc - 1) / kc : 16;
+        const double unit_clk = active * 152 > 900 ? active * 152.0 : 900.0;
+        const double t = (double)((d.RBc + nc - 1) / nc) * (units * unit_clk + (kc > 1 ? 1100.0 : 400.0));
+        if (best_t < 0.0 || t < best_t) {
+            best_t = t;
+            best = kc;
+            *nclusters = nc;
+        }
+    }
+    return best;
+}
+
+template <int B, int BDT, int XDT, int NT>
+aq_status run_cw(const Dims& d, CwArgs a, cudaStream_t st) {
+    DeviceInfo di;
+    if (aq_status e = device_info(&di); e != AQ_OK) return e;
+    auto kern = gemv_cw_kernel<B, BDT, XDT, NT>;
+    a.cshift = cw_cshift(B, a.m);
+    const size_t smem = cw_smem_bytes(B, a.m, a.cshift, NT);
+    int occ = 0;
+    if (aq_status e = prepare(kern, smem, kCwThreads, a.m, &occ); e != AQ_OK) return e;
+    a.kc = cw_cluster(d, a.m, di.sms, &a.nclusters);
+    return launch_pdl_cluster(a.kc, kern, dim3(a.nclusters * a.kc), dim3(kCwThreads), smem, st, a);
+}
+
+template <int B, int BDT, int XDT>
+aq_status run_cw_nt(const Dims& d, const CwArgs& a, cudaStream_t st) {
+    return a.batch <= 8 ? run_cw<B, BDT, XDT, 1>(d, a, st) : run_cw<B, BDT, XDT, 2>(d, a, st);
+}
+
+template <int B>
+aq_status run_cw_types(const Dims& d, const CwArgs& a, int x_dt, cudaStream_t st) {
+    if (d.book_dt == AQ_BF16)
+        return x_dt == AQ_BF16 ? run_cw_nt<B, AQ_BF16, AQ_BF16>(d, a, st) : run_cw_nt<B, AQ_BF16, AQ_F16>(d, a, st);
+    return x_dt == AQ_BF16 ? run_cw_nt<B, AQ_F16, AQ_BF16>(d, a, st) : run_cw_nt<B, AQ_F16, AQ_F16>(d, a, st);
+}
+
+}  // namespace
+
+aq_status launch_cw(const Dims& d, int m, const void* planes, const void* books, const void* scales,
+                    const void* x, int x_dt, int batch, void* y, int y_dt, const void* y_prev,
+                    cudaStream_t st) {
+    CwArgs a = {};
+    a.planes = (const uint8_t*)planes;
+    a.books = (const uint16_t*)books;
+    a.scales = (const uint16_t*)scales;
+    a.x = (const uint16_t*)x;
+    a.y = y;
+    a.y_prev = y_prev;
+    a.y_dt = y_dt;
+    a.scale_dt = d.scale_dt;
+    a.m = m;
+    a.batch = batch;
+    a.out = d.out;
+    a.in = d.in;
+    a.ng = d.ng;
+    a.rows_pad = d.rows_pad;
+    a.RBc = d.RBc;
+    a.S = d.S;
+    a.static_weights = (d.flags & AQ_LAYOUT_STATIC_WEIGHTS) ? 1 : 0;
+    a.plane_bytes = d.plane_bytes;
+    return d.B == 4 ? run_cw_types<4>(d, a, x_dt, st) : run_cw_types<8>(d, a, x_dt, st);
+}
+
+}  // namespace aq
