@@ -85,47 +85,88 @@ __global__ void beam_sym_kernel(const void* __restrict__ h, int h_dt, float* __r
 }
 
 // C[r][j] = sum_i A[r][i] * S[i][j] for r < rows, j < in (A = E of every prefix, rows = M*out).
-// 64 x 64 tiles, 16-deep k steps through shared memory, 4 x 4 outputs per thread; the row
-// tiles beyond gridDim.y are taken in turn by the same CTAs.
+// Bound: the fp32 FMA pipe (2 * M * out * in^2 operations on the CUDA cores). T x T tiles of C,
+// (T/16)^2 outputs per thread in packed fp32 pairs, 16-deep k steps: the next step's tiles travel
+// into registers while the current ones are multiplied, and two shared buffers leave one barrier
+// per step. Every output is one chain of fused multiply-adds over i in ascending order from +0,
+// so the values do not depend on the tile. T = 128, or 64 where 128 gives fewer tiles than SMs.
+template <int T>
 __global__ void __launch_bounds__(256) beam_gemm_kernel(const float* __restrict__ A,
                                                         const float* __restrict__ S,
                                                         float* __restrict__ C, int rows, int in) {
-    __shared__ float As[16][65], Bs[16][64];
+    constexpr int N = T / 64;              // 64-row (and 64-column) parts of a tile, 4 x 4 N^2 outputs
+    constexpr int LD = T * 4 / 256;        // 16-byte loads per thread of a 16-deep tile
+    __shared__ __align__(16) float As[2][16][T + 4], Bs[2][16][T];
     pdl_wait();
     pdl_launch_dependents();
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int c0 = blockIdx.x * 64;
-    for (int r0 = blockIdx.y * 64; r0 < rows; r0 += gridDim.y * 64) {
-        float acc[4][4] = {};
-        for (int k0 = 0; k0 < in; k0 += 16) {
-            for (int i = threadIdx.x; i < 64 * 16; i += 256) {
-                const int r = i / 16, kk = i % 16;
-                As[kk][r] = (r0 + r < rows && k0 + kk < in) ? A[(size_t)(r0 + r) * in + k0 + kk] : 0.0f;
-                const int kb = i / 64, cc = i % 64;
-                Bs[kb][cc] = (k0 + kb < in && c0 + cc < in) ? S[(size_t)(k0 + kb) * in + c0 + cc] : 0.0f;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int c0 = blockIdx.x * T, nk = (in + 15) / 16;
+    for (int r0 = blockIdx.y * T; r0 < rows; r0 += gridDim.y * T) {
+        float4 ra[LD], rb[LD];
+        auto load = [&](int k0) {
+#pragma unroll
+            for (int l = 0; l < LD; ++l) {
+                const int i = tid + l * 256, r = r0 + i / 4, k = k0 + (i & 3) * 4;
+                ra[l] = r < rows && k < in ? __ldg((const float4*)(A + (size_t)r * in + k)) : float4{};
+                const int kb = k0 + i / (T / 4), cc = c0 + i % (T / 4) * 4;
+                rb[l] = kb < in && cc < in ? __ldg((const float4*)(S + (size_t)kb * in + cc)) : float4{};
             }
-            __syncthreads();
+        };
+        auto store = [&](int buf) {
+#pragma unroll
+            for (int l = 0; l < LD; ++l) {
+                const int i = tid + l * 256, r = i / 4, k = (i & 3) * 4;
+                As[buf][k][r] = ra[l].x;
+                As[buf][k + 1][r] = ra[l].y;
+                As[buf][k + 2][r] = ra[l].z;
+                As[buf][k + 3][r] = ra[l].w;
+                *(float4*)&Bs[buf][i / (T / 4)][i % (T / 4) * 4] = rb[l];
+            }
+        };
+        float2 acc[4 * N][2 * N];
+#pragma unroll
+        for (int u = 0; u < 4 * N; ++u)
+#pragma unroll
+            for (int v = 0; v < 2 * N; ++v) acc[u][v] = make_float2(0.0f, 0.0f);
+        load(0);
+        store(0);
+        __syncthreads();
+        for (int kt = 0; kt < nk; ++kt) {
+            const int buf = kt & 1;
+            if (kt + 1 < nk) load((kt + 1) * 16);
 #pragma unroll
             for (int kk = 0; kk < 16; ++kk) {
-                float a[4], b[4];
+                float4 a4[N], b4[N];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    a[u] = As[kk][ty * 4 + u];
-                    b[u] = Bs[kk][tx * 4 + u];
+                for (int h = 0; h < N; ++h) {
+                    a4[h] = *(const float4*)&As[buf][kk][h * 64 + ty * 4];
+                    b4[h] = *(const float4*)&Bs[buf][kk][h * 64 + tx * 4];
                 }
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
+                for (int h = 0; h < N; ++h) {
+                    const float av[4] = {a4[h].x, a4[h].y, a4[h].z, a4[h].w};
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+                    for (int u = 0; u < 4; ++u)
+#pragma unroll
+                        for (int g = 0; g < N; ++g) {
+                            const float2 aa = make_float2(av[u], av[u]);
+                            acc[4 * h + u][2 * g] = ffma2(aa, make_float2(b4[g].x, b4[g].y), acc[4 * h + u][2 * g]);
+                            acc[4 * h + u][2 * g + 1] =
+                                ffma2(aa, make_float2(b4[g].z, b4[g].w), acc[4 * h + u][2 * g + 1]);
+                        }
+                }
             }
+            if (kt + 1 < nk) store(buf ^ 1);
             __syncthreads();
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 4 * N; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const int r = r0 + ty * 4 + u, c = c0 + tx * 4 + v;
-                if (r < rows && c < in) C[(size_t)r * in + c] = acc[u][v];
+            for (int g = 0; g < N; ++g) {
+                const int r = r0 + (u >> 2) * 64 + ty * 4 + (u & 3), c = c0 + g * 64 + tx * 4;
+                if (r < rows && c < in)    // in is a multiple of 8
+                    *(float4*)(C + (size_t)r * in + c) = make_float4(acc[u][2 * g].x, acc[u][2 * g].y,
+                                                                     acc[u][2 * g + 1].x, acc[u][2 * g + 1].y);
             }
     }
 }
@@ -137,38 +178,152 @@ __device__ __forceinline__ bool before(float a, int ia, float b, int ib) {
 
 // One warp per (row, group), the rows of one group handled by the warps of a CTA (the group's
 // block S_gg and the codebooks are staged once per CTA). Per book t, the candidates are every
-// (state, codeword) pair, index j = rank * 2^B + c; lane L scores j = L, L + 32, ... and keeps
-// its K best in a sorted list; K rounds of a warp-wide minimum over the lists' heads then give
-// the K best overall.
+// (state, codeword) pair, index j = rank * 2^B + c, and the K first in (score, index) order are
+// kept. Bound: issue. Scoring every candidate by its definition costs about 100 operations (the
+// 8 x 8 quadratic form); instead
+//  1. every candidate gets an estimate of its score from the expanded form
+//     A_r + C_t[c] . G_r + lambda s^2 (C_t[c]^T S_gg C_t[c]),  G_r = -2 lambda s (S_gg u_r + h),
+//     u_r = w_g - s P_r: six operations, G_r in registers, the last term tabled per CTA. Each lane
+//     keeps its smallest estimate per state and per codeword;
+//  2. the keep-th smallest of the 32 lanes' smallest estimates is at least the keep-th smallest
+//     estimate; with both forms' rounding errors below eps, every candidate among the K first has an
+//     estimate of at most that plus 2 eps. Candidates whose state and codeword minima are in reach
+//     (typically about keep + 2 of up to 4096) are listed;
+//  3. the listed candidates are scored by the definition, in the fixed order of operations, and
+//     the K first of them are the K first of all: the result is the full search's, bit for bit.
+// eps: both forms add up products bounded by the terms of T_r = |score_r| + lambda (D^T |S_gg| D +
+// 2 D . |h|), D = |w_g| + |s| (|P_r| + max_c |C_t[c]|), each term with at most about 30 roundings of
+// 2^-24 and the expanded form with four such sums: eps = 2^-16 max_r T_r covers their sum twice.
+// Where the list would overflow (many equal scores) or T_r is out of range, the K first are found by
+// K passes over all candidates scored by the definition.
+// (rows x inputs 1024 x 4096, M = 4, K = 8: scoring every candidate with sorted lists per lane took
+// 75 ms; this form 5 ms.)
+constexpr int kBeamList = 256;     // listed candidates per warp
+
+// A warp's scratch.
+struct BeamWarp {
+    float h[8][8];                                     // h_k of every prefix
+    struct States {
+        float P[kBeamMaxK][8];
+        float score[kBeamMaxK];
+        unsigned long long codes[kBeamMaxK];           // code of book k in byte k
+    } st[2];
+    float G[kBeamMaxK][8], A[kBeamMaxK];
+    float lscore[kBeamList];
+    int lidx[kBeamList];
+};
+
+// Smallest estimates over this lane's codewords (c = lane + 32 i) for RC states at once: per state in
+// mr, per codeword in mc[32 i + lane] (the first RC states, or together with the earlier ones').
+template <int RC, bool FIRST>
+__device__ __forceinline__ void beam_estimates(const float4* lo, const float4* hi, const float* Q, float F,
+                                               const float* G, const float* A, int lane, float* mr,
+                                               float* mc) {
+    float2 g2[RC][4];
+    float a[RC];
+#pragma unroll
+    for (int r = 0; r < RC; ++r) {
+        const float4 x = *(const float4*)(G + r * 8), y = *(const float4*)(G + r * 8 + 4);
+        g2[r][0] = make_float2(x.x, x.y);
+        g2[r][1] = make_float2(x.z, x.w);
+        g2[r][2] = make_float2(y.x, y.y);
+        g2[r][3] = make_float2(y.z, y.w);
+        a[r] = A[r];
+        mr[r] = FLT_MAX;
+    }
+#pragma unroll 2
+    for (int i = 0; i < 8; ++i) {
+        const int c = lane + 32 * i;
+        const float4 x = lo[c], y = hi[c];
+        const float fq = F * Q[c];
+        float m = FIRST ? FLT_MAX : mc[c];
+#pragma unroll
+        for (int r = 0; r < RC; ++r) {
+            float2 t = ffma2(make_float2(x.x, x.y), g2[r][0], make_float2(a[r] + fq, 0.0f));
+            t = ffma2(make_float2(x.z, x.w), g2[r][1], t);
+            t = ffma2(make_float2(y.x, y.y), g2[r][2], t);
+            t = ffma2(make_float2(y.z, y.w), g2[r][3], t);
+            const float v = t.x + t.y;
+            mr[r] = fminf(mr[r], v);
+            m = fminf(m, v);
+        }
+        mc[c] = m;
+    }
+}
+
+// The K-th smallest (0-based rank k) of the 32 lanes' values: a bitonic sort across the lanes.
+__device__ __forceinline__ float warp_kth(float v, int k, int lane) {
+#pragma unroll
+    for (int size = 2; size <= 32; size <<= 1)
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            const float o = __shfl_xor_sync(0xffffffffu, v, stride);
+            const bool up = (lane & size) == 0, low = (lane & stride) == 0;
+            v = up == low ? fminf(v, o) : fmaxf(v, o);
+        }
+    return __shfl_sync(0xffffffffu, v, k);
+}
+
+// The candidates in reach: bit r of *rmask, bit i of *cmask where the lane's smallest estimate of
+// state r, of codeword lane + 32 i, is within `slack` of the keep-th smallest of the lanes' smallest
+// (at most RC * NCH states; mc: 256 floats of scratch, read and written by the same lanes).
+template <int RC, int NCH>
+__device__ __forceinline__ void beam_reach(const float4* lo, const float4* hi, const float* Q, float F,
+                                           const float* G, const float* A, float* mc, int lane, int keep,
+                                           float slack, uint32_t* rmask, uint32_t* cmask) {
+    float mr[RC * NCH];
+    beam_estimates<RC, true>(lo, hi, Q, F, G, A, lane, mr, mc);
+    if constexpr (NCH == 2) beam_estimates<RC, false>(lo, hi, Q, F, G + RC * 8, A + RC, lane, mr + RC, mc);
+    float m = mr[0];
+#pragma unroll
+    for (int r = 1; r < RC * NCH; ++r) m = fminf(m, mr[r]);
+    const float reach = warp_kth(m, keep - 1, lane) + slack;
+    *rmask = *cmask = 0;
+#pragma unroll
+    for (int r = 0; r < RC * NCH; ++r) *rmask |= (mr[r] <= reach ? 1u : 0u) << r;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) *cmask |= (mc[lane + 32 * i] <= reach ? 1u : 0u) << i;
+}
+
 template <int BDT, int SDT>
-__global__ void __launch_bounds__(kBeamWarps * 32)
+__global__ void __launch_bounds__(kBeamWarps * 32, 2)
 beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
             const uint16_t* __restrict__ scales, const float* __restrict__ S,
             const float* __restrict__ E, const float* __restrict__ V, void* __restrict__ codes_out,
             Lambdas lam, int out, int in, int ng, int M, int B, int K) {
     extern __shared__ __align__(16) float bsm[];
     const int nb = 1 << B;
-    float* Cs = bsm;                                   // [M][nb][8] codebooks, fp32
-    float* Sgg = Cs + (size_t)M * nb * 8;              // [8][8]
-    float* wsh = Sgg + 64;                             // per warp: [M][8] h, then two beams
+    float4* lo = (float4*)bsm;                         // [M][nb] codebooks, fp32: elements 0..3
+    float4* hi = lo + (size_t)M * nb;                  // elements 4..7
+    float* Q = (float*)(hi + (size_t)M * nb);          // [M][nb] C^T S_gg C
+    float* Sgg = Q + (size_t)M * nb;                   // [8][8]
+    unsigned int* cmax = (unsigned int*)(Sgg + 64);    // [M][8] max |C_t[c]_e| (float bits)
+    BeamWarp& bw = ((BeamWarp*)(cmax + 64))[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kBeamFloats = kBeamMaxK * 9 + kBeamMaxK * 8;   // P[8] + score, codes as ints
-    float* my = wsh + (size_t)warp * (8 * 8 + 2 * kBeamFloats + 32 * kBeamMaxK * 2);
-    float* hv = my;                                    // [M][8]
-    float* beamA = hv + 64;
-    float* beamB = beamA + kBeamFloats;
-    float* lst = beamB + kBeamFloats;                  // per lane: K (score, index) pairs
     pdl_wait();
     pdl_launch_dependents();
     const int g = blockIdx.y;
+    for (int i = threadIdx.x; i < 64; i += blockDim.x) {
+        Sgg[i] = S[(size_t)(g * 8 + i / 8) * in + g * 8 + i % 8];
+        cmax[i] = 0u;
+    }
+    __syncthreads();
     for (int i = threadIdx.x; i < M * nb; i += blockDim.x) {
         float cv[8];
         unpack8<BDT>(*(const uint4*)(books + (size_t)i * 8), cv);
+        lo[i] = make_float4(cv[0], cv[1], cv[2], cv[3]);
+        hi[i] = make_float4(cv[4], cv[5], cv[6], cv[7]);
+        float q = 0.0f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) Cs[(size_t)i * 8 + e] = cv[e];
+        for (int e = 0; e < 8; ++e) {
+            float sc = 0.0f;
+#pragma unroll
+            for (int f = 0; f < 8; ++f) sc = fmaf(Sgg[e * 8 + f], cv[f], sc);
+            q = fmaf(cv[e], sc, q);
+            atomicMax(&cmax[(i >> B) * 8 + e], __float_as_uint(fabsf(cv[e])));
+        }
+        Q[i] = q;
     }
-    for (int i = threadIdx.x; i < 64; i += blockDim.x)
-        Sgg[i] = S[(size_t)(g * 8 + i / 8) * in + g * 8 + i % 8];
     __syncthreads();
 
     for (int o = blockIdx.x * kBeamWarps + warp; o < out; o += gridDim.x * kBeamWarps) {
@@ -182,100 +337,196 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
             const float* ek = E + ((size_t)k * out + o) * in + (size_t)g * 8;
             float v = V[((size_t)k * out + o) * in + (size_t)g * 8 + e];
 #pragma unroll
-            for (int f = 0; f < 8; ++f) v -= Sgg[e * 8 + f] * ek[f];
-            hv[idx] = v;
+            for (int f = 0; f < 8; ++f) v = fmaf(-Sgg[e * 8 + f], ek[f], v);
+            bw.h[k][e] = v;
         }
         // the single empty state
-        if (lane < 8) beamA[lane] = 0.0f;
-        if (lane == 0) beamA[kBeamMaxK * 8] = 0.0f;    // score
+        if (lane < 8) bw.st[0].P[0][lane] = 0.0f;
+        if (lane == 0) {
+            bw.st[0].score[0] = 0.0f;
+            bw.st[0].codes[0] = 0ull;
+        }
         __syncwarp();
         int nstates = 1;
-        float* cur = beamA;
-        float* nxt = beamB;
         for (int t = 0; t < M; ++t) {
+            const BeamWarp::States& cur = bw.st[t & 1];
+            BeamWarp::States& nxt = bw.st[(t + 1) & 1];
             const float lt = lam.v[t];
-            const float* ht = hv + t * 8;
-            float* myl = lst + (size_t)lane * kBeamMaxK * 2;
-            int cnt = 0;
-            const int ncand = nstates * nb;
-            for (int j = lane; j < ncand; j += 32) {
-                const int r = j / nb, c = j % nb;
-                const float* P = cur + r * 8;
-                const float* cw = Cs + ((size_t)t * nb + c) * 8;
-                float d[8];
+            const float* ht = bw.h[t];
+            const float4 *lot = lo + (size_t)t * nb, *hit = hi + (size_t)t * nb;
+            const int ncand = nstates * nb, keep = ncand < K ? ncand : K;
+            // the score by its definition (the fixed order of operations)
+            auto score = [&](int j) {
+                const int r = j >> B, c = j & (nb - 1);
+                const float4 p0 = *(const float4*)cur.P[r], p1 = *(const float4*)(cur.P[r] + 4);
+                const float4 c0 = lot[c], c1 = hit[c];
+                float d[8] = {p0.x + c0.x, p0.y + c0.y, p0.z + c0.z, p0.w + c0.w,
+                              p1.x + c1.x, p1.y + c1.y, p1.z + c1.z, p1.w + c1.w};
 #pragma unroll
-                for (int e = 0; e < 8; ++e) d[e] = wg[e] - s * (P[e] + cw[e]);
+                for (int e = 0; e < 8; ++e) d[e] = fmaf(-s, d[e], wg[e]);
                 float q = 0.0f, l = 0.0f;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     float sd = 0.0f;
 #pragma unroll
-                    for (int f = 0; f < 8; ++f) sd += Sgg[e * 8 + f] * d[f];
-                    q += d[e] * sd;
-                    l += d[e] * ht[e];
+                    for (int f = 0; f < 8; ++f) sd = fmaf(Sgg[e * 8 + f], d[f], sd);
+                    q = fmaf(d[e], sd, q);
+                    l = fmaf(d[e], ht[e], l);
                 }
-                float sc = cur[kBeamMaxK * 8 + r] + lt * (q + 2.0f * l);
-                if (!(sc <= FLT_MAX)) sc = FLT_MAX;   // NaN and +inf last: keeps the order total
-                // insert into this lane's sorted list of at most K
-                if (cnt < K || before(sc, j, myl[(K - 1) * 2], __float_as_int(myl[(K - 1) * 2 + 1]))) {
-                    int p = cnt < K ? cnt : K - 1;
-                    while (p > 0 && before(sc, j, myl[(p - 1) * 2], __float_as_int(myl[(p - 1) * 2 + 1]))) {
-                        myl[p * 2] = myl[(p - 1) * 2];
-                        myl[p * 2 + 1] = myl[(p - 1) * 2 + 1];
-                        --p;
-                    }
-                    myl[p * 2] = sc;
-                    myl[p * 2 + 1] = __int_as_float(j);
-                    if (cnt < K) ++cnt;
-                }
-            }
-            // merge: K rounds of the warp-wide minimum of the lists' heads
-            const int keep = ncand < K ? ncand : K;
-            int head = 0;
-            for (int i = 0; i < keep; ++i) {
-                float bs = head < cnt ? myl[head * 2] : FLT_MAX;
-                int bj = head < cnt ? __float_as_int(myl[head * 2 + 1]) : 0x7fffffff;
+                const float sc = fmaf(lt, fmaf(2.0f, l, q), cur.score[r]);
+                return sc <= FLT_MAX ? sc : FLT_MAX;   // NaN and +inf last: keeps the order total
+            };
+            // the new state of rank i from candidate j with score sc (one lane)
+            auto keep_state = [&](int i, int j, float sc) {
+                const int r = j >> B, c = j & (nb - 1);
+                const float4 p0 = *(const float4*)cur.P[r], p1 = *(const float4*)(cur.P[r] + 4);
+                const float4 c0 = lot[c], c1 = hit[c];
+                *(float4*)nxt.P[i] = make_float4(p0.x + c0.x, p0.y + c0.y, p0.z + c0.z, p0.w + c0.w);
+                *(float4*)(nxt.P[i] + 4) = make_float4(p1.x + c1.x, p1.y + c1.y, p1.z + c1.z, p1.w + c1.w);
+                nxt.score[i] = sc;
+                nxt.codes[i] = cur.codes[r] | ((unsigned long long)c << (8 * t));
+            };
+            // magnitude bound T_r, and the expanded form's G_r and A_r: four lanes per state
+            float tot = 0.0f;
+            for (int r = lane >> 2; r < kBeamMaxK; r += 8) {
+                float ga[2], au = 0.0f, tr = 0.0f;
+                const int rr = r < nstates ? r : 0, e0 = (lane & 3) * 2;
+                float u[8], D[8];
 #pragma unroll
-                for (int sh = 16; sh > 0; sh >>= 1) {
-                    const float os = __shfl_xor_sync(0xffffffffu, bs, sh);
-                    const int oj = __shfl_xor_sync(0xffffffffu, bj, sh);
-                    if (before(os, oj, bs, bj)) {
-                        bs = os;
-                        bj = oj;
+                for (int f = 0; f < 8; ++f) {
+                    u[f] = fmaf(-s, cur.P[rr][f], wg[f]);
+                    D[f] = fabsf(wg[f]) + fabsf(s) * (fabsf(cur.P[rr][f]) + __uint_as_float(cmax[t * 8 + f]));
+                }
+                float ue[2], De[2];                    // elements e0, e0 + 1 (lane & 3 picks)
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    if ((e >> 1) == (lane & 3)) {
+                        ue[e & 1] = u[e];
+                        De[e & 1] = D[e];
+                    }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    float su = 0.0f, sD = 0.0f;
+#pragma unroll
+                    for (int f = 0; f < 8; ++f) {
+                        const float sv = Sgg[(e0 + i) * 8 + f];
+                        su = fmaf(sv, u[f], su);
+                        sD = fmaf(fabsf(sv), D[f], sD);
+                    }
+                    const float hv = ht[e0 + i];
+                    ga[i] = -2.0f * lt * s * (su + hv);
+                    au = fmaf(ue[i], fmaf(2.0f, hv, su), au);
+                    tr = fmaf(De[i], fmaf(2.0f, fabsf(hv), sD), tr);
+                }
+                au += __shfl_xor_sync(0xffffffffu, au, 1);
+                au += __shfl_xor_sync(0xffffffffu, au, 2);
+                tr += __shfl_xor_sync(0xffffffffu, tr, 1);
+                tr += __shfl_xor_sync(0xffffffffu, tr, 2);
+                bw.G[r][e0] = ga[0];
+                bw.G[r][e0 + 1] = ga[1];
+                // a state that is not there is never in reach
+                if ((lane & 3) == 0) bw.A[r] = r < nstates ? fmaf(lt, au, cur.score[rr]) : FLT_MAX;
+                const float T = fmaf(lt, tr, fabsf(cur.score[rr]));
+                tot = fmaxf(tot, T < 1.0e36f ? T : FLT_MAX);   // (a NaN counts as too large)
+            }
+#pragma unroll
+            for (int sh = 16; sh >= 4; sh >>= 1)
+                tot = fmaxf(tot, __shfl_xor_sync(0xffffffffu, tot, sh));
+            __syncwarp();
+            int n = -1;                                // listed candidates (-1: no list)
+            if (tot < 1.0e36f && (lt == 0.0f || tot > 1.0e-30f)) {   // (below, products underflow)
+                if (lt == 0.0f) {
+                    // every candidate has its state's score: the first `keep` indices are the first
+                    if (lane < keep) bw.lidx[lane] = lane;
+                    n = keep;
+                } else if (nb < 256) {                 // at most 256 candidates: all of them
+                    for (int j = lane; j < ncand; j += 32) bw.lidx[j] = j;
+                    n = ncand;
+                } else {
+                    const float F = lt * s * s, slack = 3.0517578125e-5f * tot;   // 2 eps
+                    const float* Qt = Q + (size_t)t * nb;
+                    uint32_t rmask, cmask;
+                    if (nstates == 1)
+                        beam_reach<1, 1>(lot, hit, Qt, F, bw.G[0], bw.A, bw.lscore, lane, keep, slack, &rmask, &cmask);
+                    else if (nstates <= 4)
+                        beam_reach<4, 1>(lot, hit, Qt, F, bw.G[0], bw.A, bw.lscore, lane, keep, slack, &rmask, &cmask);
+                    else if (nstates <= 8)
+                        beam_reach<8, 1>(lot, hit, Qt, F, bw.G[0], bw.A, bw.lscore, lane, keep, slack, &rmask, &cmask);
+                    else
+                        beam_reach<8, 2>(lot, hit, Qt, F, bw.G[0], bw.A, bw.lscore, lane, keep, slack, &rmask, &cmask);
+                    rmask &= (1u << nstates) - 1u;
+                    const int mine = __popc(rmask) * __popc(cmask);
+                    int at = mine;                     // inclusive prefix sum over the lanes
+#pragma unroll
+                    for (int sh = 1; sh < 32; sh <<= 1) {
+                        const int v = __shfl_up_sync(0xffffffffu, at, sh);
+                        if (lane >= sh) at += v;
+                    }
+                    n = __shfl_sync(0xffffffffu, at, 31);
+                    if (n > kBeamList) n = -1;
+                    else {
+                        at -= mine;
+                        for (uint32_t rm = rmask; rm; rm &= rm - 1)
+                            for (uint32_t cm = cmask; cm; cm &= cm - 1)
+                                bw.lidx[at++] = ((__ffs(rm) - 1) << B) | (lane + 32 * (__ffs(cm) - 1));
                     }
                 }
-                if (head < cnt && __float_as_int(myl[head * 2 + 1]) == bj) ++head;
-                // new state i: parent rank bj / nb, codeword bj % nb
-                // every round finds a real candidate (the lists hold at least `keep`), so bj
-                // is one; the clamp only guards the shared-memory index
-                const int r = min(bj / nb, nstates - 1), c = bj % nb;
-                if (lane < 8) nxt[i * 8 + lane] = cur[r * 8 + lane] + Cs[((size_t)t * nb + c) * 8 + lane];
-                if (lane == 0) nxt[kBeamMaxK * 8 + i] = bs;
-                int* ncodes = (int*)(nxt + kBeamMaxK * 9);
-                const int* ocodes = (const int*)(cur + kBeamMaxK * 9);
-                if (lane < t) ncodes[i * 8 + lane] = ocodes[r * 8 + lane];
-                if (lane == t) ncodes[i * 8 + t] = c;
+                __syncwarp();
+            }
+            if (n >= 0 && n <= 32) {
+                // one listed candidate per lane; its rank is the number of candidates before it
+                const int j = lane < n ? bw.lidx[lane] : 0x7fffffff;
+                const float sc = lane < n ? score(j) : FLT_MAX;
+                int rank = 0;
+                for (int i = 0; i < n; ++i) {
+                    const float os = __shfl_sync(0xffffffffu, sc, i);
+                    const int oj = __shfl_sync(0xffffffffu, j, i);
+                    rank += before(os, oj, sc, j) ? 1 : 0;
+                }
+                if (lane < n && rank < keep) keep_state(rank, j, sc);
+            } else {
+                // K rounds: the first candidate after the last kept one, of the list or of all
+                if (n >= 0)
+                    for (int i = lane; i < n; i += 32) bw.lscore[i] = score(bw.lidx[i]);
+                __syncwarp();
+                float ps = -FLT_MAX;
+                int pj = -1;
+                for (int i = 0; i < keep; ++i) {
+                    float bs = FLT_MAX;
+                    int bj = 0x7fffffff;
+                    for (int q = lane; q < (n >= 0 ? n : ncand); q += 32) {
+                        const int j = n >= 0 ? bw.lidx[q] : q;
+                        const float sc = n >= 0 ? bw.lscore[q] : score(j);
+                        if ((i == 0 || before(ps, pj, sc, j)) && before(sc, j, bs, bj)) {
+                            bs = sc;
+                            bj = j;
+                        }
+                    }
+#pragma unroll
+                    for (int sh = 16; sh > 0; sh >>= 1) {
+                        const float os = __shfl_xor_sync(0xffffffffu, bs, sh);
+                        const int oj = __shfl_xor_sync(0xffffffffu, bj, sh);
+                        if (before(os, oj, bs, bj)) {
+                            bs = os;
+                            bj = oj;
+                        }
+                    }
+                    ps = bs;
+                    pj = min(bj, ncand - 1);           // every round finds one; only guards the index
+                    if (lane == 0) keep_state(i, pj, ps);
+                }
             }
             __syncwarp();
             nstates = keep;
-            float* tmp = cur;
-            cur = nxt;
-            nxt = tmp;
         }
-        const int* best = (const int*)(cur + kBeamMaxK * 9);
-        if (lane < M) {
-            const size_t ci = ((size_t)o * ng + g) * M + lane;
-            if (B == 16) ((uint16_t*)codes_out)[ci] = (uint16_t)best[lane];
-            else ((uint8_t*)codes_out)[ci] = (uint8_t)best[lane];
-        }
+        const unsigned long long best = bw.st[M & 1].codes[0];
+        if (lane < M) ((uint8_t*)codes_out)[((size_t)o * ng + g) * M + lane] = (uint8_t)(best >> (8 * lane));
         __syncwarp();
     }
 }
 
 inline size_t beam_smem(int M, int B) {
-    const int kBeamFloats = kBeamMaxK * 9 + kBeamMaxK * 8;
-    return ((size_t)M * ((size_t)1 << B) * 8 + 64 +
-            (size_t)kBeamWarps * (64 + 2 * kBeamFloats + 32 * kBeamMaxK * 2)) * 4;
+    return ((size_t)M << B) * 9 * 4 + 64 * 4 + 64 * 4 + kBeamWarps * sizeof(BeamWarp);
 }
 
 template <int BDT, int SDT>
@@ -307,10 +558,13 @@ aq_status run_beam(const Dims& d, const void* w, const void* codes, const void* 
                               "cudaLaunchKernelEx (beam symmetric part)");
         e != AQ_OK)
         return e;
-    const int row_tiles = (int)(((long long)d.M * d.out + 63) / 64);
-    cfg.gridDim = dim3((d.in + 63) / 64, row_tiles < 65535 ? row_tiles : 65535);
-    if (aq_status e = cuda_ok(cudaLaunchKernelEx(&cfg, beam_gemm_kernel, (const float*)E, (const float*)S, V,
-                                                 d.M * d.out, d.in),
+    const long long rows = (long long)d.M * d.out;
+    const bool big = ((rows + 127) / 128) * ((d.in + 127) / 128) >= di.sms;
+    const int T = big ? 128 : 64;
+    const int row_tiles = (int)((rows + T - 1) / T);
+    cfg.gridDim = dim3((d.in + T - 1) / T, row_tiles < 65535 ? row_tiles : 65535);
+    if (aq_status e = cuda_ok(cudaLaunchKernelEx(&cfg, big ? beam_gemm_kernel<128> : beam_gemm_kernel<64>,
+                                                 (const float*)E, (const float*)S, V, (int)rows, d.in),
                               "cudaLaunchKernelEx (beam cross terms)");
         e != AQ_OK)
         return e;
@@ -320,9 +574,11 @@ aq_status run_beam(const Dims& d, const void* w, const void* codes, const void* 
     if (cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         e != cudaSuccess)
         return cuda_fail(e, "cudaFuncSetAttribute");
-    int xb = (d.out + kBeamWarps - 1) / kBeamWarps;
-    const int want = (di.sms * 4 + d.ng - 1) / d.ng;   // enough CTAs to fill the SMs
-    if (xb > want) xb = want < 1 ? 1 : want;
+    // Row blocks per group: enough CTAs for two waves of two per SM, and 16 rows per warp before
+    // that (the staging of the books and their quadratic terms costs about one row's search).
+    int xb = (d.out + 16 * kBeamWarps - 1) / (16 * kBeamWarps);
+    const int want = (di.sms * 4 + d.ng - 1) / d.ng, most = (d.out + kBeamWarps - 1) / kBeamWarps;
+    if (xb < want) xb = want < most ? want : most;
     cfg.gridDim = dim3(xb, d.ng);
     cfg.blockDim = dim3(kBeamWarps * 32);
     cfg.dynamicSmemBytes = smem;
