@@ -124,17 +124,19 @@ aq_status aq_decode(const aq_layout* layout, int m, const void* planes, const vo
 /* ---------------------------------------------------------------- GEMV (batch 1..16)
  * y[t, o] = sum_i x[t, i] * W_m[o, i] for t < batch (Sec. 2.2 Y = W X, with W_m the prefix-m
  * reconstruction of Sec. 3.2 / Sec. 5), accumulated in fp32. The kernel reads the first m
- * planes once (HBM-bound at batch 1); 4- and 8-bit codebooks are staged on chip. No weight is
- * rounded on the way: the products are taken from tables of fp32 values (batch 1..2) or by
- * 16-bit tensor-core multiplies of the stored codewords themselves (above; where the books and
- * the activations differ in type, the bf16 side is scaled by powers of two into fp16, which is
- * exact for values within 2^29 of the largest of their book set, or of their token and slice).
+ * planes once (HBM-bound at batch 1); 4- and 8-bit codebooks are staged on chip. Up to batch 8,
+ * and wherever that is estimated to be faster, no weight is rounded on the way: the products are
+ * taken from tables of fp32 values (batch 1..2) or by 16-bit tensor-core multiplies of the stored
+ * codewords themselves (above; where the books and the activations differ in type, the bf16 side
+ * is scaled by powers of two into fp16, which is exact for values within 2^29 of the largest of
+ * their book set, or of their token and slice). Larger layers at batch 9..16 with m <= 4 run the
+ * tensor-memory kernel of aq_gemm, whose decoded weights are rounded once to fp16.
  *   x         : device, [batch][d_in] of x_dtype (AQ_F16 or AQ_BF16), row-major
  *   y         : device, [batch][d_out] of y_dtype (AQ_F16, AQ_BF16 or AQ_F32), row-major
  *   workspace : device scratch of at least aq_gemv_workspace_bytes(layout, batch) bytes:
  *               a status word and room for fp32 partial sums of every row (one per 256-input
- *               slice and token, times up to 8 codebooks with 8-bit codes at batch 1..8; the
- *               kernels of batch 3 and more leave it unused). Zero-fill it once before its first
+ *               slice and token, times up to 8 codebooks with 8-bit codes at batch 1..8; at batch
+ *               9..16 it may hold the fp16 copy of bf16 activations instead). Zero-fill it once before its first
  *               use (aq_workspace_init); every
  *               call leaves it ready for the next one.
  *               Calls that may overlap on the GPU must not share a workspace.
@@ -147,7 +149,8 @@ aq_status aq_decode(const aq_layout* layout, int m, const void* planes, const vo
  * element, with y_exact the fp64 product of the exactly widened stored values, on unit-scale
  * inputs (activations of order 1, codebook entries of the order of N(0, 0.02^2), as in the
  * benchmark layers); in terms of the inputs, fp32 accumulation of exact products: about
- * 2^-15 * |s[o]| * sum_i |x_i| sum_k |C_k[b_k]_i| at most, and one rounding to a 16-bit y. */
+ * 2^-15 * |s[o]| * sum_i |x_i| sum_k |C_k[b_k]_i| at most (2^-11 where weights are rounded), and
+ * one rounding to a 16-bit y. */
 size_t aq_gemv_workspace_bytes(const aq_layout* layout, int batch);
 aq_status aq_gemv(const aq_layout* layout, int m, const void* planes, const void* books,
                   const void* scales, const void* x, int x_dtype, int batch, void* y,
@@ -234,9 +237,10 @@ aq_status aq_gemv_static_scratch_status(void* stream);
 
 /* ---------------------------------------------------------------- GEMM (prefill)
  * Same product for many tokens (Sec. 2.2 Y = W X with W_m of Sec. 3.2 / Sec. 5):
- * y[t, o] = sum_i x[t, i] * W_m[o, i], t < tokens. Decoded weight tiles are built in shared
- * memory and multiplied on the tcgen05 tensor cores with fp32 accumulation in tensor memory
- * (up to 2047 tokens, or m = 1, W_m is never written to HBM; see workspace below). The MMA
+ * y[t, o] = sum_i x[t, i] * W_m[o, i], t < tokens. Decoded weight tiles are built in tensor
+ * memory (up to 2047 tokens, m <= 4, where that is estimated to be faster) or shared memory and
+ * multiplied on the tcgen05 tensor cores with fp32 accumulation in tensor memory (up to 2047
+ * tokens, or m = 1, 8-bit codes are never written out as W_m; see workspace below). The MMA
  * operands are fp16, over the whole range of the inputs: each decoded weight (fp32 sum of the
  * m codewords) is rounded once to fp16 after the codebooks were scaled by a power of two
  * 2^-f that keeps the largest possible sum below 2^15; bf16 activations are copied to fp16 in
@@ -244,8 +248,9 @@ aq_status aq_gemv_static_scratch_status(void* stream);
  * [2^14, 2^15); the epilogue multiplies by 2^(e_t + f). The scalings are exact, so inputs
  * already inside fp16's range give the same bits as without them, and bf16 values far outside
  * it (activation outliers, large codebook entries) are multiplied with fp16's 11-bit
- * significand instead of saturating. Supported: code_bits = 8 and 4 (4-bit layouts always
- * decode W_m into the workspace first), any m <= num_books <= 8.
+ * significand instead of saturating. Supported: code_bits = 8 and 4 (4-bit
+ * codes that do not take the tensor-memory form are decoded into the workspace first), any
+ * m <= num_books <= 8.
  *   x : device, [tokens][d_in] of x_dtype (AQ_F16 or AQ_BF16); y : device, [tokens][d_out]
  *       of y_dtype (AQ_F16, AQ_BF16 or AQ_F32).
  *   workspace : aq_gemm_workspace_bytes(layout, tokens) bytes (a 256-byte status block, one

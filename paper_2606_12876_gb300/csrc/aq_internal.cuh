@@ -101,6 +101,15 @@ aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* book
 aq_status launch_cw(const Dims& d, int m, const void* planes, const void* books, const void* scales,
                     const void* x, int x_dt, int batch, void* y, int y_dt, const void* y_prev,
                     cudaStream_t st);
+// The product with the decoded weights in tensor memory (gemm_ts.cu): its estimated time in clocks
+// (below 0: not served), and the launch (x: fp16; xfac: per-token factors or null; ws: its first word
+// is the status word).
+double ts_clocks(const Dims& d, int m, int tokens);
+aq_status launch_ts(const Dims& d, int m, const void* planes, const void* books, const void* scales,
+                    const void* x, const float* xfac, int tokens, void* y, int y_dt, void* ws, cudaStream_t st);
+// bf16 activations as fp16, each token row scaled by a power of two into fp16's range: the copy
+// [tokens][in] at dst, the rows' factors at fac.
+aq_status launch_x_to_f16(const void* x, void* dst, float* fac, int in, int tokens, cudaStream_t st);
 // aq_gemv_group: n (<= 4) layers sharing x; ws[l] = layer l's workspace region.
 aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* planes,
                             const void* const* books, const void* const* scales, const void* x,
@@ -208,6 +217,18 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     return d;
 }
 
+// True in one lane of a converged warp, the same one every time. Code that issues TMA copies, MMAs
+// or commits runs under this predicate, not under a lane comparison: their operands are uniform
+// registers, and unless the compiler knows that a single lane is active it wraps every one of them
+// in a loop over the active lanes (measured: 112 clocks per tcgen05.mma and 110 per commit under
+// `lane == 0`, 26 and 100 under elect.sync, at 128 x 16 x 16).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n .reg .pred P;\n elect.sync _|P, 0xffffffff;\n selp.u32 %0, 1, 0, P;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
 // ---- shared-memory barriers, bulk copies and programmatic dependent launch (sm_90+) -------
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -284,7 +305,20 @@ __device__ __forceinline__ void unrotate_codes(const uint32_t (&w)[8], int o, ui
 #pragma unroll
     for (int i = 0; i < 8; ++i) t[i] = (rw & 4) ? v[(i + 4) & 7] : v[i];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) u[j] = rb ? __funnelshift_l(t[(j + 7) & 7], t[j], rb) : t[j];
+    for (int j = 0; j < 8; ++j) u[j] = __funnelshift_l(t[(j + 7) & 7], t[j], rb);   // (t[j] for rb = 0)
+}
+
+// The same for the 32 four-bit codes of a row's slice unit (four words; nibble q of word j of u is
+// the code of group 8j + q).
+__device__ __forceinline__ void unrotate_nibbles(const uint32_t (&w)[4], int o, uint32_t (&u)[4]) {
+    const int r = o & 31, rw = r >> 3, rb = (r & 7) * 4;
+    uint32_t t[4], v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t[i] = (rw & 1) ? w[(i + 3) & 3] : w[i];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = (rw & 2) ? t[(i + 2) & 3] : t[i];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) u[j] = __funnelshift_l(v[(j + 3) & 3], v[j], rb);
 }
 
 // Shared-memory accesses through 32-bit shared-window addresses. lds128 is for data that no

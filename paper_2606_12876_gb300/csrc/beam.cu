@@ -91,7 +91,7 @@ __global__ void beam_sym_kernel(const void* __restrict__ h, int h_dt, float* __r
 // per step. Every output is one chain of fused multiply-adds over i in ascending order from +0,
 // so the values do not depend on the tile. T = 128, or 64 where 128 gives fewer tiles than SMs.
 template <int T>
-__global__ void __launch_bounds__(256) beam_gemm_kernel(const float* __restrict__ A,
+__global__ void __launch_bounds__(256, 2) beam_gemm_kernel(const float* __restrict__ A,
                                                         const float* __restrict__ S,
                                                         float* __restrict__ C, int rows, int in) {
     constexpr int N = T / 64;              // 64-row (and 64-column) parts of a tile, 4 x 4 N^2 outputs

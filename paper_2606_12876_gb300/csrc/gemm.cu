@@ -18,7 +18,7 @@
 //               128-token boxes per stage) and, once per 256-input slice, the code rows this
 //               CTA decodes, of the first m planes (1-D bulk copies).
 //   warp 1      allocates the pair's tensor memory (together with the peer's warp 1). In the
-//               leader CTA of a pair lane 0 issues the pair MMAs (2 token blocks x 4 K=16
+//               leader CTA of a pair an elected lane issues the pair MMAs (2 token blocks x 4 K=16
 //               steps per stage) after one barrier wait per stage, and commits the
 //               activation-stage release and accumulator-ready barriers to its pair and the
 //               weight-stage release to every CTA of the cluster. In the peer CTA lane 0 relays "stage
@@ -45,6 +45,8 @@
 #include <mutex>
 
 #include "aq_internal.cuh"
+#include "launch.cuh"
+#include "operand_scale.cuh"
 #include "tc_ptx.cuh"
 
 namespace aq {
@@ -105,58 +107,6 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi, int dt) {
     }
     __half2 h = __floats2half2_rn(lo, hi);
     return *(uint32_t*)&h;
-}
-
-__device__ __forceinline__ uint32_t f16x2(float2 v) {   // {lo, hi} -> packed fp16 pair, RN
-    uint32_t h;
-    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(v.y), "f"(v.x));
-    return h;
-}
-
-// fp16 range for any input (R9). The MMA operands are fp16; bf16 activations and bf16
-// codebooks can hold values far outside fp16's range (and fp16 books' sums can exceed it).
-// Both are therefore scaled by powers of two, which is exact: each token row of bf16
-// activations by 2^-e_t so that its largest |x| lies in [2^14, 2^15) (bf16_rows_to_f16_kernel),
-// and the codebooks by 2^-f so that the largest possible |sum of m codewords| (the sum over
-// the books of their largest |entry|) lies below 2^15 (for bf16 books also at least 2^14, so
-// that small weights do not fall into fp16's subnormal range; fp16 books are only scaled down,
-// and a single fp16 book not at all). The epilogue multiplies by 2^(e_t + f). Where nothing
-// was out of range the result is bit-identical to the unscaled computation.
-
-// Largest |entry| of a codeword of eight 16-bit values, as the bits of a non-negative float
-// (monotonic in the value, so unsigned maxima of them are maxima of the values).
-template <int BDT>
-__device__ __forceinline__ unsigned int codeword_max_bits(const uint4& c) {
-    float f[8];
-    unpack8<BDT>(c, f);
-    float mx = 0.0f;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) mx = fmaxf(mx, fabsf(f[e]));
-    return __float_as_uint(mx);
-}
-
-// f of the codebooks of prefix m from the per-book largest |entry| (float bits).
-template <int BDT>
-__device__ __forceinline__ int book_exponent(const unsigned int* wmax, int m) {
-    if (BDT == AQ_F16 && m == 1) return 0;   // one fp16 codeword is an fp16 value already
-    float tot = 0.0f;
-    for (int k = 0; k < m; ++k) tot += __uint_as_float(wmax[k]);
-    if (!(tot > 0.0f)) return 0;             // all-zero books (or NaN entries)
-    int f = exponent_of(fminf(tot, 3.0e38f)) - 14;
-    if (BDT == AQ_F16 && f < 0) f = 0;
-    return max(-100, min(100, f));
-}
-
-// A codeword times sc (a power of two), back in its own type.
-template <int BDT>
-__device__ __forceinline__ uint4 scale_codeword(const uint4& c, float sc) {
-    float f[8];
-    unpack8<BDT>(c, f);
-    uint16_t h[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) h[e] = f32_to_bits<BDT>(f[e] * sc);
-    return make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16),
-                      h[4] | ((uint32_t)h[5] << 16), h[6] | ((uint32_t)h[7] << 16));
 }
 
 // Decoded group (eight fp16 weights): sum of the MB codewords in fp32, in book order, rounded
@@ -313,7 +263,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
 
     if (warp == 0) {
         // ---------------- producer
-        if (lane == 0) {
+        if (elect_one()) {
             asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&xmap) : "memory");
             if constexpr (DENSE) asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&wmap) : "memory");
             int issued_a = 0, issued_c = 0;
@@ -371,7 +321,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
                 mbar_wait(&codes_full[j & 1], (j >> 1) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
+          if (elect_one()) {
             // ---------------- MMA issuer (leader)
             // kind::f16 instruction descriptor: fp32 accumulator, fp16 A and B, both K-major,
             // N = 256, M = 256 (pair).
@@ -398,7 +349,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
                 umma_commit_pair(&empty_b[sb], (uint16_t)((1u << (2 * NP)) - 1u));
             }
             umma_commit_pair(acc_full, (uint16_t)(0x3u << (2 * pair)));
-        } else if (lane == 0) {
+          }
+        } else if (elect_one()) {
             // ---------------- relay (peer): this CTA's half of a stage is ready
             const uint32_t leader_ready = map_to_rank(smem_u32(ready), pair << 1);
             for (int it = 0; it < nk; ++it) {
@@ -409,7 +361,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
             }
         }
     } else if (warp == 2) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             // ---------------- activation relay (leader): its A stage landed
             // The A ring is deeper than the stage barrier's ring, so before counting stage it
             // the relay waits until the barrier's previous phase (stage it - kStagesB) is done.
@@ -425,7 +377,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
             }
         }
     } else if (warp == 3) {
-        if (SHARE && lane == 0) {
+        if (SHARE && elect_one()) {
             // ---------------- copier: once this CTA's decoders have written their slab of a
             // weight stage, copy it into each partner's stage (same offset) with a bulk copy
             // that completes on that partner's stage barrier, and count this CTA's slab on its
@@ -593,9 +545,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                if (lane == 0 && tw < tokens && n0 + nc < out) tma_store_2d(&ymap, n0 + nc, tw, chunk);
+                if (tw < tokens && n0 + nc < out && elect_one()) tma_store_2d(&ymap, n0 + nc, tw, chunk);
             }
-            if (lane == 0) {   // the staged chunks are read before the CTA leaves
+            if (elect_one()) {   // the staged chunks are read before the CTA leaves
                 bulk_commit();
                 bulk_wait_read_all();
             }
@@ -1071,13 +1023,43 @@ aq_status run_gemm_dense(const Dims& d, int m, const void* planes, const void* b
                    "cudaLaunchKernelEx (dense GEMM)");
 }
 
+// Whether the tensor-memory kernel (gemm_ts.cu) takes a call: where its estimated time is below that
+// of the pair kernel with decoding in its loop, below the length at which W_m is decoded once. The
+// pair kernel's waves (76 pairs or 36 clusters of four on 152 SMs) times 64-input stages, measured:
+// 1110 / 1850 / 2200 clocks a stage for m = 1 / 3 / 4 with one pair, 1250 / 1690 for m = 2 / 4 with
+// two. (14336 x 4096, m = 4: 31.8 against 79.4 us at 100 tokens, 71.9 against 81.8 at 512; m = 1:
+// 54.0 against 45.3 at 512, where the pair kernel stays; 4096 x 14336, m = 3, 100 tokens: 30.3
+// against 211.) 4-bit layouts have no in-loop form; their other way, decoding W_m first, costs about
+// 15000 clocks and 2 bytes per weight of HBM more than its product.
+bool gemm_uses_ts(const Dims& d, int m, int tokens) {
+    if (tokens >= kGemmDenseTokens) return false;
+    const double ts = ts_clocks(d, m, tokens);
+    if (ts < 0.0) return false;
+    const int np = d.B == 4 ? 1 : gemm_pairs_per_cluster(m, tokens);
+    const long long clusters = (long long)((d.out + kBN - 1) / kBN) * ((tokens + np * kPairTokens - 1) / (np * kPairTokens));
+    const long long waves = np == 1 ? (clusters + 75) / 76 : (clusters + 35) / 36;
+    const double loop = np == 1 ? (m == 1 ? 1110.0 : 740.0 + 365.0 * m) : 810.0 + 220.0 * m;
+    const double stage = d.B == 4 ? 1100.0 : loop, extra = d.B == 4 ? 15000.0 + (double)d.out * d.in / 1500.0 : 0.0;
+    return ts < waves * (((d.in + kBK - 1) / kBK) * stage + 12000.0) + extra;
+}
+
 }  // namespace
+
+// The fp16 copy of bf16 activations at dst and the per-token factors at fac.
+aq_status launch_x_to_f16(const void* x, void* dst, float* fac, int in, int tokens, cudaStream_t st) {
+    DeviceInfo di;
+    if (aq_status e = device_info(&di); e != AQ_OK) return e;
+    const int blocks = tokens < di.sms * 8 ? tokens : di.sms * 8;
+    return launch_pdl(bf16_rows_to_f16_kernel, dim3(blocks), dim3(256), 0, st, (const uint16_t*)x, (uint16_t*)dst,
+                      fac, in, tokens);
+}
 
 aq_status launch_gemm(const Dims& d, int m, const void* planes, const void* books,
                       const void* scales, const void* x, int x_dt, int tokens, void* y, int y_dt,
                       void* ws, cudaStream_t st) {
     if (d.out == 0 || tokens == 0) return AQ_OK;
     if ((d.B != 8 && d.B != 4) || m > kGemmMaxM) return AQ_ERR_UNSUPPORTED;
+    const bool ts = gemm_uses_ts(d, m, tokens);
     const void* xh = x;
     const float* xfac = nullptr;
     if (x_dt == AQ_BF16) {
@@ -1085,26 +1067,12 @@ aq_status launch_gemm(const Dims& d, int m, const void* planes, const void* book
         // per-token factors, in the workspace
         void* dst = (char*)ws + gemm_x16_offset(tokens);
         float* fac = (float*)((char*)ws + gemm_xfac_offset());
-        DeviceInfo di;
-        if (aq_status e = device_info(&di); e != AQ_OK) return e;
-        const int blocks = tokens < di.sms * 8 ? tokens : di.sms * 8;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(blocks);
-        cfg.blockDim = dim3(256);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (aq_status e = cuda_ok(cudaLaunchKernelEx(&cfg, bf16_rows_to_f16_kernel, (const uint16_t*)x,
-                                                     (uint16_t*)dst, fac, d.in, tokens),
-                                  "cudaLaunchKernelEx (activation copy)");
-            e != AQ_OK)
-            return e;
+        if (aq_status e = launch_x_to_f16(x, dst, fac, d.in, tokens, st); e != AQ_OK) return e;
         xh = dst;
         xfac = fac;
     }
+    if (ts)
+        return launch_ts(d, m, planes, books, scales, xh, xfac, tokens, y, y_dt, ws, st);
     if (gemm_uses_dense(d, m, tokens)) {
         uint16_t* w16 = (uint16_t*)((char*)ws + gemm_w16_offset(d, tokens));
         if (d.B == 4)   // the in-loop decoders read 8-bit codes; 4-bit layouts always go dense

@@ -216,7 +216,7 @@ gemv_lut_kernel(const __grid_constant__ LutLayers L, const uint16_t* __restrict_
         // wait and queue behind whatever code copies are still in flight (measured on the
         // 14336 x 4096 layer: one stage 4-7 % faster per call than a full ring).
         load_books();
-        if (warp == kCons && lane == 0 && p_w.it < i1) issue_next();
+        if (warp == kCons && p_w.it < i1 && elect_one()) issue_next();
     }
     pdl_wait();                 // inputs may come from the preceding kernel in the stream
     pdl_launch_dependents();    // the split-K reduction may become resident (it waits for us)
@@ -228,8 +228,8 @@ gemv_lut_kernel(const __grid_constant__ LutLayers L, const uint16_t* __restrict_
     }
 
     if (warp == kCons) {
-        // ---- producer (lane 0 issues; the warp stays converged for the final barriers)
-        if (lane == 0) {
+        // ---- producer (one lane issues; the warp stays converged for the final barriers)
+        if (elect_one()) {
             while (p_w.it < i1) {
                 if (s_abort) break;
                 if (p_q >= nslots && !mbar_wait(&empty[p_slot], p_phase ^ 1u)) {
@@ -1005,12 +1005,38 @@ static aq_status launch_reduce(const Dims& d, int P, const GemvArgs& a, const vo
                                      (d.flags & AQ_LAYOUT_STATIC_WEIGHTS) ? 1 : 0, st);
 }
 
+// Whether 9..16 tokens run the tensor-memory kernel (gemm_ts.cu): where its estimated time is below
+// that of gemv_cw, which at two token tiles is bound by the tensor pipe's legacy multiplies (64 a unit
+// of 32 rows, slice and book at 4 clocks; per SM, with its fixed cost). 14336 x 4096, m = 4, 16
+// tokens: 29 against 47.7 us; 1024 x 4096, m = 4: gemv_cw stays. bf16 activations are copied to the
+// workspace first (about 3000 clocks), which has room unless the layer has few rows.
+static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt) {
+    if (batch <= 8) return false;
+    const size_t room = gemv_ws_planes(d, batch) * (size_t)d.rows_pad * 4;
+    if (x_dt == AQ_BF16 && room < kWsStatusBytes + (size_t)batch * d.in * 2) return false;
+    const double ts = ts_clocks(d, m, batch);
+    if (ts < 0.0) return false;
+    const double units = (double)d.S * m * d.RBc / 152.0;
+    return ts + (x_dt == AQ_BF16 ? 3000.0 : 0.0) < units * 400.0 + 8000.0;
+}
+
 aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* books,
                       const void* scales, const void* x, int x_dt, int batch, void* y,
                       int y_dt, void* ws, cudaStream_t st, const void* y_prev) {
     if (d.out == 0 || batch == 0) return AQ_OK;
     if (d.B == 4 && batch == 1)
         return launch_lut4(d, m, planes, books, scales, x, x_dt, y, y_dt, y_prev, st);
+    if (d.B != 16 && !y_prev && gemv_uses_ts(d, m, batch, x_dt)) {
+        const void* xh = x;
+        float* fac = nullptr;
+        if (x_dt == AQ_BF16) {   // the fp16 copy and the row factors take the partial sums' room
+            fac = (float*)((char*)ws + ws_partial_offset(d));
+            void* dst = (char*)fac + kWsStatusBytes;
+            if (aq_status e = launch_x_to_f16(x, dst, fac, d.in, batch, st); e != AQ_OK) return e;
+            xh = dst;
+        }
+        return launch_ts(d, m, planes, books, scales, xh, fac, batch, y, y_dt, ws, st);
+    }
     if (d.B == 4 || (d.B == 8 && batch > kLutMaxBatch))
         return launch_cw(d, m, planes, books, scales, x, x_dt, batch, y, y_dt, y_prev, st);
     GemvArgs a{planes, books, scales, x, x_dt, batch, y, y_dt,

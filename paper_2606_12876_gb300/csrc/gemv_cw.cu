@@ -113,18 +113,9 @@ __device__ __forceinline__ void store_unrotated(unsigned char* buf, int row, con
         *(uint4*)(buf + row * 32 + (sw ^ 1) * 16) = make_uint4(u[4], u[5], u[6], u[7]);
     } else {
         const uint32_t w[4] = {raw[0].x, raw[0].y, raw[0].z, raw[0].w};
-        const int r = row & 31, rw = r >> 3, rb = (r & 7) * 4;
-        uint32_t t[4], v[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) t[i] = (rw & 1) ? w[(i + 3) & 3] : w[i];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = (rw & 2) ? t[(i + 2) & 3] : t[i];
-        uint4 u;
-        u.x = rb ? __funnelshift_l(v[3], v[0], rb) : v[0];
-        u.y = rb ? __funnelshift_l(v[0], v[1], rb) : v[1];
-        u.z = rb ? __funnelshift_l(v[1], v[2], rb) : v[2];
-        u.w = rb ? __funnelshift_l(v[2], v[3], rb) : v[3];
-        *(uint4*)(buf + row * 16) = u;
+        uint32_t u[4];
+        unrotate_nibbles(w, row, u);
+        *(uint4*)(buf + row * 16) = make_uint4(u[0], u[1], u[2], u[3]);
     }
 }
 

@@ -253,7 +253,7 @@ wmse_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CU
     if (warp == 0) {
         // ---------------- producer: per stage the P tile of this CTA's 128 values of t and,
         // in one 3-D box, its 64 rows of E_k for the pass's prefixes
-        if (lane == 0) {
+        if (elect_one()) {
             asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&pmap) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&emap) : "memory");
             int issued = 0;
@@ -272,7 +272,8 @@ wmse_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CU
                 mbar_wait(&full[j % kWStages], (j / kWStages) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
+          if (elect_one()) {
             // ---------------- MMA issuer (leader)
             // kind::f16 instruction descriptor: fp32 accumulator, bf16 A and B, both K-major,
             // N = 256, M = 256 (pair).
@@ -297,7 +298,8 @@ wmse_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CU
                 umma_commit_pair(&empty[st], (uint16_t)0x3u);
             }
             umma_commit_pair(acc_full, (uint16_t)0x3u);
-        } else if (lane == 0) {
+          }
+        } else if (elect_one()) {
             // ---------------- relay (peer): its half of a stage landed
             const uint32_t leader_ready = map_to_rank(smem_u32(ready), 0);
             for (int it = 0; it < nk; ++it) {
@@ -307,7 +309,7 @@ wmse_kernel(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CU
             }
         }
     } else if (warp == 2) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             // ---------------- relay (leader): its half of a stage landed
             for (int it = 0; it < nk; ++it) {
                 const int st = it % kWStages;
