@@ -129,7 +129,7 @@ aq_status aq_decode(const aq_layout* layout, int m, const void* planes, const vo
  * taken from tables of fp32 values (batch 1..2) or by 16-bit tensor-core multiplies of the stored
  * codewords themselves (above; where the books and the activations differ in type, the bf16 side
  * is scaled by powers of two into fp16, which is exact for values within 2^29 of the largest of
- * their book set, or of their token and slice). Larger layers at batch 9..16 with m <= 4 run the
+ * their book set, or of their token and slice). Larger layers with 8-bit codes at batch 9..16 with m <= 4 run the
  * tensor-memory kernel of aq_gemm, whose decoded weights are rounded once to fp16.
  *   x         : device, [batch][d_in] of x_dtype (AQ_F16 or AQ_BF16), row-major
  *   y         : device, [batch][d_out] of y_dtype (AQ_F16, AQ_BF16 or AQ_F32), row-major

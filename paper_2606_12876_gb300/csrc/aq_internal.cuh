@@ -305,7 +305,7 @@ __device__ __forceinline__ void unrotate_codes(const uint32_t (&w)[8], int o, ui
 #pragma unroll
     for (int i = 0; i < 8; ++i) t[i] = (rw & 4) ? v[(i + 4) & 7] : v[i];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) u[j] = __funnelshift_l(t[(j + 7) & 7], t[j], rb);   // (t[j] for rb = 0)
+    for (int j = 0; j < 8; ++j) u[j] = rb ? __funnelshift_l(t[(j + 7) & 7], t[j], rb) : t[j];
 }
 
 // The same for the 32 four-bit codes of a row's slice unit (four words; nibble q of word j of u is

@@ -1009,9 +1009,10 @@ static aq_status launch_reduce(const Dims& d, int P, const GemvArgs& a, const vo
 // that of gemv_cw, which at two token tiles is bound by the tensor pipe's legacy multiplies (64 a unit
 // of 32 rows, slice and book at 4 clocks; per SM, with its fixed cost). 14336 x 4096, m = 4, 16
 // tokens: 29 against 47.7 us; 1024 x 4096, m = 4: gemv_cw stays. bf16 activations are copied to the
-// workspace first (about 3000 clocks), which has room unless the layer has few rows.
+// workspace first (about 3000 clocks), which has room unless the layer has few rows. 8-bit codes
+// only: with 4-bit codes every intermediate of a GEMV is fp32 or exact, and stays so.
 static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt) {
-    if (batch <= 8) return false;
+    if (batch <= 8 || d.B != 8) return false;
     const size_t room = gemv_ws_planes(d, batch) * (size_t)d.rows_pad * 4;
     if (x_dt == AQ_BF16 && room < kWsStatusBytes + (size_t)batch * d.in * 2) return false;
     const double ts = ts_clocks(d, m, batch);
@@ -1026,7 +1027,7 @@ aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* book
     if (d.out == 0 || batch == 0) return AQ_OK;
     if (d.B == 4 && batch == 1)
         return launch_lut4(d, m, planes, books, scales, x, x_dt, y, y_dt, y_prev, st);
-    if (d.B != 16 && !y_prev && gemv_uses_ts(d, m, batch, x_dt)) {
+    if (!y_prev && gemv_uses_ts(d, m, batch, x_dt)) {
         const void* xh = x;
         float* fac = nullptr;
         if (x_dt == AQ_BF16) {   // the fp16 copy and the row factors take the partial sums' room

@@ -7,8 +7,10 @@
 // with no sum, no conversion and no rounding of weights on the way. In lane 4g + c (g < 8,
 // c < 4) the fragment holds row g (and g + 8), and the four K positions that the lane owns in
 // each of two multiplies are bound to the two halves of the codeword of one group; the K order
-// of a multiply is free, so lane c walks the groups 8c .. 8c+7 of a 256-input slice, one per
-// step, and the B fragment of the step is the same group of the lane's token g: one 16-byte load.
+// of a multiply is free, so in step j (0..7) of a 256-input slice lane c takes group 4j + c, and the B
+// fragment of the step is the same group of the lane's token g: one 16-byte load, 64 contiguous
+// bytes over the lanes c. (With groups 8c + j a load touched 32 lines instead of 8; every SM reads all
+// activations, and at about half an uncoalesced request a clock and SM that took 3.4-5 us a call.)
 //
 // Bound: shared-memory wavefronts of the codeword gathers (16 bytes per code; one 16-byte load of
 // a warp is four wavefronts when no two of the eight lanes of a phase meet in a bank group). Each
@@ -100,17 +102,29 @@ __device__ __forceinline__ int f16_exponent(float mx) {
     return mx > 0.0f ? max(-100, min(100, exponent_of(mx) - 14)) : 0;
 }
 
-// The codes of a row's slice unit as stored (position p holds group (p + o) mod 32) in group order.
+// The codes of a row's slice unit as stored (position p holds group (p + o) mod 32), staged in group
+// order (B = 8: the groups 4j + c of each c together).
 template <int B>
 __device__ __forceinline__ void store_unrotated(unsigned char* buf, int row, const uint4 (&raw)[2]) {
     if constexpr (B == 8) {
         const uint32_t w[8] = {raw[0].x, raw[0].y, raw[0].z, raw[0].w, raw[1].x, raw[1].y, raw[1].z, raw[1].w};
         uint32_t u[8];
         unrotate_codes(w, row, u);
+        // byte c of the eight words (groups 4j + c) together at byte 8c: two 4 x 4 byte transposes
+        uint32_t o[4][2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t t0 = prmt(u[4 * h], u[4 * h + 1], 0x5140u), t1 = prmt(u[4 * h + 2], u[4 * h + 3], 0x5140u);
+            const uint32_t t2 = prmt(u[4 * h], u[4 * h + 1], 0x7362u), t3 = prmt(u[4 * h + 2], u[4 * h + 3], 0x7362u);
+            o[0][h] = prmt(t0, t1, 0x5410u);
+            o[1][h] = prmt(t0, t1, 0x7632u);
+            o[2][h] = prmt(t2, t3, 0x5410u);
+            o[3][h] = prmt(t2, t3, 0x7632u);
+        }
         // the row's 16-byte halves change places in rows 4..7 of every eight: no bank conflicts
         const int sw = (row >> 2) & 1;
-        *(uint4*)(buf + row * 32 + sw * 16) = make_uint4(u[0], u[1], u[2], u[3]);
-        *(uint4*)(buf + row * 32 + (sw ^ 1) * 16) = make_uint4(u[4], u[5], u[6], u[7]);
+        *(uint4*)(buf + row * 32 + sw * 16) = make_uint4(o[0][0], o[0][1], o[1][0], o[1][1]);
+        *(uint4*)(buf + row * 32 + (sw ^ 1) * 16) = make_uint4(o[2][0], o[2][1], o[3][0], o[3][1]);
     } else {
         const uint32_t w[4] = {raw[0].x, raw[0].y, raw[0].z, raw[0].w};
         uint32_t u[4];
@@ -119,21 +133,35 @@ __device__ __forceinline__ void store_unrotated(unsigned char* buf, int row, con
     }
 }
 
-// The codes of groups 8c .. 8c+7 of a staged row: eight bytes (B = 8) or eight nibbles (B = 4).
+// The codes of groups 4j + c (j = 0..7) of a staged row: eight bytes (B = 8), or the low nibbles of the
+// halves of four words (B = 4).
 template <int B>
-__device__ __forceinline__ uint2 staged_codes(const unsigned char* buf, int row, int c) {
-    if constexpr (B == 8)
-        return *(const uint2*)(buf + row * 32 + (((c >> 1) ^ ((row >> 2) & 1)) * 16) + (c & 1) * 8);
-    else
-        return make_uint2(*(const uint32_t*)(buf + row * 16 + c * 4), 0u);
-}
-template <int B>
-__device__ __forceinline__ uint32_t code_of(const uint2& w, int j) {
-    if constexpr (B == 8) return prmt(j < 4 ? w.x : w.y, 0u, 0x4440u | (uint32_t)(j & 3));
-    else return (w.x >> (4 * j)) & 15u;
-}
+struct RowCodes {
+    uint32_t w[B == 8 ? 2 : 4];
+    __device__ __forceinline__ void load(const unsigned char* buf, int row, int c) {
+        if constexpr (B == 8) {
+            const uint2 v = *(const uint2*)(buf + row * 32 + (((c >> 1) ^ ((row >> 2) & 1)) * 16) + (c & 1) * 8);
+            w[0] = v.x;
+            w[1] = v.y;
+        } else {
+            const uint4 v = *(const uint4*)(buf + row * 16);
+            w[0] = v.x >> (4 * c);
+            w[1] = v.y >> (4 * c);
+            w[2] = v.z >> (4 * c);
+            w[3] = v.w >> (4 * c);
+        }
+    }
+    __device__ __forceinline__ uint32_t code(int j) const {
+        if constexpr (B == 8) return prmt(w[j >> 2], 0u, 0x4440u | (uint32_t)(j & 3));
+        else return (w[j >> 1] >> (16 * (j & 1))) & 15u;
+    }
+};
 
-template <int B, int BDT, int XDT, int NT>
+// SHORT: chains of eight multiplies from zero, added in fp32. The tensor pipe truncates as it
+// accumulates: over the 64 multiplies of a row and four books that costs a decimal of fp32 (relative error
+// of an fp32 y 1.2e-6; short chains 2e-7, fp32 sums 1.2e-7). It is the form wherever fp32 sums were
+// replaced (up to four tokens, and 4-bit codes); it takes 3 to 10 % more time.
+template <int B, int BDT, int XDT, int NT, bool SHORT>
 __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_constant__ CwArgs a) {
     constexpr int UNIT = unit_bytes(B), NC = 1 << B, NTOK = 8 * NT;
     constexpr int MDT = BDT == AQ_BF16 && XDT == AQ_BF16 ? AQ_BF16 : AQ_F16;   // operand type
@@ -148,6 +176,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = a.kc > 1 ? (int)cluster_rank() : 0;
     const int cid = (int)blockIdx.x / a.kc;
+    const int tb = (int)blockIdx.y * NTOK;               // first token
 
     // this warp's (slice, book) units u0 .. u1-1 of every row block of the cluster; u = s*m + k
     const long long U = (long long)a.S * a.m;
@@ -220,11 +249,11 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     auto load_b = [&](int s) {
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-            const int t = 8 * nt + g;
-            const uint4* src = (const uint4*)(a.x + (size_t)t * a.in) + s * 32 + 8 * c;
+            const int t = tb + 8 * nt + g;
+            const uint4* src = (const uint4*)(a.x + (size_t)t * a.in) + s * 32 + c;
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-                bf[nt][j] = t < a.batch && s * 32 + 8 * c + j < a.ng ? __ldg(src + j) : make_uint4(0u, 0u, 0u, 0u);
+                bf[nt][j] = t < a.batch && s * 32 + 4 * j + c < a.ng ? __ldg(src + 4 * j) : make_uint4(0u, 0u, 0u, 0u);
             if constexpr (kScaleX) {
                 float mx = 0.0f;
 #pragma unroll
@@ -286,24 +315,30 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
                 if (kScaleX && u > u0) fold();
                 load_b(s);
             }
-            uint2 cw[4];
+            RowCodes<B> cw[4];
 #pragma unroll
-            for (int rr = 0; rr < 4; ++rr) cw[rr] = staged_codes<B>(buf, g + 8 * rr, c);
+            for (int rr = 0; rr < 4; ++rr) cw[rr].load(buf, g + 8 * rr, c);
             __syncwarp();                                // the buffer may be refilled
             const uint32_t base = books_u + (uint32_t)k * (NC * mul);
+            float part[2][NT][4] = {};                   // (SHORT) the current chains
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 uint4 w[4];
 #pragma unroll
-                for (int rr = 0; rr < 4; ++rr) w[rr] = lds128(base + code_of<B>(cw[rr], j) * mul);
+                for (int rr = 0; rr < 4; ++rr) w[rr] = lds128(base + cw[rr].code(j) * mul);
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
                     for (int nt = 0; nt < NT; ++nt) {
-                        mma16<MDT>(acc[mt][nt], w[2 * mt].x, w[2 * mt + 1].x, w[2 * mt].y, w[2 * mt + 1].y,
-                                   bf[nt][j].x, bf[nt][j].y);
-                        mma16<MDT>(acc[mt][nt], w[2 * mt].z, w[2 * mt + 1].z, w[2 * mt].w, w[2 * mt + 1].w,
-                                   bf[nt][j].z, bf[nt][j].w);
+                        float(&d)[4] = SHORT ? part[mt][nt] : acc[mt][nt];
+                        mma16<MDT>(d, w[2 * mt].x, w[2 * mt + 1].x, w[2 * mt].y, w[2 * mt + 1].y, bf[nt][j].x, bf[nt][j].y);
+                        mma16<MDT>(d, w[2 * mt].z, w[2 * mt + 1].z, w[2 * mt].w, w[2 * mt + 1].w, bf[nt][j].z, bf[nt][j].w);
+                        if (SHORT && (j & 3) == 3)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                acc[mt][nt][e] += part[mt][nt][e];
+                                part[mt][nt][e] = 0.0f;
+                            }
                     }
             }
         }
@@ -329,7 +364,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
                     v += p;
                 }
         }
-        const int t = tid >> 5, o = rb * 32 + (tid & 31);
+        const int t = tb + (tid >> 5), o = rb * 32 + (tid & 31);
         if (tid >= i0 && tid < i1 && t < a.batch && o < a.out) {
             float r = v * bfac * bits_to_f32_rt(a.scales[o], a.scale_dt);
             const size_t yi = (size_t)t * a.out + o;
@@ -372,22 +407,27 @@ inline int cw_cluster(const Dims& d, int m, int sms, int* nclusters) {
     return best;
 }
 
-template <int B, int BDT, int XDT, int NT>
+template <int B, int BDT, int XDT, int NT, bool SHORT>
 aq_status run_cw(const Dims& d, CwArgs a, cudaStream_t st) {
     DeviceInfo di;
     if (aq_status e = device_info(&di); e != AQ_OK) return e;
-    auto kern = gemv_cw_kernel<B, BDT, XDT, NT>;
+    auto kern = gemv_cw_kernel<B, BDT, XDT, NT, SHORT>;
     a.cshift = cw_cshift(B, a.m);
     const size_t smem = cw_smem_bytes(B, a.m, a.cshift, NT);
     int occ = 0;
     if (aq_status e = prepare(kern, smem, kCwThreads, a.m, &occ); e != AQ_OK) return e;
     a.kc = cw_cluster(d, a.m, di.sms, &a.nclusters);
-    return launch_pdl_cluster(a.kc, kern, dim3(a.nclusters * a.kc), dim3(kCwThreads), smem, st, a);
+    return launch_pdl_cluster(a.kc, kern, dim3(a.nclusters * a.kc, (a.batch + 8 * NT - 1) / (8 * NT)),
+                              dim3(kCwThreads), smem, st, a);
 }
 
+// 4-bit codes: one token tile per CTA at any batch (two tiles of short chains do not fit the registers).
 template <int B, int BDT, int XDT>
 aq_status run_cw_nt(const Dims& d, const CwArgs& a, cudaStream_t st) {
-    return a.batch <= 8 ? run_cw<B, BDT, XDT, 1>(d, a, st) : run_cw<B, BDT, XDT, 2>(d, a, st);
+    if constexpr (B == 4) return run_cw<B, BDT, XDT, 1, true>(d, a, st);
+    else if (a.batch <= 4) return run_cw<B, BDT, XDT, 1, true>(d, a, st);
+    else if (a.batch <= 8) return run_cw<B, BDT, XDT, 1, false>(d, a, st);
+    else return run_cw<B, BDT, XDT, 2, false>(d, a, st);
 }
 
 template <int B>
