@@ -126,12 +126,14 @@ def _ptr(t):
 # The current stream as a raw handle, without building a Stream object per call (torch's
 # accessor when present).
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+# The current device without torch.cuda's lazy initialisation (tensors on the GPU exist by then).
+_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
 
 
 def _stream(stream):
     if stream is None:
         if _raw_stream is not None:
-            return _raw_stream(torch.cuda.current_device())
+            return _raw_stream(_current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream

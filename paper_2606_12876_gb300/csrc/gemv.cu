@@ -838,13 +838,23 @@ aq_status run_lut_layers(const Dims* ds, const GemvArgs* as, int n, int m, cudaS
     const long long grid_b = items < di.sms ? items : di.sms;
     const long long qb = items / grid_b, rb = items % grid_b;
     long long cost_b = 0;
-    if (n == 1)
+    if (n == 1) {
+        // (unit, offset) of a share's first item, stepped without divisions: this loop runs on every call
+        const long long qu = qb / d.RBc, qo = qb % d.RBc;
+        long long off = 0;
         for (long long b = 0; b < grid_b; ++b) {
-            const long long i0 = b * qb + (b < rb ? b : rb), i1 = i0 + qb + (b < rb ? 1 : 0);
-            const long long tables = (i1 - 1) / d.RBc - i0 / d.RBc + 1;
-            const long long c = tables * kTableItems + (i1 - i0);
+            const long long len = qb + (b < rb ? 1 : 0);
+            long long units_in = qu, end = off + qo + (b < rb ? 1 : 0);   // end: offset past the share's last item
+            if (end >= d.RBc) {
+                end -= d.RBc;
+                ++units_in;
+            }
+            const long long tables = units_in + (end > 0 ? 1 : 0);
+            const long long c = tables * kTableItems + len;
             if (c > cost_b) cost_b = c;
+            off = end;
         }
+    }
     else
         for (int l = 0; l < n; ++l)   // a CTA (at most qb + 1 items) then meets at most two layers
             if ((long long)ds[l].S * m * ds[l].RBc < qb + 1) return AQ_ERR_UNSUPPORTED;

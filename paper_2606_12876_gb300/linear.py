@@ -6,14 +6,15 @@ codebooks in torch device memory, or (from_host) holds only a resident prefix in
 that loads further codebooks from host memory at run time. All work is done by libaq through
 the binding in this package.
 """
+import ctypes
 import weakref
 
 import numpy as np
 import torch
 
-from . import (AQ_BF16, AQ_F16, AQ_F32, AQ_LAYOUT_STATIC_WEIGHTS, DTYPES, TORCH_DTYPES, Layout,
-               aq_decode, aq_gemm, aq_gemv_group, gemv_group_workspace_bytes,
-               aq_gemv, aq_gemv_refine, aq_pack, aq_store_books, aq_store_create, aq_wmse,
+from . import (AQ_BF16, AQ_F16, AQ_F32, AQ_LAYOUT_STATIC_WEIGHTS, AQError, DTYPES, TORCH_DTYPES, Layout,
+               aq_decode, aq_gemv_group, gemv_group_workspace_bytes,
+               aq_gemv_refine, aq_pack, aq_store_books, aq_store_create, aq_wmse,
                wmse_workspace_bytes, aq_workspace_init,
                aq_store_device_bytes, aq_store_planes, aq_store_scales, aq_store_set_prefix,
                gemm_workspace_bytes, gemv_workspace_bytes, lib, packed_bytes,
@@ -58,7 +59,7 @@ class AQLinear:
         torch.cuda.current_stream(self.device).synchronize()
         self.layout.flags = AQ_LAYOUT_STATIC_WEIGHTS
         self.codes = codes_t if keep_codes else None
-        self._ws = {}
+        self._ws, self._ws_sizes = {}, {}
         self.store, self.resident = None, M
 
     @classmethod
@@ -100,7 +101,7 @@ class AQLinear:
         self.planes = aq_store_planes(self.store)
         self.books = aq_store_books(self.store)
         self.scales = aq_store_scales(self.store)
-        self.codes, self._ws, self.resident = None, {}, 0
+        self.codes, self._ws, self._ws_sizes, self.resident = None, {}, {}, 0
         self.set_prefix(m)
         return self
 
@@ -139,23 +140,45 @@ class AQLinear:
         """The first m planes: the only code bytes a prefix-m call reads."""
         return self.planes[: packed_bytes(self.layout, m)]
 
-    def _workspace(self, kind, n):
-        # One workspace per (kind, stream), grown on demand; GEMV calls (batch <= 16) also
-        # remember the size per batch, so a repeated call makes no size query.
-        stream = _stream(None)
+    def _workspace(self, kind, n, stream):
+        # One workspace per (kind, stream), grown on demand; the sizes of the latest batches and
+        # token counts are remembered, so a repeated call makes no size query.
+        sizes = self._ws_sizes
+        nbytes = sizes.get((kind, n))
+        if nbytes is None:
+            if len(sizes) >= 256:
+                sizes.clear()
+            nbytes = (gemv_workspace_bytes if kind == "gemv" else gemm_workspace_bytes)(self.layout, n)
+            sizes[(kind, n)] = nbytes
         key = (kind, stream)
         ws = self._ws.get(key)
-        if kind == "gemv":
-            known = self._ws.get((kind, stream, n))
-            if known is not None and ws is not None and ws.numel() >= known:
-                return ws
-        nbytes = (gemv_workspace_bytes if kind == "gemv" else gemm_workspace_bytes)(self.layout, n)
-        if ws is None or ws.numel() < nbytes:
-            ws = workspace(nbytes, self.device)
-            self._ws[key] = ws
-        if kind == "gemv":
-            self._ws[(kind, stream, n)] = nbytes
+        if ws is None or ws[1] < nbytes:
+            t = workspace(nbytes, self.device)
+            ws = self._ws[key] = (t, t.numel(), t.data_ptr())
         return ws
+
+    def _product(self, kind, x, m, y, y_dtype):
+        # One pass of argument marshalling: an eager call of a small layer is bound by the host.
+        xd = _X_CODES.get(x.dtype)
+        if xd is None:
+            xd = _dtype_code(x.dtype)
+        yd = xd if y_dtype is None else y_dtype
+        n = x.shape[0]
+        if y is None:
+            y = torch.empty((n, self.out), dtype=TORCH_DTYPES[yd], device=self.device)
+        self._check_m(m)
+        stream = _stream(None)
+        ws = self._workspace(kind, n, stream)
+        planes, books, scales = self.planes, self.books, self.scales
+        if self.store is None:
+            planes, books, scales = planes.data_ptr(), books.data_ptr(), scales.data_ptr()
+        L = lib()
+        status = (L.aq_gemv if kind == "gemv" else L.aq_gemm)(
+            ctypes.byref(self.layout), m, planes, books, scales, x.data_ptr(), xd, n, y.data_ptr(), yd, ws[2], ws[1],
+            stream)
+        if status:
+            raise AQError(status, "aq_" + kind)
+        return y
 
     def decode(self, m, out=None):
         """Dense W_m [out][in] in the book dtype (bit-exact contract of aq.h)."""
@@ -168,15 +191,7 @@ class AQLinear:
 
     def gemv(self, x, m, y=None, y_dtype=None):
         """y = x W_m^T for x of shape [batch <= 16, in]."""
-        xd = _dtype_code(x.dtype)
-        yd = xd if y_dtype is None else y_dtype
-        batch = x.shape[0]
-        if y is None:
-            y = torch.empty(batch, self.out, dtype=TORCH_DTYPES[yd], device=self.device)
-        self._check_m(m)
-        ws = self._workspace("gemv", batch)
-        aq_gemv(self.layout, m, self.planes, self.books, self.scales, x, xd, batch, y, yd, ws)
-        return y
+        return self._product("gemv", x, m, y, y_dtype)
 
     def refine(self, x, m, y_prev, y=None):
         """y = y_prev + x (s o C_{m-1}[b_{m-1}])^T: raises a prefix-(m-1) result to prefix m,
@@ -188,22 +203,14 @@ class AQLinear:
         if y is None:
             y = torch.empty(batch, self.out, dtype=TORCH_DTYPES[yd], device=self.device)
         self._check_m(m)
-        ws = self._workspace("gemv", batch)
+        ws = self._workspace("gemv", batch, _stream(None))[0]
         aq_gemv_refine(self.layout, m, self.planes, self.books, self.scales, x, xd, batch, y_prev,
                        y, yd, ws)
         return y
 
     def gemm(self, x, m, y=None, y_dtype=None):
         """y = x W_m^T for x of shape [tokens, in] on the tensor cores."""
-        xd = _dtype_code(x.dtype)
-        yd = xd if y_dtype is None else y_dtype
-        tokens = x.shape[0]
-        if y is None:
-            y = torch.empty(tokens, self.out, dtype=TORCH_DTYPES[yd], device=self.device)
-        self._check_m(m)
-        ws = self._workspace("gemm", tokens)
-        aq_gemm(self.layout, m, self.planes, self.books, self.scales, x, xd, tokens, y, yd, ws)
-        return y
+        return self._product("gemm", x, m, y, y_dtype)
 
     def wmse(self, W, H, lam=None):
         """Distortion of every prefix (Sec. 2.2 Eq. wmse-task, Sec. 5): a float64 device tensor
@@ -253,6 +260,9 @@ def gemv_group(layers, x, m, ys=None, y_dtype=None):
     aq_gemv_group(layouts, m, [lin.planes for lin in layers], [lin.books for lin in layers],
                   [lin.scales for lin in layers], x, xd, batch, ys, yd, ws)
     return ys
+
+
+_X_CODES = {torch.float16: AQ_F16, torch.bfloat16: AQ_BF16}
 
 
 def _dtype_code(dt):
