@@ -490,7 +490,7 @@ bool ts_plan(const Dims& d, int m, int tokens, const DeviceInfo& di, TsPlan* p) 
             if (qr * 53.0 * m + p->n * 0.45 > stage_clk) stage_clk = qr * 53.0 * m + p->n * 0.45;
             if (chain > stage_clk) stage_clk = chain;
             const double t = waves * (spc / 4 * 16 * stage_clk + (spc % 4 ? 16 * chain : 0.0) + 7500.0 +
-                                      (kc > 1 ? 3000.0 : 0.0) + p->n * 16.0);
+                                      (kc == 1 ? 0.0 : kc < 8 ? 3000.0 : 6000.0) + p->n * 16.0);
             if (best < 0.0 || t < best) {
                 best = t;
                 p->qr = qr;

@@ -157,11 +157,11 @@ struct RowCodes {
     }
 };
 
-// SHORT: chains of eight multiplies from zero, added in fp32. The tensor pipe truncates as it
-// accumulates: over the 64 multiplies of a row and four books that costs a decimal of fp32 (relative error
-// of an fp32 y 1.2e-6; short chains 2e-7, fp32 sums 1.2e-7). It is the form wherever fp32 sums were
-// replaced (up to four tokens, and 4-bit codes); it takes 3 to 10 % more time.
-template <int B, int BDT, int XDT, int NT, bool SHORT>
+// CHAIN: multiplies accumulated by the tensor pipe before an fp32 add takes them over (0: all of a unit
+// and the next ones). The pipe truncates as it accumulates: over the 64 multiplies of a row and four books
+// that costs a decimal of fp32 (relative error of an fp32 y 1.2e-6; chains of eight 2e-7; fp32 sums 1.2e-7).
+// Chains of eight (3 to 10 % more time) stand where calls had fp32 sums: up to four tokens, 4-bit codes.
+template <int B, int BDT, int XDT, int NT, int CHAIN>
 __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_constant__ CwArgs a) {
     constexpr int UNIT = unit_bytes(B), NC = 1 << B, NTOK = 8 * NT;
     constexpr int MDT = BDT == AQ_BF16 && XDT == AQ_BF16 ? AQ_BF16 : AQ_F16;   // operand type
@@ -279,6 +279,9 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
         float* rp = red + (pass & 1) * cw_red_floats(NT);
         float* mine = rp + (size_t)warp * NTOK * kCwPitch;
         bool first = true;
+        // the row scale of the output this thread finishes, requested before the pass's gathers
+        const int my_o = rb * 32 + (tid & 31);
+        const float my_s = tid < 32 * NTOK && my_o < a.out ? bits_to_f32_rt(a.scales[my_o], a.scale_dt) : 0.0f;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
@@ -320,7 +323,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
             for (int rr = 0; rr < 4; ++rr) cw[rr].load(buf, g + 8 * rr, c);
             __syncwarp();                                // the buffer may be refilled
             const uint32_t base = books_u + (uint32_t)k * (NC * mul);
-            float part[2][NT][4] = {};                   // (SHORT) the current chains
+            float part[2][NT][4] = {};                   // (CHAIN > 0) the current chains
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 uint4 w[4];
@@ -330,10 +333,10 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
                 for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
                     for (int nt = 0; nt < NT; ++nt) {
-                        float(&d)[4] = SHORT ? part[mt][nt] : acc[mt][nt];
+                        float(&d)[4] = CHAIN ? part[mt][nt] : acc[mt][nt];
                         mma16<MDT>(d, w[2 * mt].x, w[2 * mt + 1].x, w[2 * mt].y, w[2 * mt + 1].y, bf[nt][j].x, bf[nt][j].y);
                         mma16<MDT>(d, w[2 * mt].z, w[2 * mt + 1].z, w[2 * mt].w, w[2 * mt + 1].w, bf[nt][j].z, bf[nt][j].w);
-                        if (SHORT && (j & 3) == 3)
+                        if (CHAIN == 8 && (j & 3) == 3)
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 acc[mt][nt][e] += part[mt][nt][e];
@@ -364,9 +367,9 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
                     v += p;
                 }
         }
-        const int t = tb + (tid >> 5), o = rb * 32 + (tid & 31);
+        const int t = tb + (tid >> 5), o = my_o;
         if (tid >= i0 && tid < i1 && t < a.batch && o < a.out) {
-            float r = v * bfac * bits_to_f32_rt(a.scales[o], a.scale_dt);
+            float r = v * bfac * my_s;
             const size_t yi = (size_t)t * a.out + o;
             if (a.y_prev)
                 r = (a.y_dt == AQ_F32 ? ((const float*)a.y_prev)[yi]
@@ -384,8 +387,9 @@ inline int cw_cshift(int B, int m) { return B == 4 || m <= 4 ? 3 : 2; }
 // CTAs per cluster: the split with the smallest estimated time of the busiest cluster, in clocks:
 // passes over its row blocks times the units of a warp (a unit's gathers are 128 wavefronts, plus
 // about 24 of staging, shared by the SM's active warps, or the latency of its eight steps) and the
-// reduction of a pass (with a cluster barrier when kc > 1). Clusters of 2, 4 and 8 that are
-// resident at once: 76, 36 and 16 on 152 SMs.
+// reduction of a pass, plus what a cluster launch and its barriers cost over a plain one (measured
+// about 2 us for two or four CTAs, 6 for eight: 512 x 4096, m = 4 took 10.8 us in clusters of eight).
+// Clusters of 2, 4 and 8 that are resident at once: 76, 36 and 16 on 152 SMs.
 inline int cw_cluster(const Dims& d, int m, int sms, int* nclusters) {
     int best = 1;
     double best_t = -1.0;
@@ -397,7 +401,8 @@ inline int cw_cluster(const Dims& d, int m, int sms, int* nclusters) {
         const long long units = (U + 16 * kc - 1) / (16 * kc);
         const long long active = U < 16 * kc ? (U + kc - 1) / kc : 16;
         const double unit_clk = active * 152 > 900 ? active * 152.0 : 900.0;
-        const double t = (double)((d.RBc + nc - 1) / nc) * (units * unit_clk + (kc > 1 ? 1100.0 : 400.0));
+        const double t = (double)((d.RBc + nc - 1) / nc) * (units * unit_clk + (kc > 1 ? 1100.0 : 400.0)) +
+                         (kc == 1 ? 0.0 : kc < 8 ? 3500.0 : 11000.0);
         if (best_t < 0.0 || t < best_t) {
             best_t = t;
             best = kc;
@@ -407,11 +412,11 @@ inline int cw_cluster(const Dims& d, int m, int sms, int* nclusters) {
     return best;
 }
 
-template <int B, int BDT, int XDT, int NT, bool SHORT>
+template <int B, int BDT, int XDT, int NT, int CHAIN>
 aq_status run_cw(const Dims& d, CwArgs a, cudaStream_t st) {
     DeviceInfo di;
     if (aq_status e = device_info(&di); e != AQ_OK) return e;
-    auto kern = gemv_cw_kernel<B, BDT, XDT, NT, SHORT>;
+    auto kern = gemv_cw_kernel<B, BDT, XDT, NT, CHAIN>;
     a.cshift = cw_cshift(B, a.m);
     const size_t smem = cw_smem_bytes(B, a.m, a.cshift, NT);
     int occ = 0;
@@ -424,10 +429,10 @@ aq_status run_cw(const Dims& d, CwArgs a, cudaStream_t st) {
 // 4-bit codes: one token tile per CTA at any batch (two tiles of short chains do not fit the registers).
 template <int B, int BDT, int XDT>
 aq_status run_cw_nt(const Dims& d, const CwArgs& a, cudaStream_t st) {
-    if constexpr (B == 4) return run_cw<B, BDT, XDT, 1, true>(d, a, st);
-    else if (a.batch <= 4) return run_cw<B, BDT, XDT, 1, true>(d, a, st);
-    else if (a.batch <= 8) return run_cw<B, BDT, XDT, 1, false>(d, a, st);
-    else return run_cw<B, BDT, XDT, 2, false>(d, a, st);
+    if constexpr (B == 4) return run_cw<B, BDT, XDT, 1, 8>(d, a, st);
+    else if (a.batch <= 4) return run_cw<B, BDT, XDT, 1, 8>(d, a, st);
+    else if (a.batch <= 8) return run_cw<B, BDT, XDT, 1, 0>(d, a, st);
+    else return run_cw<B, BDT, XDT, 2, 0>(d, a, st);
 }
 
 template <int B>
