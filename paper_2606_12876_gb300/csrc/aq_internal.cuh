@@ -97,16 +97,18 @@ aq_status launch_decode(const Dims& d, int m, const void* planes, const void* bo
 aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* books,
                       const void* scales, const void* x, int x_dt, int batch, void* y,
                       int y_dt, void* ws, cudaStream_t st, const void* y_prev = nullptr);
-// The same for 2..16 tokens with 4- or 8-bit codes in one kernel (gemv_cw.cu).
-aq_status launch_cw(const Dims& d, int m, const void* planes, const void* books, const void* scales,
-                    const void* x, int x_dt, int batch, void* y, int y_dt, const void* y_prev,
-                    cudaStream_t st);
+// The same for 2..16 tokens with 4- or 8-bit codes in one kernel (gemv_cw.cu), for n (<= 4) layers that
+// share x, the code width, the types and m (n = 1: an ordinary call).
+aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, const void* const* books,
+                    const void* const* scales, const void* x, int x_dt, int batch, void* const* y, int y_dt,
+                    const void* y_prev, cudaStream_t st);
 // The product with the decoded weights in tensor memory (gemm_ts.cu): its estimated time in clocks
-// (below 0: not served), and the launch (x: fp16; xfac: per-token factors or null; ws: its first word
-// is the status word).
+// (below 0: not served), and the launch, of n (<= 4) layers as above (x: fp16; xfac: per-token factors
+// or null; ws: its first word is the status word).
 double ts_clocks(const Dims& d, int m, int tokens);
-aq_status launch_ts(const Dims& d, int m, const void* planes, const void* books, const void* scales,
-                    const void* x, const float* xfac, int tokens, void* y, int y_dt, void* ws, cudaStream_t st);
+aq_status launch_ts(const Dims* ds, int n, int m, const void* const* planes, const void* const* books,
+                    const void* const* scales, const void* x, const float* xfac, int tokens, void* const* y,
+                    int y_dt, void* ws, cudaStream_t st);
 // bf16 activations as fp16, each token row scaled by a power of two into fp16's range: the copy
 // [tokens][in] at dst, the rows' factors at fac.
 aq_status launch_x_to_f16(const void* x, void* dst, float* fac, int in, int tokens, cudaStream_t st);

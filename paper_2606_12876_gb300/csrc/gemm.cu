@@ -1072,7 +1072,7 @@ aq_status launch_gemm(const Dims& d, int m, const void* planes, const void* book
         xfac = fac;
     }
     if (ts)
-        return launch_ts(d, m, planes, books, scales, xh, xfac, tokens, y, y_dt, ws, st);
+        return launch_ts(&d, 1, m, &planes, &books, &scales, xh, xfac, tokens, &y, y_dt, ws, st);
     if (gemm_uses_dense(d, m, tokens)) {
         uint16_t* w16 = (uint16_t*)((char*)ws + gemm_w16_offset(d, tokens));
         if (d.B == 4)   // the in-loop decoders read 8-bit codes; 4-bit layouts always go dense

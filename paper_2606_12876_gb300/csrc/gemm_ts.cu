@@ -49,17 +49,24 @@ constexpr int kTsMaxM = 4;          // prefixes compiled for the sums form
 constexpr int kTsRing = 8;          // weight stages in tensor memory (32 columns each, from column 256)
 constexpr int kTsBars = 2 * kTsRing + 1;
 
-struct TsArgs {
+// One layer of a launch; a launch holds one layer, or several that share the activations and the split
+// of K (aq_gemv_group), their tiles one after the other.
+struct TsLayer {
     const uint8_t* planes;
     const uint16_t *books, *scales;
     void* y;
+    int out, rows_pad, tile0;       // tile0: the layer's first row tile of the grid
+    size_t plane_bytes;
+};
+struct TsArgs {
+    TsLayer L[4];
+    int nlayers;
     const float* xfac;              // per-token factor of the activations, or null
     unsigned int* status;
-    int y_dt, scale_dt, tokens, out, in, ng, rows_pad, S;
+    int y_dt, scale_dt, tokens, in, ng, S;
     int cshift, qr, kc, n, nsb, spc;   // n: tokens of a tile (multiple of 16); nsb: activation stages;
     int books_off, bar_off;            // spc: slices per CTA; shared-memory offsets
     int static_weights;
-    size_t plane_bytes;
 };
 
 template <int B, int BDT, int MB, bool Q4>   // Q4: four row quarters
@@ -79,7 +86,10 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     __shared__ unsigned int s_wmax[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = a.kc > 1 ? (int)cluster_rank() : 0;
-    const int row0 = (int)blockIdx.x / a.kc * 32 * a.qr;
+    int tile = (int)blockIdx.x / a.kc, layer = 0;
+    while (layer + 1 < a.nlayers && tile >= a.L[layer + 1].tile0) ++layer;
+    const TsLayer& L = a.L[layer];
+    const int row0 = (tile - L.tile0) * 32 * a.qr;
     const int t0 = (int)blockIdx.y * a.n;
     const int sl0 = rank * a.spc, nsl = max(0, min(a.S - sl0, a.spc));   // this CTA's slices
 
@@ -111,7 +121,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 #pragma unroll
         for (int l = 0; l < kPer; ++l) {
             const int i = tid + l * kTsThreads;
-            c[l] = i < m * NC ? __ldg((const uint4*)a.books + i) : make_uint4(0u, 0u, 0u, 0u);
+            c[l] = i < m * NC ? __ldg((const uint4*)L.books + i) : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
         for (int l = 0; l < kPer; ++l) {
@@ -136,13 +146,13 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         }
     };
     // the codes of a round's slices, HBM to L2
-    const int rows_here = max(0, min(32 * a.qr, a.rows_pad - row0));
+    const int rows_here = max(0, min(32 * a.qr, L.rows_pad - row0));
     auto prefetch_round = [&](int r) {
         if (rows_here > 0)
             for (int w = 0; w < 4 && 4 * r + w < nsl; ++w)
                 for (int k = 0; k < m; ++k)
-                    prefetch_l2(a.planes + (size_t)k * a.plane_bytes +
-                                    ((size_t)(sl0 + 4 * r + w) * a.rows_pad + row0) * UNIT,
+                    prefetch_l2(L.planes + (size_t)k * L.plane_bytes +
+                                    ((size_t)(sl0 + 4 * r + w) * L.rows_pad + row0) * UNIT,
                                 (uint32_t)(rows_here * UNIT));
     };
     if (a.static_weights) {   // read-only weights: requested before the preceding kernel has finished
@@ -162,7 +172,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         stage_books();
     }
     for (int i = tid; i < 32 * a.qr; i += kTsThreads)
-        scale_s[i] = row0 + i < a.out ? bits_to_f32_rt(a.scales[row0 + i], a.scale_dt) * bfac : 0.0f;
+        scale_s[i] = row0 + i < L.out ? bits_to_f32_rt(L.scales[row0 + i], a.scale_dt) * bfac : 0.0f;
     for (int i = tid; i < a.n; i += kTsThreads) xf_s[i] = a.xfac && t0 + i < a.tokens ? a.xfac[t0 + i] : 1.0f;
     tc_fence_before();
     __syncthreads();          // books staged, barriers initialised, tensor memory allocated
@@ -232,7 +242,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         // ---------------- decoders
         const int q = warp & 3, ws = warp >> 2;
         const int row = row0 + q * 32 + lane;
-        const bool row_in = row < a.rows_pad;
+        const bool row_in = row < L.rows_pad;
         const uint32_t mul = 16u << a.cshift;
         const uint32_t books_u = smem_u32(books_s) + ((uint32_t)(lane & ((1 << a.cshift) - 1)) << 4);
         const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + 256;
@@ -244,7 +254,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 #pragma unroll
             for (int i = 0; i < NW; ++i) raw[i] = 0u;
             if (row_in) {
-                const uint8_t* src = a.planes + (size_t)k * a.plane_bytes + ((size_t)s * a.rows_pad + row) * UNIT;
+                const uint8_t* src = L.planes + (size_t)k * L.plane_bytes + ((size_t)s * L.rows_pad + row) * UNIT;
                 if constexpr (B == 8) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
@@ -385,13 +395,13 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     }
     const int ntok = min(a.n, a.tokens - t0), share = (ntok + a.kc - 1) / a.kc;
     const int ta = rank * share, tb = min(ntok, ta + share);
-    const bool vec = (a.out & 7) == 0;
+    const bool vec = (L.out & 7) == 0;
     // a thread finishes eight rows (always the same ones) of every nt-th token
     const int R8 = R / 8, nt = kTsThreads / R8, rr = tid % R8 * 8, o = row0 + rr;
     float sc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) sc[e] = scale_s[rr + e];
-    for (int tl = ta + tid / R8; tl < tb && tid < nt * R8 && o < a.out; tl += nt) {
+    for (int tl = ta + tid / R8; tl < tb && tid < nt * R8 && o < L.out; tl += nt) {
         const int t = t0 + tl;
         float v[8];
 #pragma unroll
@@ -424,15 +434,15 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 for (int e = 0; e < 8; ++e) v[e] += p[i][e];
         }
         const float xf = xf_s[tl];
-        const size_t yi = (size_t)t * a.out + o;
-        const int nv = min(8, a.out - o);
+        const size_t yi = (size_t)t * L.out + o;
+        const int nv = min(8, L.out - o);
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = v[e] * xf * sc[e];
         if (vec && a.y_dt == AQ_F32) {
-            *(float4*)((float*)a.y + yi) = make_float4(v[0], v[1], v[2], v[3]);
-            *(float4*)((float*)a.y + yi + 4) = make_float4(v[4], v[5], v[6], v[7]);
+            *(float4*)((float*)L.y + yi) = make_float4(v[0], v[1], v[2], v[3]);
+            *(float4*)((float*)L.y + yi + 4) = make_float4(v[4], v[5], v[6], v[7]);
         } else if (vec) {
-            *(uint4*)((uint16_t*)a.y + yi) =
+            *(uint4*)((uint16_t*)L.y + yi) =
                 a.y_dt == AQ_F16
                     ? make_uint4(round_pack2<AQ_F16>(v[0], v[1]), round_pack2<AQ_F16>(v[2], v[3]),
                                  round_pack2<AQ_F16>(v[4], v[5]), round_pack2<AQ_F16>(v[6], v[7]))
@@ -442,8 +452,8 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 #pragma unroll
             for (int e = 0; e < 8; ++e)
                 if (e < nv) {
-                    if (a.y_dt == AQ_F32) ((float*)a.y)[yi + e] = v[e];
-                    else ((uint16_t*)a.y)[yi + e] = a.y_dt == AQ_F16 ? f32_to_bits<AQ_F16>(v[e]) : f32_to_bits<AQ_BF16>(v[e]);
+                    if (a.y_dt == AQ_F32) ((float*)L.y)[yi + e] = v[e];
+                    else ((uint16_t*)L.y)[yi + e] = a.y_dt == AQ_F16 ? f32_to_bits<AQ_F16>(v[e]) : f32_to_bits<AQ_BF16>(v[e]);
                 }
         }
     }
@@ -453,7 +463,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 // ---- host side ------------------------------------------------------------------------------
 
 struct TsPlan {
-    int n, ntiles, qr, kc, spc, cshift, nsb, books_off, bar_off;
+    int n, ntiles, qr, kc, spc, cshift, nsb, books_off, bar_off;   // (kc, spc: of the first layer)
     size_t smem;
     double clocks;                     // estimated time of the call
 };
@@ -466,7 +476,10 @@ struct TsPlan {
 // the gathers of 8 groups per row and book at 60 % of 8 codes a clock, and the activations' way
 // through it; a decoder warp's own chain (120 m + 165, a stage in four being its own), which bounds
 // one or two quarters and a last round of fewer than four slices.
-bool ts_plan(const Dims& d, int m, int tokens, const DeviceInfo& di, TsPlan* p) {
+// With a group of layers (nl > 1; the same K and number of books, so the same kc and spc each), the
+// tile height is chosen for the tiles of all of them and kc is the given one.
+bool ts_plan(const Dims* ds, int nl, int m, int tokens, const DeviceInfo& di, TsPlan* p, int only_kc = 0) {
+    const Dims& d = ds[0];
     if ((d.B != 8 && d.B != 4) || m > kTsMaxM) return false;
     p->ntiles = (tokens + 255) / 256;
     p->n = ((tokens + p->ntiles - 1) / p->ntiles + 15) / 16 * 16;
@@ -480,8 +493,10 @@ bool ts_plan(const Dims& d, int m, int tokens, const DeviceInfo& di, TsPlan* p) 
     double best = -1.0;
     for (int qr = 1; qr <= 4; ++qr)
         for (int kc = 1; kc <= 8; kc *= 2) {
-            if (kc > d.S) continue;
-            const long long tiles = (long long)((d.out + 32 * qr - 1) / (32 * qr)) * p->ntiles;
+            if (kc > d.S || (only_kc && kc != only_kc)) continue;
+            long long tiles = 0;
+            for (int l = 0; l < nl; ++l) tiles += (ds[l].out + 32 * qr - 1) / (32 * qr);
+            tiles *= p->ntiles;
             const int cap = kc == 1 ? di.sms : kc == 2 ? di.sms / 2 : kc == 4 ? di.sms * 9 / 38 : di.sms * 2 / 19;
             const int spc = (d.S + kc - 1) / kc;
             const long long waves = (tiles + cap - 1) / cap;
@@ -531,21 +546,9 @@ aq_status run_ts_m(const TsPlan& p, const CUtensorMap& map, const TsArgs& a, int
     }
 }
 
-}  // namespace
-
-double ts_clocks(const Dims& d, int m, int tokens) {
-    DeviceInfo di;
-    TsPlan p;
-    return device_info(&di) == AQ_OK && ts_plan(d, m, tokens, di, &p) ? p.clocks : -1.0;
-}
-
-// x: fp16 [tokens][in], 16-byte aligned.
-aq_status launch_ts(const Dims& d, int m, const void* planes, const void* books, const void* scales,
-                    const void* x, const float* xfac, int tokens, void* y, int y_dt, void* ws, cudaStream_t st) {
-    DeviceInfo di;
-    if (aq_status e = device_info(&di); e != AQ_OK) return e;
-    TsPlan p;
-    if (!ts_plan(d, m, tokens, di, &p)) return AQ_ERR_UNSUPPORTED;
+// One launch: plan p, the layers of a filled in, `tiles` row tiles.
+aq_status launch_ts_set(const Dims& d, int m, const TsPlan& p, TsArgs a, int tiles, const void* x, const float* xfac,
+                        int tokens, int y_dt, void* ws, cudaStream_t st) {
     EncodeTiledFn encode;
     if (aq_status e = get_encode_fn(&encode); e != AQ_OK) return e;
     CUtensorMap map;
@@ -558,20 +561,13 @@ aq_status launch_ts(const Dims& d, int m, const void* planes, const void* books,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return AQ_ERR_CUDA;
-    TsArgs a = {};
-    a.planes = (const uint8_t*)planes;
-    a.books = (const uint16_t*)books;
-    a.scales = (const uint16_t*)scales;
-    a.y = y;
     a.xfac = xfac;
     a.status = (unsigned int*)ws;
     a.y_dt = y_dt;
     a.scale_dt = d.scale_dt;
     a.tokens = tokens;
-    a.out = d.out;
     a.in = d.in;
     a.ng = d.ng;
-    a.rows_pad = d.rows_pad;
     a.S = d.S;
     a.cshift = p.cshift;
     a.qr = p.qr;
@@ -581,14 +577,76 @@ aq_status launch_ts(const Dims& d, int m, const void* planes, const void* books,
     a.spc = p.spc;
     a.books_off = p.books_off;
     a.bar_off = p.bar_off;
-    a.static_weights = (d.flags & AQ_LAYOUT_STATIC_WEIGHTS) ? 1 : 0;
-    a.plane_bytes = d.plane_bytes;
-    const int tiles = (d.out + 32 * p.qr - 1) / (32 * p.qr);
     if (d.B == 4)
         return d.book_dt == AQ_BF16 ? run_ts_m<4, AQ_BF16>(p, map, a, m, tiles, st)
                                     : run_ts_m<4, AQ_F16>(p, map, a, m, tiles, st);
     return d.book_dt == AQ_BF16 ? run_ts_m<8, AQ_BF16>(p, map, a, m, tiles, st)
                                 : run_ts_m<8, AQ_F16>(p, map, a, m, tiles, st);
+}
+
+}  // namespace
+
+double ts_clocks(const Dims& d, int m, int tokens) {
+    DeviceInfo di;
+    TsPlan p;
+    return device_info(&di) == AQ_OK && ts_plan(&d, 1, m, tokens, di, &p) ? p.clocks : -1.0;
+}
+
+// x: fp16 [tokens][in], 16-byte aligned. n layers that share it: those whose own plans have the same
+// cluster size go together (their sums are then those of their own calls), unless launches of their own
+// are estimated to be faster.
+aq_status launch_ts(const Dims* ds, int n, int m, const void* const* planes, const void* const* books,
+                    const void* const* scales, const void* x, const float* xfac, int tokens, void* const* y,
+                    int y_dt, void* ws, cudaStream_t st) {
+    DeviceInfo di;
+    if (aq_status e = device_info(&di); e != AQ_OK) return e;
+    TsPlan own[4];
+    for (int l = 0; l < n; ++l)
+        if (!ts_plan(&ds[l], 1, m, tokens, di, &own[l])) return AQ_ERR_UNSUPPORTED;
+    bool done[4] = {};
+    for (int f = 0; f < n; ++f) {
+        if (done[f]) continue;
+        Dims set[4];
+        int idx[4], ns = 0;
+        TsPlan p = own[f];
+        double apart = 0.0;
+        for (int l = f; l < n; ++l) {
+            if (done[l] || own[l].kc != own[f].kc) continue;
+            set[ns] = ds[l];
+            idx[ns++] = l;
+            apart += own[l].clocks;
+            // a launch of its own costs about 3000 clocks more than its tiles
+            TsPlan joint;
+            if (ns > 1) {
+                if (ts_plan(set, ns, m, tokens, di, &joint, own[f].kc) && joint.clocks < apart + 3000.0 * (ns - 1)) p = joint;
+                else {
+                    apart -= own[l].clocks;
+                    --ns;
+                }
+            }
+        }
+        TsArgs a = {};
+        a.nlayers = ns;
+        a.static_weights = 1;
+        int tiles = 0;
+        for (int i = 0; i < ns; ++i) {
+            const int l = idx[i];
+            done[l] = true;
+            TsLayer& L = a.L[i];
+            L.planes = (const uint8_t*)planes[l];
+            L.books = (const uint16_t*)books[l];
+            L.scales = (const uint16_t*)scales[l];
+            L.y = y[l];
+            L.out = ds[l].out;
+            L.rows_pad = ds[l].rows_pad;
+            L.plane_bytes = ds[l].plane_bytes;
+            L.tile0 = tiles;
+            tiles += (ds[l].out + 32 * p.qr - 1) / (32 * p.qr);
+            if (!(ds[l].flags & AQ_LAYOUT_STATIC_WEIGHTS)) a.static_weights = 0;
+        }
+        if (aq_status e = launch_ts_set(ds[f], m, p, a, tiles, x, xfac, tokens, y_dt, ws, st); e != AQ_OK) return e;
+    }
+    return AQ_OK;
 }
 
 }  // namespace aq

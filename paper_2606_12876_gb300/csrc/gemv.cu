@@ -1031,25 +1031,34 @@ static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt) {
     return ts + (x_dt == AQ_BF16 ? 3000.0 : 0.0) < units * 400.0 + 8000.0;
 }
 
+// The tensor-memory kernel for n layers that share x; ws0: the first layer's workspace, whose partial-sum
+// room takes the fp16 copy of bf16 activations and the row factors; status: where a device-side failure
+// is recorded.
+static aq_status launch_gemv_ts(const Dims* ds, int n, int m, const void* const* planes, const void* const* books,
+                                const void* const* scales, const void* x, int x_dt, int batch, void* const* y,
+                                int y_dt, void* ws0, void* status, cudaStream_t st) {
+    const void* xh = x;
+    float* fac = nullptr;
+    if (x_dt == AQ_BF16) {
+        fac = (float*)((char*)ws0 + ws_partial_offset(ds[0]));
+        void* dst = (char*)fac + kWsStatusBytes;
+        if (aq_status e = launch_x_to_f16(x, dst, fac, ds[0].in, batch, st); e != AQ_OK) return e;
+        xh = dst;
+    }
+    return launch_ts(ds, n, m, planes, books, scales, xh, fac, batch, y, y_dt, status, st);
+}
+
 aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* books,
                       const void* scales, const void* x, int x_dt, int batch, void* y,
                       int y_dt, void* ws, cudaStream_t st, const void* y_prev) {
     if (d.out == 0 || batch == 0) return AQ_OK;
     if (d.B == 4 && batch == 1)
         return launch_lut4(d, m, planes, books, scales, x, x_dt, y, y_dt, y_prev, st);
-    if (!y_prev && gemv_uses_ts(d, m, batch, x_dt)) {
-        const void* xh = x;
-        float* fac = nullptr;
-        if (x_dt == AQ_BF16) {   // the fp16 copy and the row factors take the partial sums' room
-            fac = (float*)((char*)ws + ws_partial_offset(d));
-            void* dst = (char*)fac + kWsStatusBytes;
-            if (aq_status e = launch_x_to_f16(x, dst, fac, d.in, batch, st); e != AQ_OK) return e;
-            xh = dst;
-        }
-        return launch_ts(d, m, planes, books, scales, xh, fac, batch, y, y_dt, ws, st);
+    if (d.B == 4 || (d.B == 8 && batch > kLutMaxBatch)) {
+        if (!y_prev && gemv_uses_ts(d, m, batch, x_dt))
+            return launch_gemv_ts(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, ws, ws, st);
+        return launch_cw(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, y_prev, st);
     }
-    if (d.B == 4 || (d.B == 8 && batch > kLutMaxBatch))
-        return launch_cw(d, m, planes, books, scales, x, x_dt, batch, y, y_dt, y_prev, st);
     GemvArgs a{planes, books, scales, x, x_dt, batch, y, y_dt,
                (float*)((char*)ws + ws_partial_offset(d)), (unsigned int*)ws};
     if (aq_status e = launch_product(d, m, a, st); e != AQ_OK) return e;
@@ -1062,8 +1071,10 @@ aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* book
 // (status word and partial planes, laid out as for aq_gemv). At batch 1 with 2^8-entry books
 // the n products are one launch of the table-lookup kernel (the items of all layers in one
 // numbering) and the n reductions one launch; otherwise, or when a CTA's items would reach
-// into more than two layers, the layers run as n ordinary calls. Either way each layer's
-// partial sums and their order are those of its own call, so the results are identical.
+// into more than two layers, the layers run as n ordinary calls. In the one-kernel forms of 2..16
+// tokens the layers with the same split of K share a launch (8B block, q/k/v and gate/up in groups: see
+// the figures in gemv_cw.cu). Either way each layer's partial sums and their order are those of its own
+// call, so the results are identical.
 aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* planes,
                             const void* const* books, const void* const* scales, const void* x,
                             int x_dt, int batch, void* const* y, int y_dt, void* const* ws,
@@ -1099,6 +1110,35 @@ aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* pla
                                              : launch_reduce_layers<AQ_F16>(dd, as, n, P, nullptr, sw, st);
         }
         if (e != AQ_ERR_UNSUPPORTED) return e;   // nothing was launched for UNSUPPORTED
+    }
+    if (ds[0].B == 4 ? batch >= 2 : ds[0].B == 8 && batch > kLutMaxBatch) {
+        // The layers that the tensor-memory kernel serves share the copy of x and launches; the others
+        // share launches of gemv_cw.
+        struct {
+            Dims d[kGroupMax];
+            const void *planes[kGroupMax], *books[kGroupMax], *scales[kGroupMax];
+            void *y[kGroupMax], *ws0;
+            int n;
+        } part[2] = {};
+        for (int l = 0; l < n; ++l) {
+            if (ds[l].out == 0) continue;
+            auto& p = part[gemv_uses_ts(ds[l], m, batch, x_dt) ? 1 : 0];
+            if (p.n == 0) p.ws0 = ws[l];
+            p.d[p.n] = ds[l];
+            p.planes[p.n] = planes[l];
+            p.books[p.n] = books[l];
+            p.scales[p.n] = scales[l];
+            p.y[p.n++] = y[l];
+        }
+        if (part[1].n > 0)
+            if (aq_status e = launch_gemv_ts(part[1].d, part[1].n, m, part[1].planes, part[1].books, part[1].scales, x,
+                                             x_dt, batch, part[1].y, y_dt, part[1].ws0, ws[0], st);
+                e != AQ_OK)
+                return e;
+        if (part[0].n > 0)
+            return launch_cw(part[0].d, part[0].n, m, part[0].planes, part[0].books, part[0].scales, x, x_dt, batch,
+                             part[0].y, y_dt, nullptr, st);
+        return AQ_OK;
     }
     for (int l = 0; l < n; ++l)
         if (aq_status e = launch_gemv(ds[l], m, planes[l], books[l], scales[l], x, x_dt, batch, y[l],

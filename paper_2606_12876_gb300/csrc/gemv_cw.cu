@@ -31,6 +31,10 @@
 // its largest |x| in [2^14, 2^15) and rounded to fp16, which is exact for values within 2^29 of
 // the largest, and the slice's sums are scaled back when they are added to the total. bf16 books
 // with fp16 activations: the books are scaled the same way (one power of two for the m books).
+//
+// Measured, 8B block (seven layers; q/k/v and gate/up as groups): 8 tokens, m = 3 86.5 us (the eight-token
+// tables and tf32 kernel before: 145.8), 4-bit codes, 4 tokens, m = 4 92.2 us (fp32 kernel before: 229.7);
+// as seven single launches 91.1 and 96.3. 14336 x 4096, m = 4, 8 tokens: 22.5 us; 4096 x 4096: 9.8 us.
 #include "aq_internal.cuh"
 #include "launch.cuh"
 #include "tc_ptx.cuh"
@@ -42,16 +46,25 @@ constexpr int kCwWarps = 16;
 constexpr int kCwThreads = kCwWarps * 32;
 constexpr int kCwPitch = 36;       // floats per token in a warp's sums (4 of padding: no conflicts)
 
-struct CwArgs {
+// One layer of a launch; a launch holds one layer, or several that share the activations and the split
+// (aq_gemv_group): cluster c of the layer takes row blocks c, c + nclusters, ...
+struct CwLayer {
     const uint8_t* planes;
-    const uint16_t *books, *scales, *x;
+    const uint16_t *books, *scales;
     void* y;
-    const void* y_prev;            // added to the product (refinement), or null
-    int y_dt, scale_dt, m, batch, out, in, ng, rows_pad, RBc, S;
-    int cshift;                    // log2 of the interleaved copies of a codebook
-    int kc, nclusters;             // CTAs per cluster, clusters (row blocks are dealt to them in turn)
-    int static_weights;
+    int out, rows_pad, RBc;
+    int c0, nclusters;             // the layer's clusters of the grid
     size_t plane_bytes;
+};
+struct CwArgs {
+    CwLayer L[4];
+    int nlayers;
+    const uint16_t* x;
+    const void* y_prev;            // added to the product (refinement), or null
+    int y_dt, scale_dt, m, batch, in, ng, S;
+    int cshift;                    // log2 of the interleaved copies of a codebook
+    int kc;                        // CTAs per cluster
+    int static_weights;
 };
 
 // Shared memory: books [m][2^B][2^cshift] x 16 B, codes 16 warps x 32 rows, the warps' sums (two
@@ -175,7 +188,10 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     float* csum = red + 2 * cw_red_floats(NT);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = a.kc > 1 ? (int)cluster_rank() : 0;
-    const int cid = (int)blockIdx.x / a.kc;
+    int cid = (int)blockIdx.x / a.kc, layer = 0;
+    while (layer + 1 < a.nlayers && cid >= a.L[layer + 1].c0) ++layer;
+    const CwLayer& L = a.L[layer];
+    cid -= L.c0;
     const int tb = (int)blockIdx.y * NTOK;               // first token
 
     // this warp's (slice, book) units u0 .. u1-1 of every row block of the cluster; u = s*m + k
@@ -188,7 +204,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     };
     auto next_item = [&](Item& it) {
         if (++it.u == u1) {
-            it = Item{it.rb + a.nclusters, u0, s0, k0};
+            it = Item{it.rb + L.nclusters, u0, s0, k0};
         } else if (++it.k == a.m) {
             it.k = 0;
             ++it.s;
@@ -196,9 +212,9 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     };
     uint4 raw[2];
     auto load_codes = [&](const Item& it) {
-        if (u0 < u1 && it.rb < a.RBc) {
-            const uint8_t* src = a.planes + (size_t)it.k * a.plane_bytes +
-                                 ((size_t)it.s * a.rows_pad + (size_t)it.rb * 32 + lane) * UNIT;
+        if (u0 < u1 && it.rb < L.RBc) {
+            const uint8_t* src = L.planes + (size_t)it.k * L.plane_bytes +
+                                 ((size_t)it.s * L.rows_pad + (size_t)it.rb * 32 + lane) * UNIT;
             raw[0] = ld_stream_v4(src);
             if constexpr (B == 8) raw[1] = ld_stream_v4(src + 16);
         }
@@ -211,18 +227,18 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
             __syncthreads();
             float mx = 0.0f;
             for (int i = tid; i < a.m * NC; i += kCwThreads)
-                mx = fmaxf(mx, max_abs8<BDT>(__ldg((const uint4*)a.books + i)));
+                mx = fmaxf(mx, max_abs8<BDT>(__ldg((const uint4*)L.books + i)));
             atomicMax(&s_bmax, __float_as_uint(mx));     // non-negative floats order as integers
             __syncthreads();
             const int f = f16_exponent(__uint_as_float(s_bmax));
             bfac = pow2f(f);
             const float sc = pow2f(-f);
             for (int i = tid; i < nslot; i += kCwThreads)
-                books_s[i] = scaled_to_f16<BDT>(__ldg((const uint4*)a.books + (i >> a.cshift)), sc);
+                books_s[i] = scaled_to_f16<BDT>(__ldg((const uint4*)L.books + (i >> a.cshift)), sc);
         } else {
 #pragma unroll 4
             for (int i = tid; i < nslot; i += kCwThreads)
-                books_s[i] = __ldg((const uint4*)a.books + (i >> a.cshift));
+                books_s[i] = __ldg((const uint4*)L.books + (i >> a.cshift));
         }
     };
     if (a.static_weights) {   // read-only weights: requested before the preceding kernel has finished
@@ -272,7 +288,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     };
 
     int pass = 0;
-    for (int rb = cid; rb < a.RBc; rb += a.nclusters, ++pass) {
+    for (int rb = cid; rb < L.RBc; rb += L.nclusters, ++pass) {
         float acc[2][NT][4];
         // The warps' sums of a pass, added in warp order. Two buffers: a pass's writes meet the sums
         // that are read two passes earlier, which every thread finished before the last barrier.
@@ -281,7 +297,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
         bool first = true;
         // the row scale of the output this thread finishes, requested before the pass's gathers
         const int my_o = rb * 32 + (tid & 31);
-        const float my_s = tid < 32 * NTOK && my_o < a.out ? bits_to_f32_rt(a.scales[my_o], a.scale_dt) : 0.0f;
+        const float my_s = tid < 32 * NTOK && my_o < L.out ? bits_to_f32_rt(L.scales[my_o], a.scale_dt) : 0.0f;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
@@ -368,14 +384,14 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
                 }
         }
         const int t = tb + (tid >> 5), o = my_o;
-        if (tid >= i0 && tid < i1 && t < a.batch && o < a.out) {
+        if (tid >= i0 && tid < i1 && t < a.batch && o < L.out) {
             float r = v * bfac * my_s;
-            const size_t yi = (size_t)t * a.out + o;
+            const size_t yi = (size_t)t * L.out + o;
             if (a.y_prev)
                 r = (a.y_dt == AQ_F32 ? ((const float*)a.y_prev)[yi]
                                       : bits_to_f32_rt(((const uint16_t*)a.y_prev)[yi], a.y_dt)) + r;
-            if (a.y_dt == AQ_F32) ((float*)a.y)[yi] = r;
-            else ((uint16_t*)a.y)[yi] = a.y_dt == AQ_F16 ? f32_to_bits<AQ_F16>(r) : f32_to_bits<AQ_BF16>(r);
+            if (a.y_dt == AQ_F32) ((float*)L.y)[yi] = r;
+            else ((uint16_t*)L.y)[yi] = a.y_dt == AQ_F16 ? f32_to_bits<AQ_F16>(r) : f32_to_bits<AQ_BF16>(r);
         }
     }
     if (a.kc > 1) cluster_sync();   // no CTA leaves while a peer may still read its sums
@@ -390,11 +406,12 @@ inline int cw_cshift(int B, int m) { return B == 4 || m <= 4 ? 3 : 2; }
 // reduction of a pass, plus what a cluster launch and its barriers cost over a plain one (measured
 // about 2 us for two or four CTAs, 6 for eight: 512 x 4096, m = 4 took 10.8 us in clusters of eight).
 // Clusters of 2, 4 and 8 that are resident at once: 76, 36 and 16 on 152 SMs.
+inline int cw_clusters(int kc, int sms) { return kc == 1 ? sms : kc == 2 ? sms / 2 : kc == 4 ? sms * 9 / 38 : sms * 2 / 19; }
 inline int cw_cluster(const Dims& d, int m, int sms, int* nclusters) {
     int best = 1;
     double best_t = -1.0;
     for (int kc = 1; kc <= 8; kc *= 2) {
-        int nc = kc == 1 ? sms : kc == 2 ? sms / 2 : kc == 4 ? sms * 9 / 38 : sms * 2 / 19;
+        int nc = cw_clusters(kc, sms);
         if (nc > d.RBc) nc = d.RBc;
         if (nc < 1) nc = 1;
         const long long U = (long long)d.S * m;
@@ -413,60 +430,95 @@ inline int cw_cluster(const Dims& d, int m, int sms, int* nclusters) {
 }
 
 template <int B, int BDT, int XDT, int NT, int CHAIN>
-aq_status run_cw(const Dims& d, CwArgs a, cudaStream_t st) {
-    DeviceInfo di;
-    if (aq_status e = device_info(&di); e != AQ_OK) return e;
+aq_status run_cw(CwArgs a, cudaStream_t st) {
     auto kern = gemv_cw_kernel<B, BDT, XDT, NT, CHAIN>;
     a.cshift = cw_cshift(B, a.m);
     const size_t smem = cw_smem_bytes(B, a.m, a.cshift, NT);
     int occ = 0;
     if (aq_status e = prepare(kern, smem, kCwThreads, a.m, &occ); e != AQ_OK) return e;
-    a.kc = cw_cluster(d, a.m, di.sms, &a.nclusters);
-    return launch_pdl_cluster(a.kc, kern, dim3(a.nclusters * a.kc, (a.batch + 8 * NT - 1) / (8 * NT)),
+    const CwLayer& last = a.L[a.nlayers - 1];
+    return launch_pdl_cluster(a.kc, kern, dim3((last.c0 + last.nclusters) * a.kc, (a.batch + 8 * NT - 1) / (8 * NT)),
                               dim3(kCwThreads), smem, st, a);
 }
 
 // 4-bit codes: one token tile per CTA at any batch (two tiles of short chains do not fit the registers).
 template <int B, int BDT, int XDT>
-aq_status run_cw_nt(const Dims& d, const CwArgs& a, cudaStream_t st) {
-    if constexpr (B == 4) return run_cw<B, BDT, XDT, 1, 8>(d, a, st);
-    else if (a.batch <= 4) return run_cw<B, BDT, XDT, 1, 8>(d, a, st);
-    else if (a.batch <= 8) return run_cw<B, BDT, XDT, 1, 0>(d, a, st);
-    else return run_cw<B, BDT, XDT, 2, 0>(d, a, st);
+aq_status run_cw_nt(const CwArgs& a, cudaStream_t st) {
+    if constexpr (B == 4) return run_cw<B, BDT, XDT, 1, 8>(a, st);
+    else if (a.batch <= 4) return run_cw<B, BDT, XDT, 1, 8>(a, st);
+    else if (a.batch <= 8) return run_cw<B, BDT, XDT, 1, 0>(a, st);
+    else return run_cw<B, BDT, XDT, 2, 0>(a, st);
 }
 
 template <int B>
-aq_status run_cw_types(const Dims& d, const CwArgs& a, int x_dt, cudaStream_t st) {
-    if (d.book_dt == AQ_BF16)
-        return x_dt == AQ_BF16 ? run_cw_nt<B, AQ_BF16, AQ_BF16>(d, a, st) : run_cw_nt<B, AQ_BF16, AQ_F16>(d, a, st);
-    return x_dt == AQ_BF16 ? run_cw_nt<B, AQ_F16, AQ_BF16>(d, a, st) : run_cw_nt<B, AQ_F16, AQ_F16>(d, a, st);
+aq_status run_cw_types(const CwArgs& a, int book_dt, int x_dt, cudaStream_t st) {
+    if (book_dt == AQ_BF16)
+        return x_dt == AQ_BF16 ? run_cw_nt<B, AQ_BF16, AQ_BF16>(a, st) : run_cw_nt<B, AQ_BF16, AQ_F16>(a, st);
+    return x_dt == AQ_BF16 ? run_cw_nt<B, AQ_F16, AQ_BF16>(a, st) : run_cw_nt<B, AQ_F16, AQ_F16>(a, st);
 }
 
 }  // namespace
 
-aq_status launch_cw(const Dims& d, int m, const void* planes, const void* books, const void* scales,
-                    const void* x, int x_dt, int batch, void* y, int y_dt, const void* y_prev,
-                    cudaStream_t st) {
-    CwArgs a = {};
-    a.planes = (const uint8_t*)planes;
-    a.books = (const uint16_t*)books;
-    a.scales = (const uint16_t*)scales;
-    a.x = (const uint16_t*)x;
-    a.y = y;
-    a.y_prev = y_prev;
-    a.y_dt = y_dt;
-    a.scale_dt = d.scale_dt;
-    a.m = m;
-    a.batch = batch;
-    a.out = d.out;
-    a.in = d.in;
-    a.ng = d.ng;
-    a.rows_pad = d.rows_pad;
-    a.RBc = d.RBc;
-    a.S = d.S;
-    a.static_weights = (d.flags & AQ_LAYOUT_STATIC_WEIGHTS) ? 1 : 0;
-    a.plane_bytes = d.plane_bytes;
-    return d.B == 4 ? run_cw_types<4>(d, a, x_dt, st) : run_cw_types<8>(d, a, x_dt, st);
+aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, const void* const* books,
+                    const void* const* scales, const void* x, int x_dt, int batch, void* const* y, int y_dt,
+                    const void* y_prev, cudaStream_t st) {
+    DeviceInfo di;
+    if (aq_status e = device_info(&di); e != AQ_OK) return e;
+    const Dims& d = ds[0];
+    int kcs[4], own[4];
+    for (int l = 0; l < n; ++l) kcs[l] = cw_cluster(ds[l], m, di.sms, &own[l]);
+    bool done[4] = {};
+    for (int f = 0; f < n; ++f) {
+        if (done[f]) continue;
+        // the layers with this one's cluster size: their sums are those of their own calls
+        CwArgs a = {};
+        a.kc = kcs[f];
+        int rbs = 0, set[4];
+        for (int l = f; l < n; ++l)
+            if (!done[l] && kcs[l] == a.kc) {
+                done[l] = true;
+                rbs += ds[l].RBc;
+                set[a.nlayers++] = l;
+            }
+        // the fewest passes that the resident clusters allow over all layers
+        const int cap = cw_clusters(a.kc, di.sms);
+        int passes = (rbs + cap - 1) / cap;
+        auto need = [&](int p) {
+            int c = 0;
+            for (int i = 0; i < a.nlayers; ++i) c += (ds[set[i]].RBc + p - 1) / p;
+            return c;
+        };
+        while (a.nlayers > 1 && need(passes) > cap) ++passes;
+        a.static_weights = 1;
+        for (int i = 0, c0 = 0; i < a.nlayers; ++i) {
+            const int l = set[i];
+            CwLayer& L = a.L[i];
+            L.planes = (const uint8_t*)planes[l];
+            L.books = (const uint16_t*)books[l];
+            L.scales = (const uint16_t*)scales[l];
+            L.y = y[l];
+            L.out = ds[l].out;
+            L.rows_pad = ds[l].rows_pad;
+            L.RBc = ds[l].RBc;
+            L.plane_bytes = ds[l].plane_bytes;
+            L.c0 = c0;
+            L.nclusters = a.nlayers > 1 ? (ds[l].RBc + passes - 1) / passes : own[l];
+            c0 += L.nclusters;
+            if (!(ds[l].flags & AQ_LAYOUT_STATIC_WEIGHTS)) a.static_weights = 0;
+        }
+        a.x = (const uint16_t*)x;
+        a.y_prev = y_prev;
+        a.y_dt = y_dt;
+        a.scale_dt = d.scale_dt;
+        a.m = m;
+        a.batch = batch;
+        a.in = d.in;
+        a.ng = d.ng;
+        a.S = d.S;
+        const aq_status e = d.B == 4 ? run_cw_types<4>(a, d.book_dt, x_dt, st) : run_cw_types<8>(a, d.book_dt, x_dt, st);
+        if (e != AQ_OK) return e;
+    }
+    return AQ_OK;
 }
 
 }  // namespace aq
