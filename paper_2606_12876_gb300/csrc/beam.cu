@@ -183,7 +183,7 @@ __device__ __forceinline__ bool before(float a, int ia, float b, int ib) {
 // 8 x 8 quadratic form); instead
 //  1. every candidate gets an estimate of its score from the expanded form
 //     A_r + C_t[c] . G_r + lambda s^2 (C_t[c]^T S_gg C_t[c]),  G_r = -2 lambda s (S_gg u_r + h),
-//     u_r = w_g - s P_r: six operations, G_r in registers, the last term tabled per CTA. Each lane
+//     u_r = w_g - s P_r: about six operations, G_r in registers, the last term tabled per CTA. Each lane
 //     keeps its smallest estimate per state and per codeword;
 //  2. the keep-th smallest of the 32 lanes' smallest estimates is at least the keep-th smallest
 //     estimate; with both forms' rounding errors below eps, every candidate among the K first has an
@@ -219,33 +219,30 @@ template <int RC, bool FIRST>
 __device__ __forceinline__ void beam_estimates(const float4* lo, const float4* hi, const float* Q, float F,
                                                const float* G, const float* A, int lane, float* mr,
                                                float* mc) {
-    float2 g2[RC][4];
-    float a[RC];
+    // two states per packed fp32 operation, the codeword's elements doubled
+    float2 g2[RC / 2][8], a2[RC / 2];
 #pragma unroll
-    for (int r = 0; r < RC; ++r) {
-        const float4 x = *(const float4*)(G + r * 8), y = *(const float4*)(G + r * 8 + 4);
-        g2[r][0] = make_float2(x.x, x.y);
-        g2[r][1] = make_float2(x.z, x.w);
-        g2[r][2] = make_float2(y.x, y.y);
-        g2[r][3] = make_float2(y.z, y.w);
-        a[r] = A[r];
-        mr[r] = FLT_MAX;
+    for (int r = 0; r < RC; r += 2) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) g2[r / 2][e] = make_float2(G[r * 8 + e], G[r * 8 + 8 + e]);
+        a2[r / 2] = make_float2(A[r], A[r + 1]);
+        mr[r] = mr[r + 1] = FLT_MAX;
     }
 #pragma unroll 2
     for (int i = 0; i < 8; ++i) {
         const int c = lane + 32 * i;
         const float4 x = lo[c], y = hi[c];
+        const float cv[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
         const float fq = F * Q[c];
         float m = FIRST ? FLT_MAX : mc[c];
 #pragma unroll
-        for (int r = 0; r < RC; ++r) {
-            float2 t = ffma2(make_float2(x.x, x.y), g2[r][0], make_float2(a[r] + fq, 0.0f));
-            t = ffma2(make_float2(x.z, x.w), g2[r][1], t);
-            t = ffma2(make_float2(y.x, y.y), g2[r][2], t);
-            t = ffma2(make_float2(y.z, y.w), g2[r][3], t);
-            const float v = t.x + t.y;
-            mr[r] = fminf(mr[r], v);
-            m = fminf(m, v);
+        for (int r = 0; r < RC; r += 2) {
+            float2 t = add2(a2[r / 2], make_float2(fq, fq));
+#pragma unroll
+            for (int e = 0; e < 8; ++e) t = ffma2(make_float2(cv[e], cv[e]), g2[r / 2][e], t);
+            mr[r] = fminf(mr[r], t.x);
+            mr[r + 1] = fminf(mr[r + 1], t.y);
+            m = fminf(fminf(m, t.x), t.y);
         }
         mc[c] = m;
     }
@@ -388,7 +385,8 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
             };
             // magnitude bound T_r, and the expanded form's G_r and A_r: four lanes per state
             float tot = 0.0f;
-            for (int r = lane >> 2; r < kBeamMaxK; r += 8) {
+            // (eight states, or all sixteen places: the estimates read no further)
+            for (int r = lane >> 2; r < (nstates > 8 ? kBeamMaxK : 8); r += 8) {
                 float ga[2], au = 0.0f, tr = 0.0f;
                 const int rr = r < nstates ? r : 0, e0 = (lane & 3) * 2;
                 float u[8], D[8];
@@ -446,8 +444,8 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
                     const float F = lt * s * s, slack = 3.0517578125e-5f * tot;   // 2 eps
                     const float* Qt = Q + (size_t)t * nb;
                     uint32_t rmask, cmask;
-                    if (nstates == 1)
-                        beam_reach<1, 1>(lot, hit, Qt, F, bw.G[0], bw.A, bw.lscore, lane, keep, slack, &rmask, &cmask);
+                    if (nstates <= 2)
+                        beam_reach<2, 1>(lot, hit, Qt, F, bw.G[0], bw.A, bw.lscore, lane, keep, slack, &rmask, &cmask);
                     else if (nstates <= 4)
                         beam_reach<4, 1>(lot, hit, Qt, F, bw.G[0], bw.A, bw.lscore, lane, keep, slack, &rmask, &cmask);
                     else if (nstates <= 8)
