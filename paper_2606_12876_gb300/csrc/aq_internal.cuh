@@ -40,8 +40,8 @@ constexpr size_t kWsStatusBytes = 256;
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline size_t ws_partial_offset(const Dims&) { return kWsStatusBytes; }
 
-// The table-lookup GEMV (2^8-entry books) serves one and two tokens, and writes one partial plane
-// per (slice, book, token); the 2^16-entry-book kernels write one per (slice, token); the
+// The table-lookup GEMV (2^8-entry books) serves one token (but for the smallest layers) and two, and
+// writes one partial plane per (slice, book, token); the 2^16-entry-book kernels write one per (slice, token); the
 // remaining GEMVs (gemv_cw, gemv_lut4) need no partial planes.
 constexpr int kLutMaxBatch = 2;
 
@@ -97,7 +97,7 @@ aq_status launch_decode(const Dims& d, int m, const void* planes, const void* bo
 aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* books,
                       const void* scales, const void* x, int x_dt, int batch, void* y,
                       int y_dt, void* ws, cudaStream_t st, const void* y_prev = nullptr);
-// The same for 2..16 tokens with 4- or 8-bit codes in one kernel (gemv_cw.cu), for n (<= 4) layers that
+// The same for up to 16 tokens with 4- or 8-bit codes in one kernel (gemv_cw.cu), for n (<= 4) layers that
 // share x, the code width, the types and m (n = 1: an ordinary call).
 aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, const void* const* books,
                     const void* const* scales, const void* x, int x_dt, int batch, void* const* y, int y_dt,

@@ -1015,6 +1015,17 @@ static aq_status launch_reduce(const Dims& d, int P, const GemvArgs& a, const vo
                                      (d.flags & AQ_LAYOUT_STATIC_WEIGHTS) ? 1 : 0, st);
 }
 
+// Whether a call runs in one kernel (gemv_cw, or gemm_ts for 9..16 tokens): 4-bit codes at two and more
+// tokens, 8-bit codes at three and more, and at one token on small layers, with at most half a unit (slice,
+// book) per warp of a CTA and 64 row blocks. There the table kernel and its reduction take 4.0 us and two
+// launches, this one 3.75 us and one launch (1024 x 1024, m = 2: an eager call 9.3 against 12.9 us); with
+// 128 row blocks it is 4.3 against 3.95 us.
+static bool gemv_uses_cw(const Dims& d, int m, int batch) {
+    if (d.B == 4) return batch >= 2;
+    if (d.B != 8) return false;
+    return batch > kLutMaxBatch || (batch == 1 && d.S * m <= 8 && d.RBc <= 64);
+}
+
 // Whether 9..16 tokens run the tensor-memory kernel (gemm_ts.cu): where its estimated time is below
 // that of gemv_cw, which at two token tiles is bound by the tensor pipe's legacy multiplies (64 a unit
 // of 32 rows, slice and book at 4 clocks; per SM, with its fixed cost). 14336 x 4096, m = 4, 16
@@ -1054,7 +1065,7 @@ aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* book
     if (d.out == 0 || batch == 0) return AQ_OK;
     if (d.B == 4 && batch == 1)
         return launch_lut4(d, m, planes, books, scales, x, x_dt, y, y_dt, y_prev, st);
-    if (d.B == 4 || (d.B == 8 && batch > kLutMaxBatch)) {
+    if (gemv_uses_cw(d, m, batch)) {
         if (!y_prev && gemv_uses_ts(d, m, batch, x_dt))
             return launch_gemv_ts(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, ws, ws, st);
         return launch_cw(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, y_prev, st);
@@ -1084,7 +1095,7 @@ aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* pla
     for (int l = 0; l < n; ++l) any_rows |= ds[l].out > 0;
     if (!any_rows) return AQ_OK;
     bool fused = n >= 2 && batch == 1 && ds[0].B == 8;
-    for (int l = 0; l < n && fused; ++l) fused = ds[l].out > 0;
+    for (int l = 0; l < n && fused; ++l) fused = ds[l].out > 0 && !gemv_uses_cw(ds[l], m, 1);
     if (fused) {
         Dims dd[kGroupMax];
         GemvArgs as[kGroupMax];
@@ -1111,7 +1122,9 @@ aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* pla
         }
         if (e != AQ_ERR_UNSUPPORTED) return e;   // nothing was launched for UNSUPPORTED
     }
-    if (ds[0].B == 4 ? batch >= 2 : ds[0].B == 8 && batch > kLutMaxBatch) {
+    bool cw = true;
+    for (int l = 0; l < n; ++l) cw = cw && gemv_uses_cw(ds[l], m, batch);
+    if (cw) {
         // The layers that the tensor-memory kernel serves share the copy of x and launches; the others
         // share launches of gemv_cw.
         struct {

@@ -173,7 +173,8 @@ struct RowCodes {
 // CHAIN: multiplies accumulated by the tensor pipe before an fp32 add takes them over (0: all of a unit
 // and the next ones). The pipe truncates as it accumulates: over the 64 multiplies of a row and four books
 // that costs a decimal of fp32 (relative error of an fp32 y 1.2e-6; chains of eight 2e-7; fp32 sums 1.2e-7).
-// Chains of eight (3 to 10 % more time) stand where calls had fp32 sums: up to four tokens, 4-bit codes.
+// Chains of eight (3 to 10 % more time) stand where calls had fp32 sums: up to four tokens, 4-bit codes;
+// single multiplies at one token (1.1 to 1.2e-7 on the small layers that come here, as the tables).
 template <int B, int BDT, int XDT, int NT, int CHAIN>
 __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_constant__ CwArgs a) {
     constexpr int UNIT = unit_bytes(B), NC = 1 << B, NTOK = 8 * NT;
@@ -340,6 +341,13 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
             __syncwarp();                                // the buffer may be refilled
             const uint32_t base = books_u + (uint32_t)k * (NC * mul);
             float part[2][NT][4] = {};                   // (CHAIN > 0) the current chains
+            auto take = [&](int mt, int nt) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    acc[mt][nt][e] += part[mt][nt][e];
+                    part[mt][nt][e] = 0.0f;
+                }
+            };
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 uint4 w[4];
@@ -351,13 +359,9 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
                     for (int nt = 0; nt < NT; ++nt) {
                         float(&d)[4] = CHAIN ? part[mt][nt] : acc[mt][nt];
                         mma16<MDT>(d, w[2 * mt].x, w[2 * mt + 1].x, w[2 * mt].y, w[2 * mt + 1].y, bf[nt][j].x, bf[nt][j].y);
+                        if (CHAIN == 1) take(mt, nt);
                         mma16<MDT>(d, w[2 * mt].z, w[2 * mt + 1].z, w[2 * mt].w, w[2 * mt + 1].w, bf[nt][j].z, bf[nt][j].w);
-                        if (CHAIN == 8 && (j & 3) == 3)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                acc[mt][nt][e] += part[mt][nt][e];
-                                part[mt][nt][e] = 0.0f;
-                            }
+                        if (CHAIN == 1 || (CHAIN == 8 && (j & 3) == 3)) take(mt, nt);
                     }
             }
         }
@@ -445,6 +449,7 @@ aq_status run_cw(CwArgs a, cudaStream_t st) {
 template <int B, int BDT, int XDT>
 aq_status run_cw_nt(const CwArgs& a, cudaStream_t st) {
     if constexpr (B == 4) return run_cw<B, BDT, XDT, 1, 8>(a, st);
+    else if (a.batch == 1) return run_cw<B, BDT, XDT, 1, 1>(a, st);
     else if (a.batch <= 4) return run_cw<B, BDT, XDT, 1, 8>(a, st);
     else if (a.batch <= 8) return run_cw<B, BDT, XDT, 1, 0>(a, st);
     else return run_cw<B, BDT, XDT, 2, 0>(a, st);
