@@ -9,7 +9,7 @@
 // tile's height is chosen to spread the rows over the SMs.
 //
 // Bound at up to about 128 tokens: the codeword gathers from shared memory (16 bytes per code).
-// The codebooks are staged in 2^cshift interleaved copies (eight: no bank conflicts, 8 codes per
+// The codebooks are staged in eight interleaved copies (no bank conflicts, 8 codes per
 // clock and SM; a single copy gives about 3).
 //
 // The decoders add the m codewords of a group in fp32, in book order, and round once to fp16 (the
@@ -24,8 +24,8 @@
 // shared memory (free once its MMAs completed) and each finishes a share of the tokens, adding the
 // CTAs' sums in rank order.
 // Measured (the call, with the copy of bf16 activations), against the pair kernel: 4096 x 14336, m = 3,
-// 100 tokens 30.3 / 211 us; 14336 x 4096, m = 4, 100 tokens 31.8 / 79.4 us, 512 tokens 71.9 / 81.8 us;
-// 16 tokens, m = 4: 29 us against gemv_cw's 47.7.
+// 100 tokens 27.5 / 211 us; 14336 x 4096, m = 4, 100 tokens 31.7 / 79.4 us, 512 tokens 73.1 / 81.8 us;
+// 16 tokens, m = 4: 27.7 us against gemv_cw's 47.7.
 // Roles: warps 0-15 decoders (warp w: quarter w mod 4, set w / 4; the warps of absent quarters idle)
 // and epilogue; one warp for TMA (and L2 prefetch of the codes), one for MMA issue and the
 // tensor-memory allocation: with qr = 4 two more warps (96 registers a thread), else two of the idle
@@ -47,6 +47,7 @@ namespace {
 constexpr int kTsDec = 16;          // decoder warps
 constexpr int kTsMaxM = 4;          // prefixes compiled for the sums form
 constexpr int kTsRing = 8;          // weight stages in tensor memory (32 columns each, from column 256)
+constexpr int kTsCopies = 3;        // log2 of the interleaved copies of a codebook
 constexpr int kTsBars = 2 * kTsRing + 1;
 
 // One layer of a launch; a launch holds one layer, or several that share the activations and the split
@@ -64,7 +65,7 @@ struct TsArgs {
     const float* xfac;              // per-token factor of the activations, or null
     unsigned int* status;
     int y_dt, scale_dt, tokens, in, ng, S;
-    int cshift, qr, kc, n, nsb, spc;   // n: tokens of a tile (multiple of 16); nsb: activation stages;
+    int qr, kc, n, nsb, spc;   // n: tokens of a tile (multiple of 16); nsb: activation stages;
     int books_off, bar_off;            // spc: slices per CTA; shared-memory offsets
     int static_weights;
 };
@@ -97,6 +98,70 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         if (tid == 0) record_status(a.status, AQ_ERR_ALIGNMENT);
         return;
     }
+    // Everything that the weights give, requested before anything is waited for: a CTA's start is one
+    // chain of latencies (codebooks, their largest entry, their copies, the first codes), and a call has the
+    // SM to itself, so none of it hides behind other work.
+    const int q = warp & 3, ws = warp >> 2;             // decoders: row quarter, slice of a round
+    const bool decoder = warp < kTsDec && q < a.qr;
+    const int row = row0 + q * 32 + lane;
+    const bool row_in = row < L.rows_pad;
+    // A row's codes of a slice, in two steps to group order (position p holds group (p + row) mod
+    // 32): the loads bring the 8-byte pieces rotated by whole pieces (B = 8), unrotate() does the
+    // rest of the rotation, a word and up to three bytes.
+    const int rr8 = (row >> 3) & 3;
+    auto load_raw = [&](int s, int k, uint32_t (&raw)[NW]) {
+#pragma unroll
+        for (int i = 0; i < NW; ++i) raw[i] = 0u;
+        if (row_in) {
+            const uint8_t* src = L.planes + (size_t)k * L.plane_bytes + ((size_t)s * L.rows_pad + row) * UNIT;
+            if constexpr (B == 8) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint2 v = __ldg((const uint2*)src + ((i - rr8) & 3));
+                    raw[2 * i] = v.x;
+                    raw[2 * i + 1] = v.y;
+                }
+            } else {
+                const uint4 v = ld_stream_v4(src);
+                raw[0] = v.x;
+                raw[1] = v.y;
+                raw[2] = v.z;
+                raw[3] = v.w;
+            }
+        }
+    };
+    uint32_t raw[MB][NW];
+    auto load_slice = [&](int s) {
+#pragma unroll
+        for (int k = 0; k < MB; ++k) load_raw(s, k, raw[k]);
+    };
+    // the codes of a round's slices, HBM to L2
+    const int rows_here = max(0, min(32 * a.qr, L.rows_pad - row0));
+    auto prefetch_round = [&](int r) {
+        if (rows_here > 0)
+            for (int w = 0; w < 4 && 4 * r + w < nsl; ++w)
+                for (int k = 0; k < m; ++k)
+                    prefetch_l2(L.planes + (size_t)k * L.plane_bytes +
+                                    ((size_t)(sl0 + 4 * r + w) * L.rows_pad + row0) * UNIT,
+                                (uint32_t)(rows_here * UNIT));
+    };
+    constexpr int kPer = (MB * NC + kTsThreads - 1) / kTsThreads;
+    uint4 bk[kPer];                                     // this thread's codewords
+    uint16_t sbits = 0;                                 // the scale of row row0 + tid
+    auto fetch = [&]() {
+#pragma unroll
+        for (int l = 0; l < kPer; ++l) {
+            const int i = tid + l * kTsThreads;
+            bk[l] = i < m * NC ? __ldg((const uint4*)L.books + i) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        if (warp == kTmaWarp && elect_one()) {
+            prefetch_round(0);
+            prefetch_round(1);
+        }
+        if (kAhead && decoder && ws < nsl) load_slice(sl0 + ws);
+        if (tid < 32 * a.qr && row0 + tid < L.out) sbits = L.scales[row0 + tid];
+    };
+    if (a.static_weights) fetch();   // read-only weights: before the preceding kernel has finished
     if (tid == 0) {
         for (int i = 0; i < kTsRing; ++i) {
             mbar_init(&full[i], a.qr + 1);
@@ -112,68 +177,42 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     __syncthreads();
-    // Books staged times 2^-f (fp16 range, operand_scale.cuh): each thread loads its codewords once
-    // and writes their copies, starting at copy `lane` so that eight lanes meet no bank twice.
-    float bfac = 1.0f;                                  // 2^f
-    auto stage_books = [&]() {
-        constexpr int kPer = (MB * NC + kTsThreads - 1) / kTsThreads;
-        uint4 c[kPer];
-#pragma unroll
-        for (int l = 0; l < kPer; ++l) {
-            const int i = tid + l * kTsThreads;
-            c[l] = i < m * NC ? __ldg((const uint4*)L.books + i) : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int l = 0; l < kPer; ++l) {
-            const int i = tid + l * kTsThreads;
-            const unsigned int mx = codeword_max_bits<BDT>(c[l]);
-            if constexpr (B == 8) {                     // the 32 codewords of a warp are of one book
-                const unsigned int wm = __reduce_max_sync(0xffffffffu, mx);
-                if (lane == 0 && i < m * NC) atomicMax(&s_wmax[i >> B], wm);
-            } else if (i < m * NC) {
-                atomicMax(&s_wmax[i >> B], mx);
-            }
-        }
-        __syncthreads();
-        const int f = book_exponent<BDT>(s_wmax, MB), nc = 1 << a.cshift;
-        bfac = pow2f(f);
-#pragma unroll
-        for (int l = 0; l < kPer; ++l) {
-            const int i = tid + l * kTsThreads;
-            const uint4 v = f ? scale_codeword<BDT>(c[l], pow2f(-f)) : c[l];
-            if (i < m * NC)
-                for (int q = 0; q < nc; ++q) books_s[(i << a.cshift) + ((q + lane) & (nc - 1))] = v;
-        }
-    };
-    // the codes of a round's slices, HBM to L2
-    const int rows_here = max(0, min(32 * a.qr, L.rows_pad - row0));
-    auto prefetch_round = [&](int r) {
-        if (rows_here > 0)
-            for (int w = 0; w < 4 && 4 * r + w < nsl; ++w)
-                for (int k = 0; k < m; ++k)
-                    prefetch_l2(L.planes + (size_t)k * L.plane_bytes +
-                                    ((size_t)(sl0 + 4 * r + w) * L.rows_pad + row0) * UNIT,
-                                (uint32_t)(rows_here * UNIT));
-    };
-    if (a.static_weights) {   // read-only weights: requested before the preceding kernel has finished
-        if (warp == kTmaWarp && elect_one()) {
-            prefetch_round(0);
-            prefetch_round(1);
-        }
-        stage_books();
-    }
-    pdl_wait();
-    pdl_launch_dependents();
     if (!a.static_weights) {
-        if (warp == kTmaWarp && elect_one()) {
-            prefetch_round(0);
-            prefetch_round(1);
-        }
-        stage_books();
+        pdl_wait();
+        pdl_launch_dependents();
+        fetch();
     }
-    for (int i = tid; i < 32 * a.qr; i += kTsThreads)
-        scale_s[i] = row0 + i < L.out ? bits_to_f32_rt(L.scales[row0 + i], a.scale_dt) * bfac : 0.0f;
-    for (int i = tid; i < a.n; i += kTsThreads) xf_s[i] = a.xfac && t0 + i < a.tokens ? a.xfac[t0 + i] : 1.0f;
+    // Books staged times 2^-f (fp16 range, operand_scale.cuh): each thread writes the eight copies of its
+    // codewords, starting at copy `lane` so that eight lanes meet no bank group twice.
+#pragma unroll
+    for (int l = 0; l < kPer; ++l) {
+        const int i = tid + l * kTsThreads;
+        const unsigned int mx = codeword_max_bits<BDT>(bk[l]);
+        if constexpr (B == 8) {                         // the 32 codewords of a warp are of one book
+            const unsigned int wm = __reduce_max_sync(0xffffffffu, mx);
+            if (lane == 0 && i < m * NC) atomicMax(&s_wmax[i >> B], wm);
+        } else if (i < m * NC) {
+            atomicMax(&s_wmax[i >> B], mx);
+        }
+    }
+    __syncthreads();
+    const int f = book_exponent<BDT>(s_wmax, MB);
+    const float bfac = pow2f(f);
+#pragma unroll
+    for (int l = 0; l < kPer; ++l) {
+        const int i = tid + l * kTsThreads;
+        const uint4 v = f ? scale_codeword<BDT>(bk[l], pow2f(-f)) : bk[l];
+        if (i < m * NC)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) books_s[i * 8 + ((c + lane) & 7)] = v;
+    }
+    if (tid < 128) scale_s[tid] = bits_to_f32_rt(sbits, a.scale_dt) * bfac;
+    if (a.static_weights) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
+    // the token factors of the preceding copy, for the epilogue
+    const float xf_r = a.xfac && tid < a.n && t0 + tid < a.tokens ? a.xfac[t0 + tid] : 1.0f;
     tc_fence_before();
     __syncthreads();          // books staged, barriers initialised, tensor memory allocated
     tc_fence_after();
@@ -238,39 +277,11 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             tc_fence_before();
         }
         __syncwarp();
-    } else if ((warp & 3) < a.qr) {
+    } else if (decoder) {
         // ---------------- decoders
-        const int q = warp & 3, ws = warp >> 2;
-        const int row = row0 + q * 32 + lane;
-        const bool row_in = row < L.rows_pad;
-        const uint32_t mul = 16u << a.cshift;
-        const uint32_t books_u = smem_u32(books_s) + ((uint32_t)(lane & ((1 << a.cshift) - 1)) << 4);
+        constexpr uint32_t mul = 16u << kTsCopies;
+        const uint32_t books_u = smem_u32(books_s) + ((uint32_t)(lane & 7) << 4);
         const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + 256;
-        // A row's codes of a slice, in two steps to group order (position p holds group (p + row) mod
-        // 32): the loads bring the 8-byte pieces rotated by whole pieces (B = 8), unrotate() does the
-        // rest of the rotation, a word and up to three bytes.
-        const int rr8 = (row >> 3) & 3;
-        auto load_raw = [&](int s, int k, uint32_t (&raw)[NW]) {
-#pragma unroll
-            for (int i = 0; i < NW; ++i) raw[i] = 0u;
-            if (row_in) {
-                const uint8_t* src = L.planes + (size_t)k * L.plane_bytes + ((size_t)s * L.rows_pad + row) * UNIT;
-                if constexpr (B == 8) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const uint2 v = __ldg((const uint2*)src + ((i - rr8) & 3));
-                        raw[2 * i] = v.x;
-                        raw[2 * i + 1] = v.y;
-                    }
-                } else {
-                    const uint4 v = ld_stream_v4(src);
-                    raw[0] = v.x;
-                    raw[1] = v.y;
-                    raw[2] = v.z;
-                    raw[3] = v.w;
-                }
-            }
-        };
         auto unrotate = [&](const uint32_t (&raw)[NW], uint32_t (&u)[NW]) {
             if constexpr (B == 8) {
                 const bool odd = (row >> 2) & 1;
@@ -321,12 +332,6 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         int base = 0;                                   // weight stages of the earlier rounds
         // The next slice's codes are requested before the last stage of a slice (when most of the
         // current ones are used up), so their way from L2 (about 2000 clocks) is not waited for.
-        uint32_t raw[MB][NW];
-        auto load_slice = [&](int s) {
-#pragma unroll
-            for (int k = 0; k < MB; ++k) load_raw(s, k, raw[k]);
-        };
-        if (kAhead && ws < nsl) load_slice(sl0 + ws);
         for (int r = 0; r < nrounds; ++r) {
             const int ns = min(4, nsl - 4 * r);
             if (ws < ns) {
@@ -374,8 +379,8 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     tc_fence_after();
     const int R = 32 * a.qr, P = R + 4;
     float* cs = (float*)smem;
-    if (warp < kTsDec && (warp & 3) < a.qr) {
-        const int q = warp & 3, ws = warp >> 2;
+    if (tid < a.n) xf_s[tid] = xf_r;
+    if (decoder) {
         for (int c = ws * 16; c < a.n; c += 64) {
             float v[16];
             if (nsl > 0) tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + c, v);
@@ -396,64 +401,52 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     const int ntok = min(a.n, a.tokens - t0), share = (ntok + a.kc - 1) / a.kc;
     const int ta = rank * share, tb = min(ntok, ta + share);
     const bool vec = (L.out & 7) == 0;
-    // a thread finishes eight rows (always the same ones) of every nt-th token
-    const int R8 = R / 8, nt = kTsThreads / R8, rr = tid % R8 * 8, o = row0 + rr;
-    float sc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) sc[e] = scale_s[rr + e];
-    for (int tl = ta + tid / R8; tl < tb && tid < nt * R8 && o < L.out; tl += nt) {
-        const int t = t0 + tl;
-        float v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = 0.0f;
+    // A thread finishes four rows (always the same ones) of every nt-th token: 16 bytes of each CTA's sums,
+    // contiguous over the lanes (eight rows, 32 bytes apart, took 5400 clocks for 28 tokens of four CTAs).
+    const int R4 = 8 * a.qr, nt = kTsThreads / R4, rr = tid % R4 * 4, o = row0 + rr;
+    const float4 sc = *(const float4*)(scale_s + rr);
+    void* const y = L.y;
+    const int out = L.out;
+    for (int tl = ta + tid / R4; tl < tb && tid < nt * R4 && o < out; tl += nt) {
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         const uint32_t addr = smem_u32(cs + tl * P + rr);
         for (int r4 = 0; r4 < a.kc; r4 += 4) {         // the CTAs' sums, in rank order; four loads in flight
-            float p[4][8];
+            float4 p[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int r = r4 + i;
+                p[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 if (r == rank) {
-                    const float4 p0 = *(const float4*)(cs + tl * P + rr), p1 = *(const float4*)(cs + tl * P + rr + 4);
-                    p[i][0] = p0.x; p[i][1] = p0.y; p[i][2] = p0.z; p[i][3] = p0.w;
-                    p[i][4] = p1.x; p[i][5] = p1.y; p[i][6] = p1.z; p[i][7] = p1.w;
+                    p[i] = *(const float4*)(cs + tl * P + rr);
                 } else if (r < a.kc) {
-                    const uint32_t src = map_to_rank(addr, (uint32_t)r);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-                        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                                     : "=f"(p[i][4 * h]), "=f"(p[i][4 * h + 1]), "=f"(p[i][4 * h + 2]), "=f"(p[i][4 * h + 3])
-                                     : "r"(src + h * 16) : "memory");
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) p[i][e] = 0.0f;
+                    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                 : "=f"(p[i].x), "=f"(p[i].y), "=f"(p[i].z), "=f"(p[i].w)
+                                 : "r"(map_to_rank(addr, (uint32_t)r)) : "memory");
                 }
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] += p[i][e];
+            for (int i = 0; i < 4; ++i) {
+                v.x += p[i].x;
+                v.y += p[i].y;
+                v.z += p[i].z;
+                v.w += p[i].w;
+            }
         }
         const float xf = xf_s[tl];
-        const size_t yi = (size_t)t * L.out + o;
-        const int nv = min(8, L.out - o);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = v[e] * xf * sc[e];
+        const size_t yi = (size_t)(t0 + tl) * out + o;
+        const float w[4] = {v.x * xf * sc.x, v.y * xf * sc.y, v.z * xf * sc.z, v.w * xf * sc.w};
         if (vec && a.y_dt == AQ_F32) {
-            *(float4*)((float*)L.y + yi) = make_float4(v[0], v[1], v[2], v[3]);
-            *(float4*)((float*)L.y + yi + 4) = make_float4(v[4], v[5], v[6], v[7]);
+            *(float4*)((float*)y + yi) = make_float4(w[0], w[1], w[2], w[3]);
         } else if (vec) {
-            *(uint4*)((uint16_t*)L.y + yi) =
-                a.y_dt == AQ_F16
-                    ? make_uint4(round_pack2<AQ_F16>(v[0], v[1]), round_pack2<AQ_F16>(v[2], v[3]),
-                                 round_pack2<AQ_F16>(v[4], v[5]), round_pack2<AQ_F16>(v[6], v[7]))
-                    : make_uint4(round_pack2<AQ_BF16>(v[0], v[1]), round_pack2<AQ_BF16>(v[2], v[3]),
-                                 round_pack2<AQ_BF16>(v[4], v[5]), round_pack2<AQ_BF16>(v[6], v[7]));
+            *(uint2*)((uint16_t*)y + yi) =
+                a.y_dt == AQ_F16 ? make_uint2(round_pack2<AQ_F16>(w[0], w[1]), round_pack2<AQ_F16>(w[2], w[3]))
+                                 : make_uint2(round_pack2<AQ_BF16>(w[0], w[1]), round_pack2<AQ_BF16>(w[2], w[3]));
         } else {
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (e < nv) {
-                    if (a.y_dt == AQ_F32) ((float*)L.y)[yi + e] = v[e];
-                    else ((uint16_t*)L.y)[yi + e] = a.y_dt == AQ_F16 ? f32_to_bits<AQ_F16>(v[e]) : f32_to_bits<AQ_BF16>(v[e]);
+            for (int e = 0; e < 4; ++e)
+                if (o + e < out) {
+                    if (a.y_dt == AQ_F32) ((float*)y)[yi + e] = w[e];
+                    else ((uint16_t*)y)[yi + e] = a.y_dt == AQ_F16 ? f32_to_bits<AQ_F16>(w[e]) : f32_to_bits<AQ_BF16>(w[e]);
                 }
         }
     }
@@ -463,7 +456,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 // ---- host side ------------------------------------------------------------------------------
 
 struct TsPlan {
-    int n, ntiles, qr, kc, spc, cshift, nsb, books_off, bar_off;   // (kc, spc: of the first layer)
+    int n, ntiles, qr, kc, spc, nsb, books_off, bar_off;   // (kc, spc: of the first layer)
     size_t smem;
     double clocks;                     // estimated time of the call
 };
@@ -483,8 +476,7 @@ bool ts_plan(const Dims* ds, int nl, int m, int tokens, const DeviceInfo& di, Ts
     if ((d.B != 8 && d.B != 4) || m > kTsMaxM) return false;
     p->ntiles = (tokens + 255) / 256;
     p->n = ((tokens + p->ntiles - 1) / p->ntiles + 15) / 16 * 16;
-    p->cshift = 3;
-    const int books = (m * 16 << d.B) << p->cshift, stage = p->n * 128;
+    const int books = (m * 16 << d.B) << kTsCopies, stage = p->n * 128;
     const int tail = (kTsBars + 1) * 8 + (128 + 256) * 4;
     int nsb = (di.smem_optin - books - tail - 1024 - 16) / stage;   // (1 KiB of static shared memory)
     if (nsb > kTsRing) nsb = kTsRing;
@@ -569,7 +561,6 @@ aq_status launch_ts_set(const Dims& d, int m, const TsPlan& p, TsArgs a, int til
     a.in = d.in;
     a.ng = d.ng;
     a.S = d.S;
-    a.cshift = p.cshift;
     a.qr = p.qr;
     a.kc = p.kc;
     a.n = p.n;

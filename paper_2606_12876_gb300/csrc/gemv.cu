@@ -1029,7 +1029,7 @@ static bool gemv_uses_cw(const Dims& d, int m, int batch) {
 // Whether 9..16 tokens run the tensor-memory kernel (gemm_ts.cu): where its estimated time is below
 // that of gemv_cw, which at two token tiles is bound by the tensor pipe's legacy multiplies (64 a unit
 // of 32 rows, slice and book at 4 clocks; per SM, with its fixed cost). 14336 x 4096, m = 4, 16
-// tokens: 29 against 47.7 us; 1024 x 4096, m = 4: gemv_cw stays. bf16 activations are copied to the
+// tokens: 27.7 against 47.7 us; 1024 x 4096, m = 4: gemv_cw stays. bf16 activations are copied to the
 // workspace first (about 3000 clocks), which has room unless the layer has few rows. 8-bit codes
 // only: with 4-bit codes every intermediate of a GEMV is fp32 or exact, and stays so.
 static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt) {
