@@ -236,10 +236,28 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
             const float sc = pow2f(-f);
             for (int i = tid; i < nslot; i += kCwThreads)
                 books_s[i] = scaled_to_f16<BDT>(__ldg((const uint4*)L.books + (i >> a.cshift)), sc);
+        } else if constexpr (B == 4) {                  // few codewords: a thread per copy
+            for (int i = tid; i < nslot; i += kCwThreads) books_s[i] = __ldg((const uint4*)L.books + (i >> a.cshift));
         } else {
-#pragma unroll 4
-            for (int i = tid; i < nslot; i += kCwThreads)
-                books_s[i] = __ldg((const uint4*)L.books + (i >> a.cshift));
+            // each codeword loaded once (two in flight), its copies written from copy `lane` on, so that eight
+            // lanes meet no bank group twice
+            auto put = [&](int i, const uint4& c) {
+                if (a.cshift == 3) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) books_s[i * 8 + ((q + lane) & 7)] = c;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) books_s[i * 4 + ((q + lane) & 3)] = c;
+                }
+            };
+            const int n = a.m * NC;
+            for (int i = tid; i < n; i += 2 * kCwThreads) {
+                const int j = i + kCwThreads;
+                const uint4 c0 = __ldg((const uint4*)L.books + i);
+                const uint4 c1 = j < n ? __ldg((const uint4*)L.books + j) : c0;
+                put(i, c0);
+                if (j < n) put(j, c1);
+            }
         }
     };
     if (a.static_weights) {   // read-only weights: requested before the preceding kernel has finished
