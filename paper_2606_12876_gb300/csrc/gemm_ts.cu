@@ -496,8 +496,8 @@ bool ts_plan(const Dims* ds, int nl, int m, int tokens, const DeviceInfo& di, Ts
             double stage_clk = p->n * 2.2 > 270.0 ? p->n * 2.2 : 270.0;
             if (qr * 53.0 * m + p->n * 0.45 > stage_clk) stage_clk = qr * 53.0 * m + p->n * 0.45;
             if (chain > stage_clk) stage_clk = chain;
-            const double t = waves * (spc / 4 * 16 * stage_clk + (spc % 4 ? 16 * chain : 0.0) + 7500.0 +
-                                      (kc == 1 ? 0.0 : kc < 8 ? 3000.0 : 6000.0) + p->n * 16.0);
+            const double t = waves * (spc / 4 * 16 * stage_clk + (spc % 4 ? 16 * chain : 0.0) + 5000.0 +
+                                      (kc == 1 ? 0.0 : kc < 8 ? 1500.0 : 4500.0) + p->n * 16.0);
             if (best < 0.0 || t < best) {
                 best = t;
                 p->qr = qr;

@@ -1026,20 +1026,19 @@ static bool gemv_uses_cw(const Dims& d, int m, int batch) {
     return batch > kLutMaxBatch || (batch == 1 && d.S * m <= 8 && d.RBc <= 64);
 }
 
-// Whether 9..16 tokens run the tensor-memory kernel (gemm_ts.cu): where its estimated time is below
-// that of gemv_cw, which at two token tiles is bound by the tensor pipe's legacy multiplies (64 a unit
-// of 32 rows, slice and book at 4 clocks; per SM, with its fixed cost). 14336 x 4096, m = 4, 16
-// tokens: 27.7 against 47.7 us; 1024 x 4096, m = 4: gemv_cw stays. bf16 activations are copied to the
-// workspace first (about 3000 clocks), which has room unless the layer has few rows. 8-bit codes
-// only: with 4-bit codes every intermediate of a GEMV is fp32 or exact, and stays so.
+// Whether 9..16 tokens run the tensor-memory kernel (gemm_ts.cu): where its estimated time is below that of
+// gemv_cw with two token tiles, which gathers every codeword twice. 16 tokens: 14336 x 4096, m = 4 27.7 us
+// (gemv_cw 47.7); 4096 x 4096, m = 4 12.2 (17.8); but 1024 x 4096, m = 2 9.0 against gemv_cw's 5.3 and
+// 1024 x 1024, m = 4 10.1 against 3.9. bf16 activations are copied to the workspace first (about 3000
+// clocks), which has room unless the layer has few rows. 8-bit codes only: with 4-bit codes every
+// intermediate of a GEMV is fp32 or exact, and stays so.
 static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt) {
     if (batch <= 8 || d.B != 8) return false;
     const size_t room = gemv_ws_planes(d, batch) * (size_t)d.rows_pad * 4;
     if (x_dt == AQ_BF16 && room < kWsStatusBytes + (size_t)batch * d.in * 2) return false;
     const double ts = ts_clocks(d, m, batch);
     if (ts < 0.0) return false;
-    const double units = (double)d.S * m * d.RBc / 152.0;
-    return ts + (x_dt == AQ_BF16 ? 3000.0 : 0.0) < units * 400.0 + 8000.0;
+    return ts + (x_dt == AQ_BF16 ? 3000.0 : 0.0) < cw_clocks(d, m, batch) + 5800.0;   // (+ its launch and start)
 }
 
 // The tensor-memory kernel for n layers that share x; ws0: the first layer's workspace, whose partial-sum

@@ -21,7 +21,7 @@
 //
 // Work split: a warp's work item is a (32-row block, slice, book); a cluster of kc CTAs (16 warps
 // each) owns whole row blocks, its warps share the row block's (slice, book) units evenly in
-// slice-major order (so a warp's B fragments, 32 or 64 registers, are loaded once per slice), and
+// slice-major order (so a warp's B fragments, 32 registers, are loaded once per slice), and
 // the warps' accumulators are added in a fixed order in shared memory (and over the cluster
 // through distributed shared memory). So the kernel writes y itself: no partial planes in the
 // workspace and no reduction launch. kc > 1 is for layers with too few row blocks for the SMs.
@@ -45,6 +45,7 @@ namespace {
 constexpr int kCwWarps = 16;
 constexpr int kCwThreads = kCwWarps * 32;
 constexpr int kCwPitch = 36;       // floats per token in a warp's sums (4 of padding: no conflicts)
+constexpr int kCwTokens = 8;       // tokens of a CTA (more: token tiles along the grid's y)
 
 // One layer of a launch; a launch holds one layer, or several that share the activations and the split
 // (aq_gemv_group): cluster c of the layer takes row blocks c, c + nclusters, ...
@@ -68,11 +69,11 @@ struct CwArgs {
 };
 
 // Shared memory: books [m][2^B][2^cshift] x 16 B, codes 16 warps x 32 rows, the warps' sums (two
-// buffers of [16][8 NT][36] floats), the CTA's sums (two buffers of [8 NT][32]; clusters only).
-constexpr size_t cw_red_floats(int nt) { return (size_t)kCwWarps * 8 * nt * kCwPitch; }
-inline size_t cw_smem_bytes(int B, int m, int cshift, int nt) {
+// buffers of [16][8][36] floats), the CTA's sums (two buffers of [8][32]; clusters only).
+constexpr size_t kCwRedFloats = (size_t)kCwWarps * kCwTokens * kCwPitch;
+inline size_t cw_smem_bytes(int B, int m, int cshift) {
     return ((size_t)m * 16 << B << cshift) + (size_t)kCwWarps * 32 * unit_bytes(B) +
-           (2 * cw_red_floats(nt) + 2 * 256 * (size_t)nt) * 4;
+           (2 * kCwRedFloats + 2 * 32 * kCwTokens) * 4;
 }
 
 template <int DT>
@@ -175,9 +176,9 @@ struct RowCodes {
 // that costs a decimal of fp32 (relative error of an fp32 y 1.2e-6; chains of eight 2e-7; fp32 sums 1.2e-7).
 // Chains of eight (3 to 10 % more time) stand where calls had fp32 sums: up to four tokens, 4-bit codes;
 // single multiplies at one token (1.1 to 1.2e-7 on the small layers that come here, as the tables).
-template <int B, int BDT, int XDT, int NT, int CHAIN>
+template <int B, int BDT, int XDT, int CHAIN>
 __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_constant__ CwArgs a) {
-    constexpr int UNIT = unit_bytes(B), NC = 1 << B, NTOK = 8 * NT;
+    constexpr int UNIT = unit_bytes(B), NC = 1 << B;
     constexpr int MDT = BDT == AQ_BF16 && XDT == AQ_BF16 ? AQ_BF16 : AQ_F16;   // operand type
     constexpr bool kScaleX = XDT != MDT, kScaleB = BDT != MDT;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -186,14 +187,14 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     const int nslot = (a.m * NC) << a.cshift;
     unsigned char* codes_s = smem + (size_t)nslot * 16;
     float* red = (float*)(codes_s + kCwWarps * 32 * UNIT);
-    float* csum = red + 2 * cw_red_floats(NT);
+    float* csum = red + 2 * kCwRedFloats;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = a.kc > 1 ? (int)cluster_rank() : 0;
     int cid = (int)blockIdx.x / a.kc, layer = 0;
     while (layer + 1 < a.nlayers && cid >= a.L[layer + 1].c0) ++layer;
     const CwLayer& L = a.L[layer];
     cid -= L.c0;
-    const int tb = (int)blockIdx.y * NTOK;               // first token
+    const int tb = (int)blockIdx.y * kCwTokens;               // first token
 
     // this warp's (slice, book) units u0 .. u1-1 of every row block of the cluster; u = s*m + k
     const long long U = (long long)a.S * a.m;
@@ -276,71 +277,62 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     unsigned char* buf = codes_s + warp * 32 * UNIT;
     const uint32_t mul = 16u << a.cshift;
     const uint32_t books_u = smem_u32(books_s) + ((uint32_t)(lane & ((1 << a.cshift) - 1)) << 4);
-    uint4 bf[NT][8];                                     // B fragments of slice cur_s
-    float fac[NT][2];                                    // (kScaleX) 2^e of tokens 2c, 2c+1
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) fac[nt][0] = fac[nt][1] = 1.0f;   // a warp without units
+    uint4 bf[8];                                         // B fragments of slice cur_s
+    float fac[2] = {1.0f, 1.0f};                         // (kScaleX) 2^e of tokens 2c, 2c+1
     int cur_s = -1;
     auto load_b = [&](int s) {
+        const int t = tb + g;
+        const uint4* src = (const uint4*)(a.x + (size_t)t * a.in) + s * 32 + c;
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-            const int t = tb + 8 * nt + g;
-            const uint4* src = (const uint4*)(a.x + (size_t)t * a.in) + s * 32 + c;
+        for (int j = 0; j < 8; ++j)
+            bf[j] = t < a.batch && s * 32 + 4 * j + c < a.ng ? __ldg(src + 4 * j) : make_uint4(0u, 0u, 0u, 0u);
+        if constexpr (kScaleX) {
+            float mx = 0.0f;
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                bf[nt][j] = t < a.batch && s * 32 + 4 * j + c < a.ng ? __ldg(src + 4 * j) : make_uint4(0u, 0u, 0u, 0u);
-            if constexpr (kScaleX) {
-                float mx = 0.0f;
+            for (int j = 0; j < 8; ++j) mx = fmaxf(mx, max_abs8<XDT>(bf[j]));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            const int e = f16_exponent(mx);
+            const float sc = pow2f(-e), up = pow2f(e);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) mx = fmaxf(mx, max_abs8<XDT>(bf[nt][j]));
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-                const int e = f16_exponent(mx);
-                const float sc = pow2f(-e), up = pow2f(e);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) bf[nt][j] = scaled_to_f16<XDT>(bf[nt][j], sc);
-                fac[nt][0] = __shfl_sync(0xffffffffu, up, 8 * c);
-                fac[nt][1] = __shfl_sync(0xffffffffu, up, 8 * c + 4);
-            }
+            for (int j = 0; j < 8; ++j) bf[j] = scaled_to_f16<XDT>(bf[j], sc);
+            fac[0] = __shfl_sync(0xffffffffu, up, 8 * c);
+            fac[1] = __shfl_sync(0xffffffffu, up, 8 * c + 4);
         }
         cur_s = s;
     };
 
     int pass = 0;
     for (int rb = cid; rb < L.RBc; rb += L.nclusters, ++pass) {
-        float acc[2][NT][4];
+        float acc[2][4];
         // The warps' sums of a pass, added in warp order. Two buffers: a pass's writes meet the sums
         // that are read two passes earlier, which every thread finished before the last barrier.
-        float* rp = red + (pass & 1) * cw_red_floats(NT);
-        float* mine = rp + (size_t)warp * NTOK * kCwPitch;
+        float* rp = red + (pass & 1) * kCwRedFloats;
+        float* mine = rp + (size_t)warp * kCwTokens * kCwPitch;
         bool first = true;
         // the row scale of the output this thread finishes, requested before the pass's gathers
         const int my_o = rb * 32 + (tid & 31);
-        const float my_s = tid < 32 * NTOK && my_o < L.out ? bits_to_f32_rt(L.scales[my_o], a.scale_dt) : 0.0f;
+        const float my_s = tid < 32 * kCwTokens && my_o < L.out ? bits_to_f32_rt(L.scales[my_o], a.scale_dt) : 0.0f;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.0f;
+            for (int e = 0; e < 4; ++e) acc[mt][e] = 0.0f;
         // The accumulators into the warp's sums in shared memory; with kScaleX once per slice, times
         // the slice's 2^e (added to the earlier slices'), else once at the end of the pass.
         auto fold = [&]() {
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        float* p = mine + (8 * nt + 2 * c + (e & 1)) * kCwPitch + 16 * mt + 8 * (e >> 1) + g;
-                        if constexpr (kScaleX) {
-                            const float v = acc[mt][nt][e] * fac[nt][e & 1];
-                            *p = first ? v : *p + v;
-                            acc[mt][nt][e] = 0.0f;
-                        } else {
-                            *p = acc[mt][nt][e];
-                        }
+                for (int e = 0; e < 4; ++e) {
+                    float* p = mine + (2 * c + (e & 1)) * kCwPitch + 16 * mt + 8 * (e >> 1) + g;
+                    if constexpr (kScaleX) {
+                        const float v = acc[mt][e] * fac[e & 1];
+                        *p = first ? v : *p + v;
+                        acc[mt][e] = 0.0f;
+                    } else {
+                        *p = acc[mt][e];
                     }
+                }
             first = false;
         };
         for (int u = u0; u < u1; ++u) {
@@ -358,12 +350,12 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
             for (int rr = 0; rr < 4; ++rr) cw[rr].load(buf, g + 8 * rr, c);
             __syncwarp();                                // the buffer may be refilled
             const uint32_t base = books_u + (uint32_t)k * (NC * mul);
-            float part[2][NT][4] = {};                   // (CHAIN > 0) the current chains
-            auto take = [&](int mt, int nt) {
+            float part[2][4] = {};                       // (CHAIN > 0) the current chains
+            auto take = [&](int mt) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    acc[mt][nt][e] += part[mt][nt][e];
-                    part[mt][nt][e] = 0.0f;
+                    acc[mt][e] += part[mt][e];
+                    part[mt][e] = 0.0f;
                 }
             };
 #pragma unroll
@@ -372,26 +364,24 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
 #pragma unroll
                 for (int rr = 0; rr < 4; ++rr) w[rr] = lds128(base + cw[rr].code(j) * mul);
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        float(&d)[4] = CHAIN ? part[mt][nt] : acc[mt][nt];
-                        mma16<MDT>(d, w[2 * mt].x, w[2 * mt + 1].x, w[2 * mt].y, w[2 * mt + 1].y, bf[nt][j].x, bf[nt][j].y);
-                        if (CHAIN == 1) take(mt, nt);
-                        mma16<MDT>(d, w[2 * mt].z, w[2 * mt + 1].z, w[2 * mt].w, w[2 * mt + 1].w, bf[nt][j].z, bf[nt][j].w);
-                        if (CHAIN == 1 || (CHAIN == 8 && (j & 3) == 3)) take(mt, nt);
-                    }
+                for (int mt = 0; mt < 2; ++mt) {
+                    float(&d)[4] = CHAIN ? part[mt] : acc[mt];
+                    mma16<MDT>(d, w[2 * mt].x, w[2 * mt + 1].x, w[2 * mt].y, w[2 * mt + 1].y, bf[j].x, bf[j].y);
+                    if (CHAIN == 1) take(mt);
+                    mma16<MDT>(d, w[2 * mt].z, w[2 * mt + 1].z, w[2 * mt].w, w[2 * mt + 1].w, bf[j].z, bf[j].w);
+                    if (CHAIN == 1 || (CHAIN == 8 && (j & 3) == 3)) take(mt);
+                }
             }
         }
         fold();
         __syncthreads();
-        const int i0 = a.kc > 1 ? rank * (32 * NTOK / a.kc) : 0;      // outputs this CTA finishes
-        const int i1 = a.kc > 1 ? i0 + 32 * NTOK / a.kc : 32 * NTOK;
-        float* cs = csum + (pass & 1) * 32 * NTOK;
+        const int i0 = a.kc > 1 ? rank * (32 * kCwTokens / a.kc) : 0;      // outputs this CTA finishes
+        const int i1 = a.kc > 1 ? i0 + 32 * kCwTokens / a.kc : 32 * kCwTokens;
+        float* cs = csum + (pass & 1) * 32 * kCwTokens;
         float v = 0.0f;
-        if (tid < 32 * NTOK) {
+        if (tid < 32 * kCwTokens) {
 #pragma unroll
-            for (int w = 0; w < kCwWarps; ++w) v += rp[((size_t)w * NTOK + (tid >> 5)) * kCwPitch + (tid & 31)];
+            for (int w = 0; w < kCwWarps; ++w) v += rp[((size_t)w * kCwTokens + (tid >> 5)) * kCwPitch + (tid & 31)];
             if (a.kc > 1) cs[tid] = v;
         }
         if (a.kc > 1) {
@@ -424,23 +414,27 @@ inline int cw_cshift(int B, int m) { return B == 4 || m <= 4 ? 3 : 2; }
 
 // CTAs per cluster: the split with the smallest estimated time of the busiest cluster, in clocks:
 // passes over its row blocks times the units of a warp (a unit's gathers are 128 wavefronts, plus
-// about 24 of staging, shared by the SM's active warps, or the latency of its eight steps) and the
-// reduction of a pass, plus what a cluster launch and its barriers cost over a plain one (measured
+// about 32 of staging and the rest, shared by the SM's active warps, or the latency of its eight steps)
+// and about 1500 clocks of reduction and start-up a pass, plus what a cluster launch and its barriers cost over a plain one (measured
 // about 2 us for two or four CTAs, 6 for eight: 512 x 4096, m = 4 took 10.8 us in clusters of eight).
 // Clusters of 2, 4 and 8 that are resident at once: 76, 36 and 16 on 152 SMs.
-inline int cw_clusters(int kc, int sms) { return kc == 1 ? sms : kc == 2 ? sms / 2 : kc == 4 ? sms * 9 / 38 : sms * 2 / 19; }
-inline int cw_cluster(const Dims& d, int m, int sms, int* nclusters) {
+// With several token tiles each tile has its share of the SMs.
+inline int cw_tiles(int batch) { return (batch + kCwTokens - 1) / kCwTokens; }
+inline int cw_clusters(int kc, int tiles, int sms) {
+    const int n = (kc == 1 ? sms : kc == 2 ? sms / 2 : kc == 4 ? sms * 9 / 38 : sms * 2 / 19) / tiles;
+    return n < 1 ? 1 : n;
+}
+inline int cw_cluster(const Dims& d, int m, int tiles, int sms, int* nclusters, double* clocks) {
     int best = 1;
     double best_t = -1.0;
     for (int kc = 1; kc <= 8; kc *= 2) {
-        int nc = cw_clusters(kc, sms);
+        int nc = cw_clusters(kc, tiles, sms);
         if (nc > d.RBc) nc = d.RBc;
-        if (nc < 1) nc = 1;
         const long long U = (long long)d.S * m;
         const long long units = (U + 16 * kc - 1) / (16 * kc);
         const long long active = U < 16 * kc ? (U + kc - 1) / kc : 16;
-        const double unit_clk = active * 152 > 900 ? active * 152.0 : 900.0;
-        const double t = (double)((d.RBc + nc - 1) / nc) * (units * unit_clk + (kc > 1 ? 1100.0 : 400.0)) +
+        const double unit_clk = active * 160 > 900 ? active * 160.0 : 900.0;
+        const double t = (double)((d.RBc + nc - 1) / nc) * (units * unit_clk + (kc > 1 ? 2200.0 : 1500.0)) +
                          (kc == 1 ? 0.0 : kc < 8 ? 3500.0 : 11000.0);
         if (best_t < 0.0 || t < best_t) {
             best_t = t;
@@ -448,39 +442,45 @@ inline int cw_cluster(const Dims& d, int m, int sms, int* nclusters) {
             *nclusters = nc;
         }
     }
+    *clocks = best_t;
     return best;
 }
 
-template <int B, int BDT, int XDT, int NT, int CHAIN>
+template <int B, int BDT, int XDT, int CHAIN>
 aq_status run_cw(CwArgs a, cudaStream_t st) {
-    auto kern = gemv_cw_kernel<B, BDT, XDT, NT, CHAIN>;
+    auto kern = gemv_cw_kernel<B, BDT, XDT, CHAIN>;
     a.cshift = cw_cshift(B, a.m);
-    const size_t smem = cw_smem_bytes(B, a.m, a.cshift, NT);
+    const size_t smem = cw_smem_bytes(B, a.m, a.cshift);
     int occ = 0;
     if (aq_status e = prepare(kern, smem, kCwThreads, a.m, &occ); e != AQ_OK) return e;
     const CwLayer& last = a.L[a.nlayers - 1];
-    return launch_pdl_cluster(a.kc, kern, dim3((last.c0 + last.nclusters) * a.kc, (a.batch + 8 * NT - 1) / (8 * NT)),
-                              dim3(kCwThreads), smem, st, a);
+    return launch_pdl_cluster(a.kc, kern, dim3((last.c0 + last.nclusters) * a.kc, cw_tiles(a.batch)), dim3(kCwThreads), smem, st, a);
 }
 
-// 4-bit codes: one token tile per CTA at any batch (two tiles of short chains do not fit the registers).
 template <int B, int BDT, int XDT>
-aq_status run_cw_nt(const CwArgs& a, cudaStream_t st) {
-    if constexpr (B == 4) return run_cw<B, BDT, XDT, 1, 8>(a, st);
-    else if (a.batch == 1) return run_cw<B, BDT, XDT, 1, 1>(a, st);
-    else if (a.batch <= 4) return run_cw<B, BDT, XDT, 1, 8>(a, st);
-    else if (a.batch <= 8) return run_cw<B, BDT, XDT, 1, 0>(a, st);
-    else return run_cw<B, BDT, XDT, 2, 0>(a, st);
+aq_status run_cw_chain(const CwArgs& a, cudaStream_t st) {
+    if constexpr (B == 4) return run_cw<B, BDT, XDT, 8>(a, st);
+    else if (a.batch == 1) return run_cw<B, BDT, XDT, 1>(a, st);
+    else if (a.batch <= 4) return run_cw<B, BDT, XDT, 8>(a, st);
+    else return run_cw<B, BDT, XDT, 0>(a, st);
 }
 
 template <int B>
 aq_status run_cw_types(const CwArgs& a, int book_dt, int x_dt, cudaStream_t st) {
     if (book_dt == AQ_BF16)
-        return x_dt == AQ_BF16 ? run_cw_nt<B, AQ_BF16, AQ_BF16>(a, st) : run_cw_nt<B, AQ_BF16, AQ_F16>(a, st);
-    return x_dt == AQ_BF16 ? run_cw_nt<B, AQ_F16, AQ_BF16>(a, st) : run_cw_nt<B, AQ_F16, AQ_F16>(a, st);
+        return x_dt == AQ_BF16 ? run_cw_chain<B, AQ_BF16, AQ_BF16>(a, st) : run_cw_chain<B, AQ_BF16, AQ_F16>(a, st);
+    return x_dt == AQ_BF16 ? run_cw_chain<B, AQ_F16, AQ_BF16>(a, st) : run_cw_chain<B, AQ_F16, AQ_F16>(a, st);
 }
 
 }  // namespace
+
+double cw_clocks(const Dims& d, int m, int batch) {
+    DeviceInfo di;
+    int nc;
+    double t = -1.0;
+    if (device_info(&di) == AQ_OK) cw_cluster(d, m, cw_tiles(batch), di.sms, &nc, &t);
+    return t;
+}
 
 aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, const void* const* books,
                     const void* const* scales, const void* x, int x_dt, int batch, void* const* y, int y_dt,
@@ -489,7 +489,9 @@ aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, con
     if (aq_status e = device_info(&di); e != AQ_OK) return e;
     const Dims& d = ds[0];
     int kcs[4], own[4];
-    for (int l = 0; l < n; ++l) kcs[l] = cw_cluster(ds[l], m, di.sms, &own[l]);
+    const int tiles = cw_tiles(batch);
+    double clocks;
+    for (int l = 0; l < n; ++l) kcs[l] = cw_cluster(ds[l], m, tiles, di.sms, &own[l], &clocks);
     bool done[4] = {};
     for (int f = 0; f < n; ++f) {
         if (done[f]) continue;
@@ -504,7 +506,7 @@ aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, con
                 set[a.nlayers++] = l;
             }
         // the fewest passes that the resident clusters allow over all layers
-        const int cap = cw_clusters(a.kc, di.sms);
+        const int cap = cw_clusters(a.kc, tiles, di.sms);
         int passes = (rbs + cap - 1) / cap;
         auto need = [&](int p) {
             int c = 0;
