@@ -1044,9 +1044,10 @@ aq_status run_gemm_dense(const Dims& d, int m, const void* planes, const void* b
 // two. (14336 x 4096, m = 4: 31.7 against 79.4 us at 100 tokens, 73.1 against 81.8 at 512; m = 1:
 // 54.0 against 45.3 at 512, where the pair kernel stays; 4096 x 14336, m = 3, 100 tokens: 27.5
 // against 211.) 4-bit layouts have no in-loop form; their other way, decoding W_m first, costs about
-// 15000 clocks and 2 bytes per weight of HBM more than its product.
+// 15000 clocks and 2 bytes per weight of HBM more than its product. Five and more books leave too
+// little shared memory for the activation stages of more than a few tokens.
 bool gemm_uses_ts(const Dims& d, int m, int tokens) {
-    if (tokens >= kGemmDenseTokens) return false;
+    if (tokens >= kGemmDenseTokens || m > 4) return false;
     const double ts = ts_clocks(d, m, tokens);
     if (ts < 0.0) return false;
     const int np = d.B == 4 ? 1 : gemm_pairs_per_cluster(m, tokens);

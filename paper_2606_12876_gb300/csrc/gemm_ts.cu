@@ -20,12 +20,14 @@
 // slices in turn. A stage has one barrier for both operands (an arrival per decoder warp, and the
 // TMA's bytes) and one commit: every shared-memory operation of the issuing thread queues behind
 // the gathers (about 100 clocks each), so at few tokens its barrier operations would be the bound
-// (two waits with abort flags and two commits per stage: 0.35 us a stage; one of each: 0.13). A cluster of kc CTAs splits the slices of a tile; every CTA stages its sums in
-// shared memory (free once its MMAs completed) and each finishes a share of the tokens, adding the
-// CTAs' sums in rank order.
+// (two waits with abort flags and two commits per stage: 0.35 us a stage; one of each: 0.13). A
+// cluster of kc CTAs splits the slices of a tile; every CTA stages its sums in shared memory (free
+// once its MMAs completed) and each finishes a share of the tokens, adding the CTAs' sums in rank
+// order.
 // Measured (the call, with the copy of bf16 activations), against the pair kernel: 4096 x 14336, m = 3,
-// 100 tokens 27.5 / 211 us; 14336 x 4096, m = 4, 100 tokens 31.7 / 79.4 us, 512 tokens 73.1 / 81.8 us;
-// 16 tokens, m = 4: 27.7 us against gemv_cw's 47.7.
+// 100 tokens 28.0 / 213 us; 14336 x 4096, m = 4, 100 tokens 31.7 / 79.4 us, 512 tokens 74 / 83 us; 16 tokens,
+// m = 4: 27.6 us against 54.9 of the tf32 kernel before and 47.7 of gemv_cw. Five to eight books,
+// 14336 x 4096, 16 tokens: 32 / 37 / 56 / 64 us (tf32 kernel: 66 / 77 / 88 / 179).
 // Roles: warps 0-15 decoders (warp w: quarter w mod 4, set w / 4; the warps of absent quarters idle)
 // and epilogue; one warp for TMA (and L2 prefetch of the codes), one for MMA issue and the
 // tensor-memory allocation: with qr = 4 two more warps (96 registers a thread), else two of the idle
@@ -45,9 +47,10 @@ namespace aq {
 namespace {
 
 constexpr int kTsDec = 16;          // decoder warps
-constexpr int kTsMaxM = 4;          // prefixes compiled for the sums form
+constexpr int kTsMaxM = 8;          // prefixes compiled (4-bit codes: 4)
 constexpr int kTsRing = 8;          // weight stages in tensor memory (32 columns each, from column 256)
-constexpr int kTsCopies = 3;        // log2 of the interleaved copies of a codebook
+// Log2 of the interleaved copies of a codebook: eight while m books of them fit.
+constexpr int ts_copies(int m) { return m <= 6 ? 3 : 2; }
 constexpr int kTsBars = 2 * kTsRing + 1;
 
 // One layer of a launch; a launch holds one layer, or several that share the activations and the split
@@ -75,7 +78,8 @@ __global__ void __launch_bounds__(Q4 ? 576 : 512, 1)
 gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ TsArgs a) {
     constexpr int UNIT = unit_bytes(B), NC = 1 << B, NW = UNIT / 4, m = MB;
     constexpr int kTsThreads = Q4 ? 576 : 512, kTmaWarp = Q4 ? 16 : 3, kMmaWarp = Q4 ? 17 : 7;
-    constexpr bool kAhead = !(Q4 && MB == 4);           // next slice's codes in registers ahead of use
+    constexpr bool kAhead = MB <= (Q4 ? 3 : 4);         // next slice's codes in registers ahead of use
+    constexpr int kCopies = ts_copies(MB);
     extern __shared__ __align__(1024) unsigned char smem[];
     uint4* books_s = (uint4*)(smem + a.books_off);
     uint64_t* full = (uint64_t*)(smem + a.bar_off);     // both operands of a stage are in place
@@ -182,7 +186,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         pdl_launch_dependents();
         fetch();
     }
-    // Books staged times 2^-f (fp16 range, operand_scale.cuh): each thread writes the eight copies of its
+    // Books staged times 2^-f (fp16 range, operand_scale.cuh): each thread writes the copies of its
     // codewords, starting at copy `lane` so that eight lanes meet no bank group twice.
 #pragma unroll
     for (int l = 0; l < kPer; ++l) {
@@ -204,7 +208,7 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         const uint4 v = f ? scale_codeword<BDT>(bk[l], pow2f(-f)) : bk[l];
         if (i < m * NC)
 #pragma unroll
-            for (int c = 0; c < 8; ++c) books_s[i * 8 + ((c + lane) & 7)] = v;
+            for (int c = 0; c < 1 << kCopies; ++c) books_s[(i << kCopies) + ((c + lane) & ((1 << kCopies) - 1))] = v;
     }
     if (tid < 128) scale_s[tid] = bits_to_f32_rt(sbits, a.scale_dt) * bfac;
     if (a.static_weights) {
@@ -279,8 +283,8 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         __syncwarp();
     } else if (decoder) {
         // ---------------- decoders
-        constexpr uint32_t mul = 16u << kTsCopies;
-        const uint32_t books_u = smem_u32(books_s) + ((uint32_t)(lane & 7) << 4);
+        constexpr uint32_t mul = 16u << kCopies;
+        const uint32_t books_u = smem_u32(books_s) + ((uint32_t)(lane & ((1 << kCopies) - 1)) << 4);
         const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + 256;
         auto unrotate = [&](const uint32_t (&raw)[NW], uint32_t (&u)[NW]) {
             if constexpr (B == 8) {
@@ -468,22 +472,25 @@ struct TsPlan {
 // MMAs (268 clocks at 112 tokens, 556 at 256); the issuer's barrier and commit (270); shared memory:
 // the gathers of 8 groups per row and book at 60 % of 8 codes a clock, and the activations' way
 // through it; a decoder warp's own chain (120 m + 165, a stage in four being its own), which bounds
-// one or two quarters and a last round of fewer than four slices.
+// one or two quarters and a last round of fewer than four slices. From five books the codes of a slice are
+// waited for (their registers leave no room to load them ahead), and from seven the four copies of a book
+// cost about twice the gathers; three quarters at most keep 128 registers a thread.
 // With a group of layers (nl > 1; the same K and number of books, so the same kc and spc each), the
 // tile height is chosen for the tiles of all of them and kc is the given one.
 bool ts_plan(const Dims* ds, int nl, int m, int tokens, const DeviceInfo& di, TsPlan* p, int only_kc = 0) {
     const Dims& d = ds[0];
-    if ((d.B != 8 && d.B != 4) || m > kTsMaxM) return false;
+    if ((d.B != 8 && d.B != 4) || m > (d.B == 8 ? kTsMaxM : 4)) return false;
     p->ntiles = (tokens + 255) / 256;
     p->n = ((tokens + p->ntiles - 1) / p->ntiles + 15) / 16 * 16;
-    const int books = (m * 16 << d.B) << kTsCopies, stage = p->n * 128;
+    const int books = (m * 16 << d.B) << ts_copies(m), stage = p->n * 128;
     const int tail = (kTsBars + 1) * 8 + (128 + 256) * 4;
     int nsb = (di.smem_optin - books - tail - 1024 - 16) / stage;   // (1 KiB of static shared memory)
     if (nsb > kTsRing) nsb = kTsRing;
     if (nsb < 2) return false;
     p->nsb = nsb;
     double best = -1.0;
-    for (int qr = 1; qr <= 4; ++qr)
+    const double gathers = m <= 6 ? m : 1.9 * m;
+    for (int qr = 1; qr <= (m <= 4 ? 4 : 3); ++qr)
         for (int kc = 1; kc <= 8; kc *= 2) {
             if (kc > d.S || (only_kc && kc != only_kc)) continue;
             long long tiles = 0;
@@ -492,9 +499,9 @@ bool ts_plan(const Dims* ds, int nl, int m, int tokens, const DeviceInfo& di, Ts
             const int cap = kc == 1 ? di.sms : kc == 2 ? di.sms / 2 : kc == 4 ? di.sms * 9 / 38 : di.sms * 2 / 19;
             const int spc = (d.S + kc - 1) / kc;
             const long long waves = (tiles + cap - 1) / cap;
-            const double chain = 120.0 * m + 165.0 + p->n * 0.3;
+            const double chain = (m <= 6 ? 120.0 : 180.0) * m + (m <= 4 ? 165.0 : 565.0) + p->n * 0.3;
             double stage_clk = p->n * 2.2 > 270.0 ? p->n * 2.2 : 270.0;
-            if (qr * 53.0 * m + p->n * 0.45 > stage_clk) stage_clk = qr * 53.0 * m + p->n * 0.45;
+            if (qr * 53.0 * gathers + p->n * 0.45 > stage_clk) stage_clk = qr * 53.0 * gathers + p->n * 0.45;
             if (chain > stage_clk) stage_clk = chain;
             const double t = waves * (spc / 4 * 16 * stage_clk + (spc % 4 ? 16 * chain : 0.0) + 5000.0 +
                                       (kc == 1 ? 0.0 : kc < 8 ? 1500.0 : 4500.0) + p->n * 16.0);
@@ -520,7 +527,9 @@ bool ts_plan(const Dims* ds, int nl, int m, int tokens, const DeviceInfo& di, Ts
 
 template <int B, int BDT, int MB>
 aq_status run_ts(const TsPlan& p, const CUtensorMap& map, const TsArgs& a, int tiles, cudaStream_t st) {
-    auto kern = p.qr == 4 ? gemm_ts_kernel<B, BDT, MB, true> : gemm_ts_kernel<B, BDT, MB, false>;
+    auto kern = gemm_ts_kernel<B, BDT, MB, false>;
+    if constexpr (MB <= 4)
+        if (p.qr == 4) kern = gemm_ts_kernel<B, BDT, MB, true>;
     const int threads = p.qr == 4 ? 576 : 512;
     int occ = 0;
     // slot 0: the limit is raised to the most a launch may use; each plan stays below it
@@ -534,8 +543,17 @@ aq_status run_ts_m(const TsPlan& p, const CUtensorMap& map, const TsArgs& a, int
         case 1: return run_ts<B, BDT, 1>(p, map, a, tiles, st);
         case 2: return run_ts<B, BDT, 2>(p, map, a, tiles, st);
         case 3: return run_ts<B, BDT, 3>(p, map, a, tiles, st);
-        default: return run_ts<B, BDT, 4>(p, map, a, tiles, st);
+        case 4: return run_ts<B, BDT, 4>(p, map, a, tiles, st);
     }
+    if constexpr (B == 8) {
+        switch (m) {
+            case 5: return run_ts<B, BDT, 5>(p, map, a, tiles, st);
+            case 6: return run_ts<B, BDT, 6>(p, map, a, tiles, st);
+            case 7: return run_ts<B, BDT, 7>(p, map, a, tiles, st);
+            case 8: return run_ts<B, BDT, 8>(p, map, a, tiles, st);
+        }
+    }
+    return AQ_ERR_UNSUPPORTED;
 }
 
 // One launch: plan p, the layers of a filled in, `tiles` row tiles.

@@ -1,5 +1,6 @@
-// gemv_cw: y = x * W_m^T for 2..16 tokens with 4- and 8-bit codes (the prefix-m reconstruction
-// of Sec. 3.2 / Sec. 5; Y = W X of Sec. 2.2), one kernel per call.
+// gemv_cw: y = x * W_m^T for 1..16 tokens with 4- and 8-bit codes (the prefix-m reconstruction
+// of Sec. 3.2 / Sec. 5; Y = W X of Sec. 2.2), one kernel per call. gemv.cu and gemm.cu say which
+// calls come here.
 //
 // By linearity in the books (Sec. 5), x_g . (sum_k C_k[b_k]) = sum_k x_g . C_k[b_k], and a
 // 16-byte codeword is, as it stands, the eight weights of one row and group: it goes straight
@@ -17,7 +18,12 @@
 // codebook is staged in 2^cshift interleaved copies, lane L reading copy L mod 2^cshift: with
 // eight copies there are no conflicts whatever the codes (a single copy costs about 2.6 times the
 // wavefronts). At 8 codes per clock and SM the gate projection (14336 x 4096, m = 4) cannot take
-// less than 12.6 us; every other unit (issue 34 %, tensor pipe at 16 tokens 50 %) has slack.
+// less than 12.6 us for eight tokens; the issue slots (34 %) and the tensor pipe (25 %) have slack.
+//
+// A CTA holds eight tokens (the N of the multiply); 9..16 tokens are two token tiles along the grid's y,
+// which gather every codeword twice. (One tile of 16 tokens spilled registers and kept fewer loads in
+// flight: 1024 x 4096, m = 2, 16 tokens 9.0 us, two tiles 5.3.) Larger layers run gemm_ts.cu instead, which
+// decodes once for all tokens (ts_clocks against cw_clocks, in gemv.cu).
 //
 // Work split: a warp's work item is a (32-row block, slice, book); a cluster of kc CTAs (16 warps
 // each) owns whole row blocks, its warps share the row block's (slice, book) units evenly in
@@ -32,9 +38,9 @@
 // the largest, and the slice's sums are scaled back when they are added to the total. bf16 books
 // with fp16 activations: the books are scaled the same way (one power of two for the m books).
 //
-// Measured, 8B block (seven layers; q/k/v and gate/up as groups): 8 tokens, m = 3 86.5 us (the eight-token
-// tables and tf32 kernel before: 145.8), 4-bit codes, 4 tokens, m = 4 92.2 us (fp32 kernel before: 229.7);
-// as seven single launches 91.1 and 96.3. 14336 x 4096, m = 4, 8 tokens: 22.5 us; 4096 x 4096: 9.8 us.
+// Measured, 8B block (seven layers; q/k/v and gate/up as groups): 8 tokens, m = 3 83.5 us (the eight-token
+// tables and tf32 kernel before: 145.8), 4-bit codes, 4 tokens, m = 4 91.1 us (fp32 kernel before: 229.7).
+// 14336 x 4096, 8 tokens: m = 3 17.8 us, m = 4 22.1 us; 1024 x 1024, m = 4, 16 tokens: 3.9 us.
 #include "aq_internal.cuh"
 #include "launch.cuh"
 #include "tc_ptx.cuh"
@@ -410,13 +416,14 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
 }
 
 // Copies of a codebook (log2): eight while they fit next to the sums, else four.
-inline int cw_cshift(int B, int m) { return B == 4 || m <= 4 ? 3 : 2; }
+inline int cw_cshift(int B, int m) { return B == 4 || m <= 5 ? 3 : 2; }
 
 // CTAs per cluster: the split with the smallest estimated time of the busiest cluster, in clocks:
-// passes over its row blocks times the units of a warp (a unit's gathers are 128 wavefronts, plus
-// about 32 of staging and the rest, shared by the SM's active warps, or the latency of its eight steps)
-// and about 1500 clocks of reduction and start-up a pass, plus what a cluster launch and its barriers cost over a plain one (measured
-// about 2 us for two or four CTAs, 6 for eight: 512 x 4096, m = 4 took 10.8 us in clusters of eight).
+// passes over its row blocks times the units of a warp (a unit's gathers are 128 wavefronts, about
+// twice that with four copies of a book, plus about 32 of staging and the rest, shared by the SM's
+// active warps, or the latency of its eight steps) and about 1500 clocks of reduction and start-up a
+// pass, plus what a cluster launch and its barriers cost over a plain one (measured about 2 us for two
+// or four CTAs, 6 for eight: 512 x 4096, m = 4 took 10.8 us in clusters of eight).
 // Clusters of 2, 4 and 8 that are resident at once: 76, 36 and 16 on 152 SMs.
 // With several token tiles each tile has its share of the SMs.
 inline int cw_tiles(int batch) { return (batch + kCwTokens - 1) / kCwTokens; }
@@ -433,7 +440,8 @@ inline int cw_cluster(const Dims& d, int m, int tiles, int sms, int* nclusters, 
         const long long U = (long long)d.S * m;
         const long long units = (U + 16 * kc - 1) / (16 * kc);
         const long long active = U < 16 * kc ? (U + kc - 1) / kc : 16;
-        const double unit_clk = active * 160 > 900 ? active * 160.0 : 900.0;
+        const double gather = cw_cshift(d.B, m) == 3 ? 160.0 : 300.0;
+        const double unit_clk = active * gather > 900.0 ? active * gather : 900.0;
         const double t = (double)((d.RBc + nc - 1) / nc) * (units * unit_clk + (kc > 1 ? 2200.0 : 1500.0)) +
                          (kc == 1 ? 0.0 : kc < 8 ? 3500.0 : 11000.0);
         if (best_t < 0.0 || t < best_t) {
