@@ -85,70 +85,80 @@ __global__ void beam_sym_kernel(const void* __restrict__ h, int h_dt, float* __r
 }
 
 // C[r][j] = sum_i A[r][i] * S[i][j] for r < rows, j < in (A = E of every prefix, rows = M*out).
-// Bound: the fp32 FMA pipe (2 * M * out * in^2 operations on the CUDA cores). T x T tiles of C,
-// (T/16)^2 outputs per thread in packed fp32 pairs, 16-deep k steps: the next step's tiles travel
-// into registers while the current ones are multiplied, and two shared buffers leave one barrier
-// per step. Every output is one chain of fused multiply-adds over i in ascending order from +0,
-// so the values do not depend on the tile. T = 128, or 64 where 128 gives fewer tiles than SMs.
+// Bound: the fp32 FMA pipe (2 * M * out * in^2 operations on the CUDA cores), with shared memory close
+// behind: a 16-byte load of a warp is four wavefronts even where lanes share it, so 8 x 8 outputs per
+// thread (16 words for 64 FMAs) cost as many clocks of shared memory as of FMAs. T x T tiles of C; at
+// T = 128 a thread has 8 x 16 outputs (24 words for 128 FMAs; 128 threads), in packed fp32 pairs (1024 x
+// 4096, M = 4, the call: 6.69 ms with 8 x 8, 6.35 with 8 x 16; with A's elements stored twice, which
+// saves the packing moves, 7.24). 16-deep k steps: the next step's tiles travel (A through registers,
+// which transposes it, S by cp.async) while the current ones are multiplied, and two shared buffers
+// leave one barrier per step. Every output is one chain of fused multiply-adds over i in ascending
+// order from +0, so the values do not depend on the tile. T = 128, or 64 where 128 gives fewer tiles
+// than SMs.
 template <int T>
-__global__ void __launch_bounds__(256, 2) beam_gemm_kernel(const float* __restrict__ A,
-                                                        const float* __restrict__ S,
-                                                        float* __restrict__ C, int rows, int in) {
-    constexpr int N = T / 64;              // 64-row (and 64-column) parts of a tile, 4 x 4 N^2 outputs
-    constexpr int LD = T * 4 / 256;        // 16-byte loads per thread of a 16-deep tile
+constexpr int kBeamGemmThreads = T == 128 ? 128 : 256;
+template <int T>
+__global__ void __launch_bounds__(kBeamGemmThreads<T>, 2) beam_gemm_kernel(const float* __restrict__ A,
+                                                                           const float* __restrict__ S,
+                                                                           float* __restrict__ C, int rows, int in) {
+    constexpr int NT = kBeamGemmThreads<T>, TX = NT / 16;      // thread columns
+    constexpr int N = T / 64, NC = T / (4 * TX);               // 4-row and 4-column parts per thread
+    constexpr int LD = T * 4 / NT;         // 16-byte loads per thread of a 16-deep tile
     __shared__ __align__(16) float As[2][16][T + 4], Bs[2][16][T];
     pdl_wait();
     pdl_launch_dependents();
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
     const int c0 = blockIdx.x * T, nk = (in + 15) / 16;
     for (int r0 = blockIdx.y * T; r0 < rows; r0 += gridDim.y * T) {
-        float4 ra[LD], rb[LD];
-        auto load = [&](int k0) {
+        float4 ra[LD];
+        auto load = [&](int k0, int buf) {
 #pragma unroll
             for (int l = 0; l < LD; ++l) {
-                const int i = tid + l * 256, r = r0 + i / 4, k = k0 + (i & 3) * 4;
+                const int i = tid + l * NT, r = r0 + i / 4, k = k0 + (i & 3) * 4;
                 ra[l] = r < rows && k < in ? __ldg((const float4*)(A + (size_t)r * in + k)) : float4{};
                 const int kb = k0 + i / (T / 4), cc = c0 + i % (T / 4) * 4;
-                rb[l] = kb < in && cc < in ? __ldg((const float4*)(S + (size_t)kb * in + cc)) : float4{};
+                float4* dst = (float4*)&Bs[buf][i / (T / 4)][i % (T / 4) * 4];
+                if (kb < in && cc < in) cp_async16(dst, S + (size_t)kb * in + cc);
+                else *dst = float4{};
             }
+            cp_async_commit();
         };
         auto store = [&](int buf) {
 #pragma unroll
             for (int l = 0; l < LD; ++l) {
-                const int i = tid + l * 256, r = i / 4, k = (i & 3) * 4;
+                const int i = tid + l * NT, r = i / 4, k = (i & 3) * 4;
                 As[buf][k][r] = ra[l].x;
                 As[buf][k + 1][r] = ra[l].y;
                 As[buf][k + 2][r] = ra[l].z;
                 As[buf][k + 3][r] = ra[l].w;
-                *(float4*)&Bs[buf][i / (T / 4)][i % (T / 4) * 4] = rb[l];
             }
         };
-        float2 acc[4 * N][2 * N];
+        float2 acc[4 * N][2 * NC];
 #pragma unroll
         for (int u = 0; u < 4 * N; ++u)
 #pragma unroll
-            for (int v = 0; v < 2 * N; ++v) acc[u][v] = make_float2(0.0f, 0.0f);
-        load(0);
+            for (int v = 0; v < 2 * NC; ++v) acc[u][v] = make_float2(0.0f, 0.0f);
+        load(0, 0);
         store(0);
+        cp_async_wait<0>();
         __syncthreads();
         for (int kt = 0; kt < nk; ++kt) {
             const int buf = kt & 1;
-            if (kt + 1 < nk) load((kt + 1) * 16);
+            if (kt + 1 < nk) load((kt + 1) * 16, buf ^ 1);
 #pragma unroll
             for (int kk = 0; kk < 16; ++kk) {
-                float4 a4[N], b4[N];
+                float4 a4[N], b4[NC];
 #pragma unroll
-                for (int h = 0; h < N; ++h) {
-                    a4[h] = *(const float4*)&As[buf][kk][h * 64 + ty * 4];
-                    b4[h] = *(const float4*)&Bs[buf][kk][h * 64 + tx * 4];
-                }
+                for (int h = 0; h < N; ++h) a4[h] = *(const float4*)&As[buf][kk][h * 64 + ty * 4];
+#pragma unroll
+                for (int g = 0; g < NC; ++g) b4[g] = *(const float4*)&Bs[buf][kk][g * 4 * TX + tx * 4];
 #pragma unroll
                 for (int h = 0; h < N; ++h) {
                     const float av[4] = {a4[h].x, a4[h].y, a4[h].z, a4[h].w};
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
 #pragma unroll
-                        for (int g = 0; g < N; ++g) {
+                        for (int g = 0; g < NC; ++g) {
                             const float2 aa = make_float2(av[u], av[u]);
                             acc[4 * h + u][2 * g] = ffma2(aa, make_float2(b4[g].x, b4[g].y), acc[4 * h + u][2 * g]);
                             acc[4 * h + u][2 * g + 1] =
@@ -157,13 +167,14 @@ __global__ void __launch_bounds__(256, 2) beam_gemm_kernel(const float* __restri
                 }
             }
             if (kt + 1 < nk) store(buf ^ 1);
+            cp_async_wait<0>();
             __syncthreads();
         }
 #pragma unroll
         for (int u = 0; u < 4 * N; ++u)
 #pragma unroll
-            for (int g = 0; g < N; ++g) {
-                const int r = r0 + (u >> 2) * 64 + ty * 4 + (u & 3), c = c0 + g * 64 + tx * 4;
+            for (int g = 0; g < NC; ++g) {
+                const int r = r0 + (u >> 2) * 64 + ty * 4 + (u & 3), c = c0 + g * 4 * TX + tx * 4;
                 if (r < rows && c < in)    // in is a multiple of 8
                     *(float4*)(C + (size_t)r * in + c) = make_float4(acc[u][2 * g].x, acc[u][2 * g].y,
                                                                      acc[u][2 * g + 1].x, acc[u][2 * g + 1].y);
@@ -197,7 +208,7 @@ __device__ __forceinline__ bool before(float a, int ia, float b, int ib) {
 // Where the list would overflow (many equal scores) or T_r is out of range, the K first are found by
 // K passes over all candidates scored by the definition.
 // (rows x inputs 1024 x 4096, M = 4, K = 8: scoring every candidate with sorted lists per lane took
-// 75 ms; this form 5 ms.)
+// 75 ms, this form 3.9 ms.)
 constexpr int kBeamList = 256;     // listed candidates per warp
 
 // A warp's scratch.
@@ -561,6 +572,7 @@ aq_status run_beam(const Dims& d, const void* w, const void* codes, const void* 
     const int T = big ? 128 : 64;
     const int row_tiles = (int)((rows + T - 1) / T);
     cfg.gridDim = dim3((d.in + T - 1) / T, row_tiles < 65535 ? row_tiles : 65535);
+    cfg.blockDim = dim3(big ? kBeamGemmThreads<128> : kBeamGemmThreads<64>);
     if (aq_status e = cuda_ok(cudaLaunchKernelEx(&cfg, big ? beam_gemm_kernel<128> : beam_gemm_kernel<64>,
                                                  (const float*)E, (const float*)S, V, (int)rows, d.in),
                               "cudaLaunchKernelEx (beam cross terms)");
