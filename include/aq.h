@@ -126,22 +126,23 @@ aq_status aq_decode(const aq_layout* layout, int m, const void* planes, const vo
  * reconstruction of Sec. 3.2 / Sec. 5), accumulated in fp32. The kernel reads the first m
  * planes once (HBM-bound at batch 1); 4- and 8-bit codebooks are staged on chip. Up to batch 8,
  * and wherever that is estimated to be faster, no weight is rounded on the way: the products are
- * taken from tables of fp32 values (batch 1..2) or by 16-bit tensor-core multiplies of the stored
- * codewords themselves (above; where the books and the activations differ in type, the bf16 side
- * is scaled by powers of two into fp16, which is exact for values within 2^29 of the largest of
- * their book set, or of their token and slice). Larger layers with 8-bit codes at batch 9..16 with m <= 4 run the
- * tensor-memory kernel of aq_gemm, whose decoded weights are rounded once to fp16.
+ * taken from tables of fp32 values (batch 1..2 with 8-bit codes, batch 1 with 4-bit codes) or by
+ * 16-bit tensor-core multiplies of the stored codewords themselves (batch above, and small layers
+ * at batch 1; where the books and the activations differ in type, the bf16 side is scaled by
+ * powers of two into fp16, which is exact for values within 2^29 of the largest of their book
+ * set, or of their token and slice). Larger layers with 8-bit codes at batch 9..16 run
+ * the tensor-memory kernel of aq_gemm, whose decoded weights are rounded once to fp16.
  *   x         : device, [batch][d_in] of x_dtype (AQ_F16 or AQ_BF16), row-major
  *   y         : device, [batch][d_out] of y_dtype (AQ_F16, AQ_BF16 or AQ_F32), row-major
  *   workspace : device scratch of at least aq_gemv_workspace_bytes(layout, batch) bytes:
  *               a status word and room for fp32 partial sums of every row (one per 256-input
  *               slice and token, times up to 8 codebooks with 8-bit codes at batch 1..8; at batch
- *               9..16 it may hold the fp16 copy of bf16 activations instead). Zero-fill it once before its first
- *               use (aq_workspace_init); every
- *               call leaves it ready for the next one.
+ *               9..16 it may hold the fp16 copy of bf16 activations instead). Zero-fill it once
+ *               before its first use (aq_workspace_init); every call leaves it ready for the next
+ *               one.
  *               Calls that may overlap on the GPU must not share a workspace.
- * Enqueued with programmatic dependent launch: with 8-bit codes at batch 1..2 and 16-bit codes
- * the product (fp32 partial sums per slice, and per codebook with 8-bit codes, into the
+ * Enqueued with programmatic dependent launch: with 8-bit codes at batch 1..2 (but for small
+ * layers at batch 1) and 16-bit codes the product (fp32 partial sums per slice, and per codebook with 8-bit codes, into the
  * workspace) and a split-K reduction that sums each row's partials, scales it and writes y;
  * otherwise one kernel that writes y itself. Each waits for the preceding grid before reading
  * activations. The sums are added in a fixed order, so the result does not depend on scheduling.
@@ -164,8 +165,10 @@ aq_status aq_gemv(const aq_layout* layout, int m, const void* planes, const void
  * partial sums and their summation order are those of its own call. At batch 1 with 2^8-entry
  * codebooks the n products run as one kernel over the items of all layers and the n
  * reductions as one kernel, so the group pays the fixed cost of a call (two kernel boundaries,
- * the activation load, the first table build) once instead of n times; otherwise the layers
- * are computed one after the other, as n calls of aq_gemv.
+ * the activation load, the first table build) once instead of n times. In the one-kernel forms
+ * (see aq_gemv) the layers that split the input dimension the same way share a launch, and the
+ * tensor-memory kernel's layers the fp16 copy of x; otherwise the layers are computed one after
+ * the other, as n calls of aq_gemv.
  *   n        : 1..4 layers
  *   layouts  : n layouts with the same in_features, code_bits, book_dtype and scale_dtype
  *   m        : 1 <= m <= num_books of every layer

@@ -204,14 +204,6 @@ __device__ __forceinline__ uint4 ld_stream_v4(const void* p) {
     return r;
 }
 
-// 32-bit shared-window address of a pointer into shared memory, and plain shared loads and
-// stores through it (no generic-address conversion per access).
-__device__ __forceinline__ float lds_f32(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-    return v;
-}
-
 // Byte permute (PTX prmt, generic mode): selector nibbles pick bytes of {b:a}; a nibble
 // with bit 3 set replicates the sign bit of the picked byte.
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {

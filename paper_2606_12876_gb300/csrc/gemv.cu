@@ -1,7 +1,9 @@
 // aq_gemv: y = x * W_m^T for 1..16 tokens, W_m the prefix-m additive reconstruction
 // (Sec. 3.2 group sums, restricted to the first m codebooks as in Sec. 5; Y = W X of Sec. 2.2).
 // This file holds the dispatch and the kernels of the smallest batches and of 2^16-entry books;
-// 2..16 tokens with 4-bit codes and 3..16 with 8-bit codes run gemv_cw.cu.
+// 2..16 tokens with 4-bit codes, 3..16 with 8-bit codes and one token on small layers run
+// gemv_cw.cu, larger layers with 8-bit codes at 9..16 tokens gemm_ts.cu (gemv_uses_cw,
+// gemv_uses_ts below).
 //
 // Work split (split-K): the input dimension is cut into slices of 32 groups (256 inputs).
 // A work item is (slice, 32-row block) for the direct and gather kernels and (slice,
@@ -453,7 +455,8 @@ gemv_lut_kernel(const __grid_constant__ LutLayers L, const uint16_t* __restrict_
 template <int NB, int BDT>
 __global__ void __launch_bounds__(256)
 gemv_direct_kernel(const uint8_t* __restrict__ planes, const uint16_t* __restrict__ books,
-                   const uint16_t* __restrict__ x, int x_dt, float* __restrict__ partials, int m, int batch, int in, int rows_pad, int RBc,
+                   const uint16_t* __restrict__ x, int x_dt, float* __restrict__ partials, int m, int batch, int in,
+                   int rows_pad, int RBc,
                    int rb_per_chunk, size_t plane_bytes) {
     constexpr int UNIT = unit_bytes(16);
     constexpr int kWarps = 8;
@@ -1081,9 +1084,10 @@ aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* book
 // (status word and partial planes, laid out as for aq_gemv). At batch 1 with 2^8-entry books
 // the n products are one launch of the table-lookup kernel (the items of all layers in one
 // numbering) and the n reductions one launch; otherwise, or when a CTA's items would reach
-// into more than two layers, the layers run as n ordinary calls. In the one-kernel forms of 2..16
-// tokens the layers with the same split of K share a launch (8B block, q/k/v and gate/up in groups: see
-// the figures in gemv_cw.cu). Either way each layer's partial sums and their order are those of its own
+// into more than two layers, the layers run as n ordinary calls. In the one-kernel forms the
+// layers with the same split of K share a launch (8B block as four calls, q/k/v and gate/up in
+// groups, against seven calls: 8 tokens, m = 3 86.5 against 91.1 us, 4-bit codes, 4 tokens, m = 4
+// 92.2 against 96.3, when the group came). Either way each layer's partial sums and their order are those of its own
 // call, so the results are identical.
 aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* planes,
                             const void* const* books, const void* const* scales, const void* x,

@@ -241,8 +241,8 @@ _group_ws = {}
 
 
 def gemv_group(layers, x, m, ys=None, y_dtype=None):
-    """y_l = x W_m,l^T for AQLinear layers that share the input x (aq_gemv_group: one product
-    and one reduction launch at batch 1); returns the list of outputs."""
+    """y_l = x W_m,l^T for AQLinear layers that share the input x (aq_gemv_group: the layers
+    share launches); returns the list of outputs."""
     xd = _dtype_code(x.dtype)
     yd = xd if y_dtype is None else y_dtype
     batch = x.shape[0]
