@@ -656,7 +656,7 @@ __global__ void __launch_bounds__(1024) bf16_rows_to_f16_kernel(const uint16_t* 
         int et = 0;
         if (mx != 0) {
             const int eb = (int)((mx >> 7) & 0xffu);           // biased bf16 exponent
-            et = max(-100, min(100, (eb == 0 ? 1 : eb) - 127 - 14));
+            et = max(-126, eb - 127 - 14);     // at most 114; 2^126 makes any smaller value a normal fp16 one
         }
         const float sc = pow2f(-et);
         uint4* out = (uint4*)(dst + (size_t)t * in);

@@ -117,10 +117,9 @@ __device__ __forceinline__ float max_abs8(const uint4& v) {
     return mx;
 }
 
-// The exponent e that puts mx * 2^-e in [2^14, 2^15); 0 for 0, clamped so that 2^e and 2^-e are floats.
-__device__ __forceinline__ int f16_exponent(float mx) {
-    return mx > 0.0f ? max(-100, min(100, exponent_of(mx) - 14)) : 0;
-}
+// The exponent e that puts mx * 2^-e in [2^14, 2^15); 0 for 0. At most 114 (infinity); at least -126,
+// so that 2^-e is a float: bf16 values are multiples of 2^-133, which 2^126 makes normal fp16 values.
+__device__ __forceinline__ int f16_exponent(float mx) { return mx > 0.0f ? max(-126, exponent_of(mx) - 14) : 0; }
 
 // The codes of a row's slice unit as stored (position p holds group (p + o) mod 32), staged in group
 // order (B = 8: the groups 4j + c of each c together).

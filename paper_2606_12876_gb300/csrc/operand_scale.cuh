@@ -43,7 +43,7 @@ __device__ __forceinline__ int book_exponent(const unsigned int* wmax, int m) {
     if (!(tot > 0.0f)) return 0;             // all-zero books (or NaN entries)
     int f = exponent_of(fminf(tot, 3.0e38f)) - 14;
     if (BDT == AQ_F16 && f < 0) f = 0;
-    return max(-100, min(100, f));
+    return max(-126, f);                     // (at most 113; the smallest bf16 value is 2^-133)
 }
 
 // A codeword times sc (a power of two), back in its own type.
