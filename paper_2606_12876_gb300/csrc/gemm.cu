@@ -108,6 +108,9 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi, int dt) {
     __half2 h = __floats2half2_rn(lo, hi);
     return *(uint32_t*)&h;
 }
+__device__ __forceinline__ uint4 pack8(const float* v, int dt) {
+    return make_uint4(pack2(v[0], v[1], dt), pack2(v[2], v[3], dt), pack2(v[4], v[5], dt), pack2(v[6], v[7], dt));
+}
 
 // Decoded group (eight fp16 weights): sum of the MB codewords in fp32, in book order, rounded
 // once to fp16. code[k] is the group's code in plane k; book k starts at books + k*4096.
@@ -514,34 +517,40 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
         // Vector stores need 16-byte aligned row segments: out a multiple of 8 (the output
         // pointer itself is 16-byte aligned by contract).
         const bool vec = (out & 7) == 0;
+        const int q = warp & 3;                       // tensor-memory lane quarter
+        const int i = (warp - kDecWarp0) >> 2;        // token block (accumulator)
+        const int tw = t0 + i * 2 * kBM + (int)rank * kBM + q * 32;   // the warp's first token
+        const int t = tw + lane;
+        const float xf = (xfac && t < tokens) ? xfac[t] : 1.0f;   // 2^e_t (bf16 activations)
+        // 32 accumulators of rows nc .. nc + 31 as outputs (the order: operand_scale.cuh)
+        auto finish = [&](float (&v)[32], int nc) {
+            if (xf < 1.0f)
+#pragma unroll
+                for (int e = 0; e < 32; ++e) v[e] *= xf;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) v[e] *= scale_s[nc + e];
+            if (xf > 1.0f)
+#pragma unroll
+                for (int e = 0; e < 32; ++e) v[e] *= xf;
+        };
         if (ready && y_tma) {
             // 16-bit y by TMA stores: every MMA has completed, so the operand rings are free;
             // each warp stages its 32 tokens x 256 rows as eight 32 x 32 chunks (2 KiB each, a
             // token's 64 bytes per row of the chunk, 16-byte pieces placed by the 64-byte
             // swizzle of the store's tensor map: piece j of token row r at j ^ ((r >> 1) & 3),
             // conflict-free) and stores each chunk with one bulk tensor store.
-            const int q = warp & 3;                       // tensor-memory lane quarter
-            const int i = (warp - kDecWarp0) >> 2;        // token block (accumulator)
-            const int tw = t0 + i * 2 * kBM + (int)rank * kBM + q * 32;   // the warp's first token
-            const int t = tw + lane;
-            const float xf = (xfac && t < tokens) ? xfac[t] : 1.0f;   // 2^e_t (bf16 activations)
             const uint32_t stage = smem_u32(smem + kOffA) + (uint32_t)(warp - kDecWarp0) * (kBN / 32) * 2048u;
             const uint32_t sw = (uint32_t)(lane >> 1) & 3u;
             for (int nc = 0; nc < kBN; nc += 32) {
                 float v[32];
                 tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + i * kBN + nc, v);
-                if (xf != 1.0f)
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) v[e] *= xf;   // exact: a power of two
+                finish(v, nc);
                 const uint32_t chunk = stage + (uint32_t)(nc / 32) * 2048u;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int e = 8 * j;
                     sts128(chunk + (uint32_t)lane * 64u + (((uint32_t)j ^ sw) << 4),
-                           make_uint4(pack2(v[e] * scale_s[nc + e], v[e + 1] * scale_s[nc + e + 1], y_dt),
-                                      pack2(v[e + 2] * scale_s[nc + e + 2], v[e + 3] * scale_s[nc + e + 3], y_dt),
-                                      pack2(v[e + 4] * scale_s[nc + e + 4], v[e + 5] * scale_s[nc + e + 5], y_dt),
-                                      pack2(v[e + 6] * scale_s[nc + e + 6], v[e + 7] * scale_s[nc + e + 7], y_dt)));
+                           pack8(v + e, y_dt));
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
@@ -553,16 +562,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
             }
             __syncwarp();
         } else if (ready) {
-            const int q = warp & 3;                       // tensor-memory lane quarter
-            const int i = (warp - kDecWarp0) >> 2;        // token block (accumulator)
-            const int t = t0 + i * 2 * kBM + (int)rank * kBM + q * 32 + lane;
-            const float xf = (xfac && t < tokens) ? xfac[t] : 1.0f;   // 2^e_t (bf16 activations)
             for (int nc = 0; nc < kBN; nc += 32) {
                 float v[32];
                 tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + i * kBN + nc, v);
-                if (xf != 1.0f)
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) v[e] *= xf;   // exact: a power of two
+                finish(v, nc);
                 if (t < tokens) {
                     const size_t base = (size_t)t * out + n0 + nc;
                     if (vec && n0 + nc + 32 <= out) {
@@ -570,25 +573,20 @@ gemm_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CU
                             float4* yp = (float4*)((float*)y + base);
 #pragma unroll
                             for (int e = 0; e < 32; e += 4)
-                                yp[e / 4] = make_float4(v[e] * scale_s[nc + e], v[e + 1] * scale_s[nc + e + 1],
-                                                        v[e + 2] * scale_s[nc + e + 2], v[e + 3] * scale_s[nc + e + 3]);
+                                yp[e / 4] = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
                         } else {
                             uint4* yp = (uint4*)((uint16_t*)y + base);
 #pragma unroll
                             for (int e = 0; e < 32; e += 8)
-                                yp[e / 8] = make_uint4(pack2(v[e] * scale_s[nc + e], v[e + 1] * scale_s[nc + e + 1], y_dt),
-                                                       pack2(v[e + 2] * scale_s[nc + e + 2], v[e + 3] * scale_s[nc + e + 3], y_dt),
-                                                       pack2(v[e + 4] * scale_s[nc + e + 4], v[e + 5] * scale_s[nc + e + 5], y_dt),
-                                                       pack2(v[e + 6] * scale_s[nc + e + 6], v[e + 7] * scale_s[nc + e + 7], y_dt));
+                                yp[e / 8] = pack8(v + e, y_dt);
                         }
                     } else {
 #pragma unroll
                         for (int e = 0; e < 32; ++e) {
                             if (n0 + nc + e < out) {
-                                const float val = v[e] * scale_s[nc + e];
-                                if (y_dt == AQ_F32) ((float*)y)[base + e] = val;
-                                else if (y_dt == AQ_BF16) ((uint16_t*)y)[base + e] = f32_to_bits<AQ_BF16>(val);
-                                else ((uint16_t*)y)[base + e] = f32_to_bits<AQ_F16>(val);
+                                if (y_dt == AQ_F32) ((float*)y)[base + e] = v[e];
+                                else if (y_dt == AQ_BF16) ((uint16_t*)y)[base + e] = f32_to_bits<AQ_BF16>(v[e]);
+                                else ((uint16_t*)y)[base + e] = f32_to_bits<AQ_F16>(v[e]);
                             }
                         }
                     }

@@ -438,7 +438,8 @@ gemm_ts_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         }
         const float xf = xf_s[tl];
         const size_t yi = (size_t)(t0 + tl) * out + o;
-        const float w[4] = {v.x * xf * sc.x, v.y * xf * sc.y, v.z * xf * sc.z, v.w * xf * sc.w};
+        auto scaled = [&](float p, float s) { return p * (xf > 1.0f ? s : xf) * (xf > 1.0f ? xf : s); };   // operand_scale.cuh
+        const float w[4] = {scaled(v.x, sc.x), scaled(v.y, sc.y), scaled(v.z, sc.z), scaled(v.w, sc.w)};
         if (vec && a.y_dt == AQ_F32) {
             *(float4*)((float*)y + yi) = make_float4(w[0], w[1], w[2], w[3]);
         } else if (vec) {

@@ -19,8 +19,11 @@ __device__ __forceinline__ uint32_t f16x2(float2 v) {   // {lo, hi} -> packed fp
 // and the codebooks by 2^-f so that the largest possible |sum of m codewords| (the sum over
 // the books of their largest |entry|) lies below 2^15 (for bf16 books also at least 2^14, so
 // that small weights do not fall into fp16's subnormal range; fp16 books are only scaled down,
-// and a single fp16 book not at all). The epilogue multiplies by 2^(e_t + f). Where nothing
-// was out of range the result is bit-identical to the unscaled computation.
+// and a single fp16 book not at all). The epilogue multiplies by 2^e_t and by s 2^f: the scaled sums
+// stay below about 2^46, so the order that overflows only where y does is s 2^f first for e_t > 0 and
+// 2^e_t first otherwise. (Always 2^e_t first, activations of 2^112 and weights of 2^-4, scaled by 2^18,
+// gave infinity for y of about 2^112.) Where nothing was out of range the result is bit-identical to the
+// unscaled computation.
 
 // Largest |entry| of a codeword of eight 16-bit values, as the bits of a non-negative float
 // (monotonic in the value, so unsigned maxima of them are maxima of the values).

@@ -73,3 +73,19 @@ def test_codebook_range(out, inp, M, B, e):
     x_bits = scaled_x(100, inp, "f16", 0, seed=inp)
     for m in sorted({1, M}):
         check(layer, x_bits, "f16", m, TOKENS)
+
+
+@pytest.mark.parametrize("ew,ex", [(0, 112), (-118, 118), (100, -112), (-60, 100)])
+@pytest.mark.parametrize("out,inp,M,B", [(40, 264, 3, 8), (700, 2056, 5, 8), (72, 520, 4, 4)])
+def test_large_times_small(out, inp, M, B, ew, ex):
+    """bf16 books and activations whose scale factors together exceed the range of either."""
+    layer = scaled_layer(out, inp, M, B, "bf16", ew, seed=out)
+    x_bits = scaled_x(100, inp, "bf16", ex, seed=inp)
+    for m in sorted({1, M}):
+        check(layer, x_bits, "bf16", m, TOKENS)
+
+
+def test_large_times_small_dense():
+    """The same where W_m is decoded first (2048 tokens and more)."""
+    layer = scaled_layer(72, 264, 3, 8, "bf16", -118, seed=1)
+    check(layer, scaled_x(2048, 264, "bf16", 118, seed=2), "bf16", 3, (2048,))
