@@ -43,6 +43,7 @@
 // 14336 x 4096, 8 tokens: m = 3 17.8 us, m = 4 22.1 us; 1024 x 1024, m = 4, 16 tokens: 3.9 us.
 #include "aq_internal.cuh"
 #include "launch.cuh"
+#include "operand_scale.cuh"
 #include "tc_ptx.cuh"
 
 namespace aq {
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
             __syncthreads();
             float mx = 0.0f;
             for (int i = tid; i < a.m * NC; i += kCwThreads)
-                mx = fmaxf(mx, max_abs8<BDT>(__ldg((const uint4*)L.books + i)));
+                mx = fmaxf(mx, __uint_as_float(codeword_max_bits<BDT>(__ldg((const uint4*)L.books + i))));
             atomicMax(&s_bmax, __float_as_uint(mx));     // non-negative floats order as integers
             __syncthreads();
             const int f = f16_exponent(__uint_as_float(s_bmax));

@@ -25,15 +25,16 @@ __device__ __forceinline__ uint32_t f16x2(float2 v) {   // {lo, hi} -> packed fp
 // gave infinity for y of about 2^112.) Where nothing was out of range the result is bit-identical to the
 // unscaled computation.
 
-// Largest |entry| of a codeword of eight 16-bit values, as the bits of a non-negative float
-// (monotonic in the value, so unsigned maxima of them are maxima of the values).
+// Largest finite |entry| of a codeword of eight 16-bit values, as the bits of a non-negative float
+// (monotonic in the value, so unsigned maxima of them are maxima of the values). Infinities and NaN stay
+// what they are at any scale; counted here, one infinite entry would scale every finite one to zero.
 template <int BDT>
 __device__ __forceinline__ unsigned int codeword_max_bits(const uint4& c) {
     float f[8];
     unpack8<BDT>(c, f);
     float mx = 0.0f;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) mx = fmaxf(mx, fabsf(f[e]));
+    for (int e = 0; e < 8; ++e) mx = fmaxf(mx, fabsf(f[e]) < INFINITY ? fabsf(f[e]) : 0.0f);
     return __float_as_uint(mx);
 }
 
@@ -43,7 +44,7 @@ __device__ __forceinline__ int book_exponent(const unsigned int* wmax, int m) {
     if (BDT == AQ_F16 && m == 1) return 0;   // one fp16 codeword is an fp16 value already
     float tot = 0.0f;
     for (int k = 0; k < m; ++k) tot += __uint_as_float(wmax[k]);
-    if (!(tot > 0.0f)) return 0;             // all-zero books (or NaN entries)
+    if (!(tot > 0.0f)) return 0;             // no finite entry but zeros
     int f = exponent_of(fminf(tot, 3.0e38f)) - 14;
     if (BDT == AQ_F16 && f < 0) f = 0;
     return max(-126, f);                     // (at most 113; the smallest bf16 value is 2^-133)

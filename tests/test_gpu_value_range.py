@@ -89,3 +89,32 @@ def test_large_times_small_dense():
     """The same where W_m is decoded first (2048 tokens and more)."""
     layer = scaled_layer(72, 264, 3, 8, "bf16", -118, seed=1)
     check(layer, scaled_x(2048, 264, "bf16", 118, seed=2), "bf16", 3, (2048,))
+
+
+@pytest.mark.parametrize("bdt,xdt", [("f16", "f16"), ("f16", "bf16"), ("bf16", "f16"), ("bf16", "bf16")])
+@pytest.mark.parametrize("out,inp,M,B", [(40, 256, 3, 8), (700, 2048, 5, 8), (72, 512, 4, 4)])
+def test_infinite_codeword(out, inp, M, B, bdt, xdt):
+    """An infinite entry in a book: rows that use its codeword are not finite, the others keep their values
+    (codeword 0 stays finite: the positions past a row's last group hold code 0)."""
+    layer = scaled_layer(out, inp, M, B, bdt, 0, seed=out)
+    used = np.zeros(out, bool)
+    used[::9] = True
+    layer["codes"] = np.where(layer["codes"] == 7, 6, layer["codes"]).astype(layer["codes"].dtype)
+    layer["codes"][used, 3, 0] = 7
+    layer["books"] = np.array(layer["books"], np.uint16)
+    layer["books"][0, 7, 2] = 0x7c00 if bdt == "f16" else 0x7f80
+    x_bits = scaled_x(100, inp, xdt, 0, seed=inp)
+    finite = dict(layer, books=layer["books"].copy())
+    finite["books"][0, 7, 2] = 0
+    lin = AQLinear.from_layer(layer)
+    x = x_to_device(x_bits, xdt)
+    absl = dict(finite, books=finite["books"] & 0x7fff, scales=np.asarray(layer["scales"], np.uint16) & 0x7fff)
+    for m in sorted({1, M}):
+        ref = oracle.product_exact(finite, x_bits, xdt, m)
+        A = np.abs(_widen(x_bits, xdt)) @ np.abs(oracle.reconstruct_exact(absl, m)).T
+        for b in TOKENS:
+            y = U.to_f64((lin.gemv if b <= 16 else lin.gemm)(x[:b], m, y_dtype=aq.AQ_F32))
+            bad = ~(np.abs(y - ref[:b]) <= (2.0 ** -11 + 2.0 ** -13) * A[:b])
+            assert not bad[:, ~used].any(), "m=%d tokens=%d: %d outputs of rows that do not use it" % (
+                m, b, int(bad[:, ~used].sum()))
+            assert not np.isfinite(y[:, used]).any(), "m=%d tokens=%d" % (m, b)
