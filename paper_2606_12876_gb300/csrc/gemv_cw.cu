@@ -42,6 +42,7 @@
 // tables and tf32 kernel before: 145.8), 4-bit codes, 4 tokens, m = 4 91.1 us (fp32 kernel before: 229.7).
 // 14336 x 4096, 8 tokens: m = 3 17.8 us, m = 4 22.1 us; 1024 x 1024, m = 4, 16 tokens: 3.9 us.
 #include "aq_internal.cuh"
+#include "cw_split.h"
 #include "launch.cuh"
 #include "operand_scale.cuh"
 #include "tc_ptx.cuh"
@@ -506,22 +507,14 @@ aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, con
         // the layers with this one's cluster size: their sums are those of their own calls
         CwArgs a = {};
         a.kc = kcs[f];
-        int rbs = 0, set[4];
+        int rbs[4], set[4];
         for (int l = f; l < n; ++l)
             if (!done[l] && kcs[l] == a.kc) {
                 done[l] = true;
-                rbs += ds[l].RBc;
+                rbs[a.nlayers] = ds[l].RBc;
                 set[a.nlayers++] = l;
             }
-        // the fewest passes that the resident clusters allow over all layers
-        const int cap = cw_clusters(a.kc, tiles, di.sms);
-        int passes = (rbs + cap - 1) / cap;
-        auto need = [&](int p) {
-            int c = 0;
-            for (int i = 0; i < a.nlayers; ++i) c += (ds[set[i]].RBc + p - 1) / p;
-            return c;
-        };
-        while (a.nlayers > 1 && need(passes) > cap) ++passes;
+        const int passes = cw_group_passes(rbs, a.nlayers, cw_clusters(a.kc, tiles, di.sms));
         a.static_weights = 1;
         for (int i = 0, c0 = 0; i < a.nlayers; ++i) {
             const int l = set[i];
@@ -535,7 +528,7 @@ aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, con
             L.RBc = ds[l].RBc;
             L.plane_bytes = ds[l].plane_bytes;
             L.c0 = c0;
-            L.nclusters = a.nlayers > 1 ? (ds[l].RBc + passes - 1) / passes : own[l];
+            L.nclusters = a.nlayers > 1 ? cw_layer_clusters(ds[l].RBc, passes) : own[l];
             c0 += L.nclusters;
             if (!(ds[l].flags & AQ_LAYOUT_STATIC_WEIGHTS)) a.static_weights = 0;
         }
