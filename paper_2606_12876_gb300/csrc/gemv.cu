@@ -1036,7 +1036,7 @@ static bool gemv_uses_cw(const Dims& d, int m, int batch) {
 // clocks), which has room unless the layer has few rows. 8-bit codes only: with 4-bit codes every
 // intermediate of a GEMV is fp32 or exact, and stays so.
 static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt) {
-    if (batch <= 8 || d.B != 8) return false;
+    if (batch <= 8 || d.B != 8 || m == 1) return false;
     const size_t room = gemv_ws_planes(d, batch) * (size_t)d.rows_pad * 4;
     if (x_dt == AQ_BF16 && room < kWsStatusBytes + (size_t)batch * d.in * 2) return false;
     const double ts = ts_clocks(d, m, batch);

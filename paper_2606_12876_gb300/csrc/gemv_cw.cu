@@ -178,16 +178,18 @@ struct RowCodes {
     }
 };
 
-// CHAIN: multiplies accumulated by the tensor pipe before an fp32 add takes them over (0: all of a unit
-// and the next ones). The pipe truncates as it accumulates: over the 64 multiplies of a row and four books
-// that costs a decimal of fp32 (relative error of an fp32 y 1.2e-6; chains of eight 2e-7; fp32 sums 1.2e-7).
-// Chains of eight (3 to 10 % more time) stand where calls had fp32 sums: up to four tokens, 4-bit codes;
-// single multiplies at one token (1.1 to 1.2e-7 on the small layers that come here, as the tables).
+// CHAIN: multiplies (of 16 inputs) that the tensor pipe accumulates before an fp32 addition takes them over. The
+// pipe truncates as it accumulates, so the longer the chain, the larger the error of an fp32 y:
+//   1: the two multiplies of a step are added, then the steps of a unit, then the units of a warp: as accurate as
+//      the table kernel's fp32 sums (1.0 times its error at 1024 x 1024, 0.7 to 0.9 on longer rows);
+//   4: two steps: 0.5 to 0.95 times the error of fp32 sums in input order;
+//   0: all units of a warp (4096 x 14336, m = 1 / 4: 1.1e-6 / 4.3e-6).
 template <int B, int BDT, int XDT, int CHAIN>
 __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_constant__ CwArgs a) {
     constexpr int UNIT = unit_bytes(B), NC = 1 << B;
     constexpr int MDT = BDT == AQ_BF16 && XDT == AQ_BF16 ? AQ_BF16 : AQ_F16;   // operand type
     constexpr bool kScaleX = XDT != MDT, kScaleB = BDT != MDT;
+    constexpr int kTake = CHAIN == 4 ? 2 : 8;           // steps between the additions to the accumulators
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ unsigned int s_bmax;
     uint4* books_s = (uint4*)smem;
@@ -207,13 +209,12 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     const long long U = (long long)a.S * a.m;
     const int nwarps = kCwWarps * a.kc, gw = rank * kCwWarps + warp;
     const int u0 = (int)(U * gw / nwarps), u1 = (int)(U * (gw + 1) / nwarps);
-    const int s0 = u0 / a.m, k0 = u0 - s0 * a.m;
     struct Item {
         int rb, u, s, k;
     };
     auto next_item = [&](Item& it) {
         if (++it.u == u1) {
-            it = Item{it.rb + L.nclusters, u0, s0, k0};
+            it = Item{it.rb + L.nclusters, u0, u0 / a.m, u0 % a.m};
         } else if (++it.k == a.m) {
             it.k = 0;
             ++it.s;
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
             if constexpr (B == 8) raw[1] = ld_stream_v4(src + 16);
         }
     };
-    Item nxt{cid, u0, s0, k0};
+    Item nxt{cid, u0, u0 / a.m, u0 % a.m};
     float bfac = 1.0f;                                   // 2^f of the staged books (kScaleB)
     auto stage_books = [&]() {
         if constexpr (kScaleB) {
@@ -318,8 +319,8 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
         float* mine = rp + (size_t)warp * kCwTokens * kCwPitch;
         bool first = true;
         // the row scale of the output this thread finishes, requested before the pass's gathers
-        const int my_o = rb * 32 + (tid & 31);
-        const float my_s = tid < 32 * kCwTokens && my_o < L.out ? bits_to_f32_rt(L.scales[my_o], a.scale_dt) : 0.0f;
+        auto my_o = [&]() { return rb * 32 + (tid & 31); };
+        const uint16_t my_s = tid < 32 * kCwTokens && my_o() < L.out ? L.scales[my_o()] : (uint16_t)0;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
@@ -357,14 +358,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
             for (int rr = 0; rr < 4; ++rr) cw[rr].load(buf, g + 8 * rr, c);
             __syncwarp();                                // the buffer may be refilled
             const uint32_t base = books_u + (uint32_t)k * (NC * mul);
-            float part[2][4] = {};                       // (CHAIN > 0) the current chains
-            auto take = [&](int mt) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    acc[mt][e] += part[mt][e];
-                    part[mt][e] = 0.0f;
-                }
-            };
+            float part[2][4] = {};                       // the unit's sums (CHAIN 1), the current chain (4)
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 uint4 w[4];
@@ -372,11 +366,24 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
                 for (int rr = 0; rr < 4; ++rr) w[rr] = lds128(base + cw[rr].code(j) * mul);
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt) {
-                    float(&d)[4] = CHAIN ? part[mt] : acc[mt];
-                    mma16<MDT>(d, w[2 * mt].x, w[2 * mt + 1].x, w[2 * mt].y, w[2 * mt + 1].y, bf[j].x, bf[j].y);
-                    if (CHAIN == 1) take(mt);
-                    mma16<MDT>(d, w[2 * mt].z, w[2 * mt + 1].z, w[2 * mt].w, w[2 * mt + 1].w, bf[j].z, bf[j].w);
-                    if (CHAIN == 1 || (CHAIN == 8 && (j & 3) == 3)) take(mt);
+                    const uint4 &p = w[2 * mt], &q = w[2 * mt + 1];
+                    if constexpr (CHAIN == 1) {
+                        float d[4] = {}, e[4] = {};
+                        mma16<MDT>(d, p.x, q.x, p.y, q.y, bf[j].x, bf[j].y);
+                        mma16<MDT>(e, p.z, q.z, p.w, q.w, bf[j].z, bf[j].w);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) part[mt][i] += d[i] + e[i];
+                    } else {
+                        float(&d)[4] = CHAIN ? part[mt] : acc[mt];
+                        mma16<MDT>(d, p.x, q.x, p.y, q.y, bf[j].x, bf[j].y);
+                        mma16<MDT>(d, p.z, q.z, p.w, q.w, bf[j].z, bf[j].w);
+                    }
+                    if (CHAIN && j % kTake == kTake - 1)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            acc[mt][i] += part[mt][i];
+                            part[mt][i] = 0.0f;
+                        }
                 }
             }
         }
@@ -387,8 +394,14 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
         float* cs = csum + (pass & 1) * 32 * kCwTokens;
         float v = 0.0f;
         if (tid < 32 * kCwTokens) {
+            float t[kCwWarps];
 #pragma unroll
-            for (int w = 0; w < kCwWarps; ++w) v += rp[((size_t)w * kCwTokens + (tid >> 5)) * kCwPitch + (tid & 31)];
+            for (int w = 0; w < kCwWarps; ++w) t[w] = rp[((size_t)w * kCwTokens + (tid >> 5)) * kCwPitch + (tid & 31)];
+#pragma unroll
+            for (int n = kCwWarps / 2; n > 0; n /= 2)
+#pragma unroll
+                for (int w = 0; w < n; ++w) t[w] = t[2 * w] + t[2 * w + 1];
+            v = t[0];
             if (a.kc > 1) cs[tid] = v;
         }
         if (a.kc > 1) {
@@ -402,9 +415,9 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
                     v += p;
                 }
         }
-        const int t = tb + (tid >> 5), o = my_o;
+        const int t = tb + (tid >> 5), o = my_o();
         if (tid >= i0 && tid < i1 && t < a.batch && o < L.out) {
-            float r = v * bfac * my_s;
+            float r = v * bfac * bits_to_f32_rt(my_s, a.scale_dt);
             const size_t yi = (size_t)t * L.out + o;
             if (a.y_prev)
                 r = (a.y_dt == AQ_F32 ? ((const float*)a.y_prev)[yi]
@@ -466,11 +479,13 @@ aq_status run_cw(CwArgs a, cudaStream_t st) {
     return launch_pdl_cluster(a.kc, kern, dim3((last.c0 + last.nclusters) * a.kc, cw_tiles(a.batch)), dim3(kCwThreads), smem, st, a);
 }
 
+// The chain by what the other forms of the product give: 8-bit codes have fp32 tables up to two tokens, and one
+// book's codewords are exact everywhere; sums of several books from five tokens are otherwise rounded to 11 bits
+// (2e-4), where any chain will do. 4-bit codes: fp32 sums over the inputs in order (2 to 3e-7).
 template <int B, int BDT, int XDT>
 aq_status run_cw_chain(const CwArgs& a, cudaStream_t st) {
-    if constexpr (B == 4) return run_cw<B, BDT, XDT, 8>(a, st);
-    else if (a.batch == 1) return run_cw<B, BDT, XDT, 1>(a, st);
-    else if (a.batch <= 4) return run_cw<B, BDT, XDT, 8>(a, st);
+    if constexpr (B == 4) return run_cw<B, BDT, XDT, 4>(a, st);
+    else if (a.batch <= 4 || a.m == 1) return run_cw<B, BDT, XDT, 1>(a, st);
     else return run_cw<B, BDT, XDT, 0>(a, st);
 }
 
