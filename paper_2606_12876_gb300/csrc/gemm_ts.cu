@@ -475,7 +475,9 @@ struct TsPlan {
 // through it; a decoder warp's own chain (120 m + 165, a stage in four being its own), which bounds
 // one or two quarters and a last round of fewer than four slices. From five books the codes of a slice are
 // waited for (their registers leave no room to load them ahead), and from seven the four copies of a book
-// cost about twice the gathers; three quarters at most keep 128 registers a thread.
+// cost about twice the gathers; three quarters at most keep 128 registers a thread. Eight clusters of eight are
+// resident at once beside the preceding call's (see cw_cluster); sixteen ran in two waves (1024 x 8192, m = 2,
+// 16 tokens: 15.3 us where eight of them, 256 rows, took 7.9).
 // With a group of layers (nl > 1; the same K and number of books, so the same kc and spc each), the
 // tile height is chosen for the tiles of all of them and kc is the given one.
 bool ts_plan(const Dims* ds, int nl, int m, int tokens, const DeviceInfo& di, TsPlan* p, int only_kc = 0) {
@@ -497,15 +499,15 @@ bool ts_plan(const Dims* ds, int nl, int m, int tokens, const DeviceInfo& di, Ts
             long long tiles = 0;
             for (int l = 0; l < nl; ++l) tiles += (ds[l].out + 32 * qr - 1) / (32 * qr);
             tiles *= p->ntiles;
-            const int cap = kc == 1 ? di.sms : kc == 2 ? di.sms / 2 : kc == 4 ? di.sms * 9 / 38 : di.sms * 2 / 19;
+            const int cap = kc == 1 ? di.sms : kc == 2 ? di.sms / 2 : kc == 4 ? di.sms * 9 / 38 : di.sms / 19;
             const int spc = (d.S + kc - 1) / kc;
             const long long waves = (tiles + cap - 1) / cap;
-            const double chain = (m <= 6 ? 120.0 : 180.0) * m + (m <= 4 ? 165.0 : 565.0) + p->n * 0.3;
+            const double chain = (m <= 6 ? 120.0 : 180.0) * m + (m <= 4 ? 165.0 : 200.0) + p->n * 0.3;
             double stage_clk = p->n * 2.2 > 270.0 ? p->n * 2.2 : 270.0;
             if (qr * 53.0 * gathers + p->n * 0.45 > stage_clk) stage_clk = qr * 53.0 * gathers + p->n * 0.45;
             if (chain > stage_clk) stage_clk = chain;
             const double t = waves * (spc / 4 * 16 * stage_clk + (spc % 4 ? 16 * chain : 0.0) + 5000.0 +
-                                      (kc == 1 ? 0.0 : kc < 8 ? 1500.0 : 4500.0) + p->n * 16.0);
+                                      (kc == 1 ? 0.0 : 1500.0) + p->n * 16.0);
             if (best < 0.0 || t < best) {
                 best = t;
                 p->qr = qr;

@@ -1030,18 +1030,20 @@ static bool gemv_uses_cw(const Dims& d, int m, int batch) {
 }
 
 // Whether 9..16 tokens run the tensor-memory kernel (gemm_ts.cu): where its estimated time is below that of
-// gemv_cw with two token tiles, which gathers every codeword twice. 16 tokens: 14336 x 4096, m = 4 27.7 us
-// (gemv_cw 47.7); 4096 x 4096, m = 4 12.2 (17.8); but 1024 x 4096, m = 2 9.0 against gemv_cw's 5.3 and
-// 1024 x 1024, m = 4 10.1 against 3.9. bf16 activations are copied to the workspace first (about 3000
-// clocks), which has room unless the layer has few rows. 8-bit codes only: with 4-bit codes every
-// intermediate of a GEMV is fp32 or exact, and stays so.
+// gemv_cw with two token tiles, which gathers every codeword twice. Both estimates leave out the launch; gemm_ts's
+// is about 1500 clocks high at 16 tokens, and bf16 activations are copied to the workspace first (about 3000
+// clocks), which has room unless the layer has few rows. Over 256 to 14336 rows, 1024 to 14336 inputs and two to
+// five books the choice costs at most 11 % of the faster one. 16 tokens, fp16 x: 14336 x 4096, m = 4 24.8 us (gemv_cw
+// 41.3); 4096 x 4096, m = 4 11.5 (15.6); but 1024 x 4096, m = 2 8.2 against gemv_cw's 5.4, 1024 x 8192, m = 4
+// 19.2 against 10.6. 8-bit codes and several books only: with 4-bit codes or one book every intermediate of a
+// GEMV is fp32 or exact, and stays so.
 static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt) {
     if (batch <= 8 || d.B != 8 || m == 1) return false;
     const size_t room = gemv_ws_planes(d, batch) * (size_t)d.rows_pad * 4;
     if (x_dt == AQ_BF16 && room < kWsStatusBytes + (size_t)batch * d.in * 2) return false;
     const double ts = ts_clocks(d, m, batch);
     if (ts < 0.0) return false;
-    return ts + (x_dt == AQ_BF16 ? 3000.0 : 0.0) < cw_clocks(d, m, batch) + 5800.0;   // (+ its launch and start)
+    return ts + (x_dt == AQ_BF16 ? 3000.0 : 0.0) < cw_clocks(d, m, batch) + 1500.0;
 }
 
 // The tensor-memory kernel for n layers that share x; ws0: the first layer's workspace, whose partial-sum

@@ -434,15 +434,20 @@ inline int cw_cshift(int B, int m) { return B == 4 || m <= 5 ? 3 : 2; }
 
 // CTAs per cluster: the split with the smallest estimated time of the busiest cluster, in clocks:
 // passes over its row blocks times the units of a warp (a unit's gathers are 128 wavefronts, about
-// twice that with four copies of a book, plus about 32 of staging and the rest, shared by the SM's
-// active warps, or the latency of its eight steps) and about 1500 clocks of reduction and start-up a
-// pass, plus what a cluster launch and its barriers cost over a plain one (measured about 2 us for two
-// or four CTAs, 6 for eight: 512 x 4096, m = 4 took 10.8 us in clusters of eight).
-// Clusters of 2, 4 and 8 that are resident at once: 76, 36 and 16 on 152 SMs.
-// With several token tiles each tile has its share of the SMs.
+// twice that with four copies of a book, plus staging, conversions and sums, shared by the SM's
+// active warps, or about 2000 clocks of latencies where few are) and 1500 to 2200 clocks of reduction and
+// start-up a pass, plus what a cluster launch and its barriers cost over a plain one: 600, 1000 and 2000 clocks
+// for 2, 4 and 8 CTAs, and 2400 and 2000 more for 2 and 4 where the call's CTAs exceed half of the SMs (its
+// clusters then wait for those of the preceding kernel). Measured with the cluster size given, 8-bit
+// codes, 3 tokens, fp16 x, clusters of 1 / 2 / 4 / 8: 256 x 8192, m = 1 5.5 / 4.6 / 4.4 / 4.7 us, m = 4
+// 15.1 / 9.5 / 6.4 / 5.3; 1024 x 4096, m = 1 3.6 / 4.4 / 5.2 / 11.3, m = 4 8.6 / 6.4 / 6.1 / 14.9; 32 x 32768,
+// m = 1 16.7 / 10.2 / 6.5 / 4.5.
+// Clusters of 2, 4 and 8 that are resident at once: 76, 36 and (beside the preceding call's) 8 on 152 SMs;
+// sixteen clusters of eight took twice the time of eight (512 x 8192, m = 1: 8.8 us). With several token tiles
+// each tile has its share of the SMs.
 inline int cw_tiles(int batch) { return (batch + kCwTokens - 1) / kCwTokens; }
 inline int cw_clusters(int kc, int tiles, int sms) {
-    const int n = (kc == 1 ? sms : kc == 2 ? sms / 2 : kc == 4 ? sms * 9 / 38 : sms * 2 / 19) / tiles;
+    const int n = (kc == 1 ? sms : kc == 2 ? sms / 2 : kc == 4 ? sms * 9 / 38 : sms / 19) / tiles;
     return n < 1 ? 1 : n;
 }
 inline int cw_cluster(const Dims& d, int m, int tiles, int sms, int* nclusters, double* clocks) {
@@ -454,10 +459,11 @@ inline int cw_cluster(const Dims& d, int m, int tiles, int sms, int* nclusters, 
         const long long U = (long long)d.S * m;
         const long long units = (U + 16 * kc - 1) / (16 * kc);
         const long long active = U < 16 * kc ? (U + kc - 1) / kc : 16;
-        const double gather = cw_cshift(d.B, m) == 3 ? 160.0 : 300.0;
-        const double unit_clk = active * gather > 900.0 ? active * gather : 900.0;
-        const double t = (double)((d.RBc + nc - 1) / nc) * (units * unit_clk + (kc > 1 ? 2200.0 : 1500.0)) +
-                         (kc == 1 ? 0.0 : kc < 8 ? 3500.0 : 11000.0);
+        const double gather = cw_cshift(d.B, m) != 3 ? 300.0 : d.B == 8 ? 185.0 : 160.0;
+        const double unit_clk = active * gather > 2000.0 ? active * gather : 2000.0;
+        const bool wide = 2 * nc * kc * tiles > sms;
+        const double cluster = kc == 1 ? 0.0 : kc == 2 ? (wide ? 3000.0 : 600.0) : kc == 4 ? (wide ? 3000.0 : 1000.0) : 2000.0;
+        const double t = (double)((d.RBc + nc - 1) / nc) * (units * unit_clk + (kc > 1 ? 2200.0 : 1500.0)) + cluster;
         if (best_t < 0.0 || t < best_t) {
             best_t = t;
             best = kc;
