@@ -40,10 +40,9 @@ constexpr size_t kWsStatusBytes = 256;
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline size_t ws_partial_offset(const Dims&) { return kWsStatusBytes; }
 
-// The table-lookup GEMV (2^8-entry books) serves one token (but for the smallest layers) and two, and
-// writes one partial plane per (slice, book, token); the 2^16-entry-book kernels write one per (slice, token); the
-// remaining GEMVs (gemv_cw, gemv_lut4) need no partial planes.
-constexpr int kLutMaxBatch = 2;
+// The table-lookup GEMV (2^8-entry books; one token but for the smallest layers, two, and three or four on some
+// larger layers) writes one partial plane per (slice, book, token); the 2^16-entry-book kernels write one per
+// (slice, token); the remaining GEMVs (gemv_cw, gemv_lut4) need no partial planes.
 
 // Partial planes that a GEMV workspace has room for. The size is part of the interface (callers
 // keep workspaces across releases), so it stays what earlier kernels needed: S planes per token,

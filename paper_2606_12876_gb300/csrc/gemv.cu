@@ -1,9 +1,9 @@
 // aq_gemv: y = x * W_m^T for 1..16 tokens, W_m the prefix-m additive reconstruction
 // (Sec. 3.2 group sums, restricted to the first m codebooks as in Sec. 5; Y = W X of Sec. 2.2).
 // This file holds the dispatch and the kernels of the smallest batches and of 2^16-entry books;
-// 2..16 tokens with 4-bit codes, 3..16 with 8-bit codes and one token on small layers run
-// gemv_cw.cu, larger layers with 8-bit codes at 9..16 tokens gemm_ts.cu (gemv_uses_cw,
-// gemv_uses_ts below).
+// 2..16 tokens with 4-bit codes, most of 3..16 with 8-bit codes and one token on small layers run
+// gemv_cw.cu, larger layers with 8-bit codes at 9..16 tokens gemm_ts.cu (gemv_uses_lut4,
+// gemv_uses_cw, gemv_uses_ts below).
 //
 // Work split (split-K): the input dimension is cut into slices of 32 groups (256 inputs).
 // A work item is (slice, 32-row block) for the direct and gather kernels and (slice,
@@ -14,7 +14,7 @@
 // scales the row and stores y, with the rows spread evenly over the GPU.
 //
 // Product kernels, chosen by batch, code width and prefix:
-//  * gemv_lut (B = 8; 1 or 2 tokens). By linearity,
+//  * gemv_lut (B = 8; 1 or 2 tokens, 3 or 4 on some larger layers). By linearity,
 //    x_g . (sum_k C_k[b_k]) = sum_k T_k[g][b_k] with T_k[g][j] = x_g . C_k[j]. A persistent
 //    CTA (one per SM) walks a contiguous range of work items; for each (slice, book) it builds
 //    that book's T for the 32 groups in shared memory (32 KiB per token), then every code
@@ -37,7 +37,7 @@
 namespace aq {
 namespace {
 
-// ------------------------------------------------------------------ LUT kernel (B = 8, b <= 2)
+// ------------------------------------------------------------------ LUT kernel (B = 8, b <= 4)
 
 constexpr int kCons = 16;                         // consumer warps (two 32-row blocks each per stage)
 constexpr int kLutThreads = (kCons + 1) * 32;     // + one producer warp
@@ -46,12 +46,12 @@ constexpr int kSlot = kStageRb * 1024;            // one ring slot = one plane o
 constexpr int kSlots = 4;                         // largest ring depth (128 KiB)
 constexpr int kXStage = 8;                        // (token, slice) activation rows staged up front
 
-// Tables: 64 KiB, a half per token (NT = 1 uses the two halves for consecutive units).
-constexpr int kLutTableBytes = 65536;
+// Tables: 64 KiB per two tokens, a half per token (NT = 1 uses the two halves for consecutive units).
+constexpr int lut_table_bytes(int nt) { return nt == 4 ? 131072 : 65536; }
 
 // Shared memory: [T][codebooks m x 4 KiB][activations 8 x 1 KiB fp32][ring][barriers]
-inline size_t lut_smem_bytes(int m, int slots, int nsets = 1) {
-    return (size_t)kLutTableBytes + (size_t)nsets * m * 4096 + kXStage * 1024 +
+inline size_t lut_smem_bytes(int nt, int m, int slots, int nsets = 1) {
+    return (size_t)lut_table_bytes(nt) + (size_t)nsets * m * 4096 + kXStage * 1024 +
            (size_t)slots * kSlot + 2 * kSlots * 8;
 }
 
@@ -69,12 +69,12 @@ inline size_t lut_smem_bytes(int m, int slots, int nsets = 1) {
 // built while the other half still serves the previous unit; j*256 + g*4 is produced from a
 // code byte by one prmt.
 //
-// NT = 2 tokens: token t's table is half t, so the same prmt offset serves both tokens and the
-// token is a constant of the load: a code byte costs one prmt plus one load and one add per
-// token. The tables are rebuilt in place (a barrier first) and the partial planes are per (unit,
-// token). Three and more tokens run gemv_cw.cu: it reads 16 bytes per code byte whatever the
-// batch, the tables 4 bytes per token plus their builds (4096 x 4096, m = 4: 9.8 against 12.1 us
-// with four tokens, but 9.3 against 8.4 with two).
+// NT = 2 or 4 tokens: token t's table is half t mod 2 of the 64 KiB table t / 2, so the same prmt offset
+// serves all tokens and the token is a constant of the load: a code byte costs one prmt plus one load and
+// one add per token. The tables are rebuilt in place (a barrier first) and the partial planes are per
+// (unit, token). Three and four tokens come here only where gemv_cw.cu leaves SMs idle (gemv_uses_lut4):
+// that one reads 16 bytes per code byte whatever the batch, the tables 4 bytes per token plus their
+// builds (4096 x 4096, m = 4: 9.5 against 12.1 us with four tokens, but 9.3 against 8.4 with two).
 //
 // A CTA owns the items [i0, i1) and walks them in stages of up to 32 items that never cross a
 // unit. For each stage the producer warp copies the stage's rows of the unit's book plane into
@@ -107,11 +107,12 @@ gemv_lut_kernel(const __grid_constant__ LutLayers L, const uint16_t* __restrict_
     unsigned char* T = smem;
     const int nl = GROUP ? L.n : 1;             // layers (a single call: one, known at compile time)
     const int nsets = nl > 1 ? 2 : 1;           // codebook sets staged (layers per CTA)
-    uint4* Cb = (uint4*)(smem + kLutTableBytes);                              // [nsets][m][256] codewords
+    constexpr int kTB = lut_table_bytes(NT);
+    uint4* Cb = (uint4*)(smem + kTB);                                         // [nsets][m][256] codewords
     // [NT][kXSlices][256] activations in fp32; group g of a slice at 128-byte line g/4, its
     // two 16-byte halves at quads (2*(g%4) + half) ^ (g/4 mod 8), so the table build's reads
     // (eight lanes at eight different lines) hit eight different bank quads.
-    unsigned char* xs = smem + kLutTableBytes + (size_t)nsets * m * 4096;
+    unsigned char* xs = smem + kTB + (size_t)nsets * m * 4096;
     unsigned char* ring = xs + kXStage * 1024;                     // nslots x 32 KiB
     uint64_t* full = (uint64_t*)(ring + (size_t)nslots * kSlot);
     uint64_t* empty = full + kSlots;
@@ -352,7 +353,7 @@ gemv_lut_kernel(const __grid_constant__ LutLayers L, const uint16_t* __restrict_
 #pragma unroll 1
                     for (int t = 0; t < NT; ++t) {
                         load_xv(t);
-                        build(T + t * 128 + gq * 16);
+                        build(T + (t >> 1) * 65536 + (t & 1) * 128 + gq * 16);
                     }
                 }
                 cur_s = s;
@@ -392,7 +393,7 @@ gemv_lut_kernel(const __grid_constant__ LutLayers L, const uint16_t* __restrict_
                     const unsigned char* Tb = T + decltype(half)::value;
                     // token t of the table entry at offset o (token 0 when NT = 1)
                     auto ld = [&](uint32_t o, int t) {
-                        return *(const float*)(Tb + t * 128 + o);
+                        return *(const float*)(Tb + (t >> 1) * 65536 + (t & 1) * 128 + o);
                     };
                     if (two) {
 #pragma unroll
@@ -790,11 +791,11 @@ aq_status run_lut_layers(const Dims* ds, const GemvArgs* as, int n, int m, cudaS
     }
     const int nsets = n > 1 ? 2 : 1;
     // As many 32 KiB ring slots as fit next to the tables, codebooks and activations (<= 4).
-    const size_t fixed = lut_smem_bytes(m, 0, nsets) + 8192;   // + static shared memory and slack
+    const size_t fixed = lut_smem_bytes(NT, m, 0, nsets) + 8192;   // + static shared memory and slack
     int nslots = di.smem_optin > (int)fixed ? (int)((di.smem_optin - fixed) / kSlot) : 0;
     if (nslots > kSlots) nslots = kSlots;
     if (nslots < 2) return AQ_ERR_UNSUPPORTED;
-    const size_t smem = lut_smem_bytes(m, nslots, nsets);
+    const size_t smem = lut_smem_bytes(NT, m, nslots, nsets);
     int occ = 0;
     if (aq_status e = prepare(kern, smem, kLutThreads, m * nsets, &occ); e != AQ_OK) return e;
     LutLayers L = {};
@@ -964,8 +965,8 @@ static aq_status launch_lut4(const Dims& d, int m, const void* planes, const voi
     }
 }
 
-// The product kernels that write fp32 partial sums into the workspace: the table lookups (B = 8,
-// one or two tokens) and the 2^16-entry-book kernels.
+// The product kernels that write fp32 partial sums into the workspace: the table lookups (B = 8, up
+// to four tokens) and the 2^16-entry-book kernels.
 static aq_status launch_product(const Dims& d, int m, const GemvArgs& a, cudaStream_t st) {
     const int bb = d.book_dt == AQ_BF16, xb = a.x_dt == AQ_BF16;
     if (d.B == 16) return bb ? dispatch16<AQ_BF16>(d, m, a, st) : dispatch16<AQ_F16>(d, m, a, st);
@@ -977,11 +978,19 @@ static aq_status launch_product(const Dims& d, int m, const GemvArgs& a, cudaStr
             default: return run_lut<AQ_BF16, AQ_BF16, 1>(d, m, a, st);
         }
     }
+    if (a.batch == 2) {
+        switch (bb * 2 + xb) {
+            case 0: return run_lut<AQ_F16, AQ_F16, 2>(d, m, a, st);
+            case 1: return run_lut<AQ_F16, AQ_BF16, 2>(d, m, a, st);
+            case 2: return run_lut<AQ_BF16, AQ_F16, 2>(d, m, a, st);
+            default: return run_lut<AQ_BF16, AQ_BF16, 2>(d, m, a, st);
+        }
+    }
     switch (bb * 2 + xb) {
-        case 0: return run_lut<AQ_F16, AQ_F16, 2>(d, m, a, st);
-        case 1: return run_lut<AQ_F16, AQ_BF16, 2>(d, m, a, st);
-        case 2: return run_lut<AQ_BF16, AQ_F16, 2>(d, m, a, st);
-        default: return run_lut<AQ_BF16, AQ_BF16, 2>(d, m, a, st);
+        case 0: return run_lut<AQ_F16, AQ_F16, 4>(d, m, a, st);
+        case 1: return run_lut<AQ_F16, AQ_BF16, 4>(d, m, a, st);
+        case 2: return run_lut<AQ_BF16, AQ_F16, 4>(d, m, a, st);
+        default: return run_lut<AQ_BF16, AQ_BF16, 4>(d, m, a, st);
     }
 }
 
@@ -1018,15 +1027,30 @@ static aq_status launch_reduce(const Dims& d, int P, const GemvArgs& a, const vo
                                      (d.flags & AQ_LAYOUT_STATIC_WEIGHTS) ? 1 : 0, st);
 }
 
+// Whether three or four tokens (8-bit codes, up to four books: the two 64 KiB tables and more codebooks leave
+// room for a single code stage) run the table kernel: on layers of more row blocks than SMs, whose last pass
+// leaves SMs of gemv_cw idle, where its estimate (about 100 ns an item of an SM and 5.9 us of launches, table
+// builds and the reduction) is the smaller one. 3 tokens, fp16 books, bf16 x: 5632 x 8192, m = 4 20.6 against 26.4 us,
+// 8192 x 8192, m = 4 26.5 / 31.2, 11008 x 4096, m = 3 16.1 / 18.2; but 14336 x 4096 (three full passes), m = 4 24.3
+// against 23.6, and below 48 units the estimates are too close (11008 x 4096, m = 2 14.6 / 13.5).
+static bool gemv_uses_lut4(const Dims& d, int m, int batch, int x_dt) {
+    DeviceInfo di;
+    if (d.B != 8 || m > 4 || batch < 3 || batch > 4 || d.S * m < 48 || device_info(&di) != AQ_OK || d.RBc <= di.sms)
+        return false;
+    const double lut = 11200.0 + 185.0 * d.S * m * d.RBc / di.sms;
+    const double mixed = d.book_dt == AQ_F16 && x_dt == AQ_BF16 ? 500.0 * ((d.RBc - 1) / di.sms + 1) * ((d.S + 15) / 16) : 0.0;
+    return lut < cw_clocks(d, m, batch) + 2850.0 + mixed;
+}
+
 // Whether a call runs in one kernel (gemv_cw, or gemm_ts for 9..16 tokens): 4-bit codes at two and more
-// tokens, 8-bit codes at three and more, and at one token on small layers, with at most half a unit (slice,
+// tokens, 8-bit codes at three and more (but see gemv_uses_lut4), and at one token on small layers, with at most half a unit (slice,
 // book) per warp of a CTA and 64 row blocks. There the table kernel and its reduction take 4.0 us and two
 // launches, this one 3.75 us and one launch (1024 x 1024, m = 2: an eager call 9.3 against 12.9 us); with
 // 128 row blocks it is 4.3 against 3.95 us.
-static bool gemv_uses_cw(const Dims& d, int m, int batch) {
+static bool gemv_uses_cw(const Dims& d, int m, int batch, int x_dt) {
     if (d.B == 4) return batch >= 2;
     if (d.B != 8) return false;
-    return batch > kLutMaxBatch || (batch == 1 && d.S * m <= 8 && d.RBc <= 64);
+    return (batch > 2 && !gemv_uses_lut4(d, m, batch, x_dt)) || (batch == 1 && d.S * m <= 8 && d.RBc <= 64);
 }
 
 // Whether 9..16 tokens run the tensor-memory kernel (gemm_ts.cu): where its estimated time is below that of
@@ -1069,7 +1093,7 @@ aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* book
     if (d.out == 0 || batch == 0) return AQ_OK;
     if (d.B == 4 && batch == 1)
         return launch_lut4(d, m, planes, books, scales, x, x_dt, y, y_dt, y_prev, st);
-    if (gemv_uses_cw(d, m, batch)) {
+    if (gemv_uses_cw(d, m, batch, x_dt)) {
         if (!y_prev && gemv_uses_ts(d, m, batch, x_dt))
             return launch_gemv_ts(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, ws, ws, st);
         return launch_cw(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, y_prev, st);
@@ -1100,7 +1124,7 @@ aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* pla
     for (int l = 0; l < n; ++l) any_rows |= ds[l].out > 0;
     if (!any_rows) return AQ_OK;
     bool fused = n >= 2 && batch == 1 && ds[0].B == 8;
-    for (int l = 0; l < n && fused; ++l) fused = ds[l].out > 0 && !gemv_uses_cw(ds[l], m, 1);
+    for (int l = 0; l < n && fused; ++l) fused = ds[l].out > 0 && !gemv_uses_cw(ds[l], m, 1, x_dt);
     if (fused) {
         Dims dd[kGroupMax];
         GemvArgs as[kGroupMax];
@@ -1128,7 +1152,7 @@ aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* pla
         if (e != AQ_ERR_UNSUPPORTED) return e;   // nothing was launched for UNSUPPORTED
     }
     bool cw = true;
-    for (int l = 0; l < n; ++l) cw = cw && gemv_uses_cw(ds[l], m, batch);
+    for (int l = 0; l < n; ++l) cw = cw && gemv_uses_cw(ds[l], m, batch, x_dt);
     if (cw) {
         // The layers that the tensor-memory kernel serves share the copy of x and launches; the others
         // share launches of gemv_cw.
