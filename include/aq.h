@@ -162,13 +162,14 @@ aq_status aq_gemv(const aq_layout* layout, int m, const void* planes, const void
  * reconstruction of Sec. 3.2 / Sec. 5 for several layers that read the same activations,
  * such as a decoder block's query, key and value projections, or its gate and up projections.)
  * y_l = x * W_m,l^T for l < n, each as aq_gemv would compute it, bit for bit: every layer's
- * partial sums and their summation order are those of its own call. At batch 1 with 2^8-entry
- * codebooks the n products run as one kernel over the items of all layers and the n
- * reductions as one kernel, so the group pays the fixed cost of a call (two kernel boundaries,
- * the activation load, the first table build) once instead of n times. In the one-kernel forms
- * (see aq_gemv) the layers that split the input dimension the same way share a launch, and the
- * tensor-memory kernel's layers the fp16 copy of x; otherwise the layers are computed one after
- * the other, as n calls of aq_gemv.
+ * partial sums and their summation order are those of its own call. The layers whose own calls
+ * take the same form share launches, so the group pays the fixed cost of a call (kernel
+ * boundaries, the activation load, the first table build) once instead of n times: at batch 1
+ * with 2^8-entry codebooks the table kernel's products run as one kernel over the items of all
+ * its layers and their reductions as one kernel; in the one-kernel forms (see aq_gemv) the layers
+ * that split the input dimension the same way share a launch, and the tensor-memory kernel's
+ * layers the fp16 copy of x. Layers of other forms are computed one after the other, as calls of
+ * aq_gemv.
  *   n        : 1..4 layers
  *   layouts  : n layouts with the same in_features, code_bits, book_dtype and scale_dtype
  *   m        : 1 <= m <= num_books of every layer

@@ -95,7 +95,8 @@ aq_status launch_decode(const Dims& d, int m, const void* planes, const void* bo
 // y_prev (optional): added to the product (y = y_prev + product), read in y's type.
 aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* books,
                       const void* scales, const void* x, int x_dt, int batch, void* y,
-                      int y_dt, void* ws, cudaStream_t st, const void* y_prev = nullptr);
+                      int y_dt, void* ws, cudaStream_t st, const void* y_prev = nullptr,
+                      void* status = nullptr);
 // The same for up to 16 tokens with 4- or 8-bit codes in one kernel (gemv_cw.cu), for n (<= 4) layers that
 // share x, the code width, the types and m (n = 1: an ordinary call).
 aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, const void* const* books,

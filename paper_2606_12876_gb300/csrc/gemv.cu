@@ -1089,17 +1089,18 @@ static aq_status launch_gemv_ts(const Dims* ds, int n, int m, const void* const*
 
 aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* books,
                       const void* scales, const void* x, int x_dt, int batch, void* y,
-                      int y_dt, void* ws, cudaStream_t st, const void* y_prev) {
+                      int y_dt, void* ws, cudaStream_t st, const void* y_prev, void* status) {
     if (d.out == 0 || batch == 0) return AQ_OK;
+    if (!status) status = ws;
     if (d.B == 4 && batch == 1)
         return launch_lut4(d, m, planes, books, scales, x, x_dt, y, y_dt, y_prev, st);
     if (gemv_uses_cw(d, m, batch, x_dt)) {
         if (!y_prev && gemv_uses_ts(d, m, batch, x_dt))
-            return launch_gemv_ts(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, ws, ws, st);
+            return launch_gemv_ts(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, ws, status, st);
         return launch_cw(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, y_prev, st);
     }
     GemvArgs a{planes, books, scales, x, x_dt, batch, y, y_dt,
-               (float*)((char*)ws + ws_partial_offset(d)), (unsigned int*)ws};
+               (float*)((char*)ws + ws_partial_offset(d)), (unsigned int*)status};
     if (aq_status e = launch_product(d, m, a, st); e != AQ_OK) return e;
     const int P = d.B == 8 ? d.S * m : d.S;   // partial planes per token
     return d.scale_dt == AQ_BF16 ? launch_reduce<AQ_BF16>(d, P, a, y_prev, st)
@@ -1107,86 +1108,89 @@ aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* book
 }
 
 // aq_gemv_group: n layers that share the activations x. ws[l] is layer l's workspace region
-// (status word and partial planes, laid out as for aq_gemv). At batch 1 with 2^8-entry books
-// the n products are one launch of the table-lookup kernel (the items of all layers in one
-// numbering) and the n reductions one launch; otherwise, or when a CTA's items would reach
-// into more than two layers, the layers run as n ordinary calls. In the one-kernel forms the
-// layers with the same split of K share a launch (8B block as four calls, q/k/v and gate/up in
-// groups, against seven calls: 8 tokens, m = 3 86.5 against 91.1 us, 4-bit codes, 4 tokens, m = 4
-// 92.2 against 96.3, when the group came). Either way each layer's partial sums and their order are those of its own
-// call, so the results are identical.
+// (status word and partial planes, laid out as for aq_gemv). The layers are parted by the form that
+// their own calls take, and those of a form share launches:
+//  * gemv_cw and gemm_ts: the layers with the same split of K share a launch, and the tensor-memory layers
+//    the fp16 copy of x (8B block as four calls, q/k/v and gate/up in groups, against seven calls: 8
+//    tokens, m = 3 86.5 against 91.1 us, 4-bit codes, 4 tokens, m = 4 92.2 against 96.3, when the group came);
+//  * the table kernel at one token: the products are one launch (the items of all layers in one numbering)
+//    and the reductions one launch, unless a CTA's items would reach into more than two layers;
+//  * the others run as ordinary calls.
+// Either way each layer's partial sums and their order are those of its own call, so the results are
+// identical. (4096, 1024 and 1024 rows, 1024 inputs, m = 2, one token, the first layer by tables and the others by
+// gemv_cw: 8.1 us; as three calls 10.7; all three by tables, which the small layers' own calls are not, 5.8.)
 aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* planes,
                             const void* const* books, const void* const* scales, const void* x,
                             int x_dt, int batch, void* const* y, int y_dt, void* const* ws,
                             cudaStream_t st) {
     if (batch == 0) return AQ_OK;
-    bool any_rows = false;
-    for (int l = 0; l < n; ++l) any_rows |= ds[l].out > 0;
-    if (!any_rows) return AQ_OK;
-    bool fused = n >= 2 && batch == 1 && ds[0].B == 8;
-    for (int l = 0; l < n && fused; ++l) fused = ds[l].out > 0 && !gemv_uses_cw(ds[l], m, 1, x_dt);
-    if (fused) {
-        Dims dd[kGroupMax];
-        GemvArgs as[kGroupMax];
-        int flags = AQ_LAYOUT_STATIC_WEIGHTS;
-        for (int l = 0; l < n; ++l) {
-            dd[l] = ds[l];
-            flags &= ds[l].flags;
-            as[l] = GemvArgs{planes[l], books[l], scales[l], x, x_dt, batch, y[l], y_dt,
-                             (float*)((char*)ws[l] + ws_partial_offset(ds[l])), (unsigned int*)ws[0]};
-        }
-        dd[0].flags = flags;   // prefetch before the grid wait only if every layer's weights are static
-        const int bb = ds[0].book_dt == AQ_BF16, xb = x_dt == AQ_BF16;
-        aq_status e;
-        switch (bb * 2 + xb) {
-            case 0: e = run_lut_layers<AQ_F16, AQ_F16, 1>(dd, as, n, m, st); break;
-            case 1: e = run_lut_layers<AQ_F16, AQ_BF16, 1>(dd, as, n, m, st); break;
-            case 2: e = run_lut_layers<AQ_BF16, AQ_F16, 1>(dd, as, n, m, st); break;
-            default: e = run_lut_layers<AQ_BF16, AQ_BF16, 1>(dd, as, n, m, st); break;
-        }
-        if (e == AQ_OK) {
-            const int P = ds[0].S * m, sw = flags ? 1 : 0;
-            return ds[0].scale_dt == AQ_BF16 ? launch_reduce_layers<AQ_BF16>(dd, as, n, P, nullptr, sw, st)
-                                             : launch_reduce_layers<AQ_F16>(dd, as, n, P, nullptr, sw, st);
-        }
-        if (e != AQ_ERR_UNSUPPORTED) return e;   // nothing was launched for UNSUPPORTED
+    enum { kCw, kTs, kTables, kOther, kForms };
+    struct Part {
+        Dims d[kGroupMax];
+        const void *planes[kGroupMax], *books[kGroupMax], *scales[kGroupMax];
+        void *y[kGroupMax], *ws[kGroupMax];
+        int n;
+    } parts[kForms] = {};
+    for (int l = 0; l < n; ++l) {
+        if (ds[l].out == 0) continue;
+        const int form = gemv_uses_cw(ds[l], m, batch, x_dt) ? (gemv_uses_ts(ds[l], m, batch, x_dt) ? kTs : kCw)
+                         : ds[l].B == 8 && batch == 1        ? kTables
+                                                             : kOther;
+        Part& p = parts[form];
+        p.d[p.n] = ds[l];
+        p.planes[p.n] = planes[l];
+        p.books[p.n] = books[l];
+        p.scales[p.n] = scales[l];
+        p.ws[p.n] = ws[l];
+        p.y[p.n++] = y[l];
     }
-    bool cw = true;
-    for (int l = 0; l < n; ++l) cw = cw && gemv_uses_cw(ds[l], m, batch, x_dt);
-    if (cw) {
-        // The layers that the tensor-memory kernel serves share the copy of x and launches; the others
-        // share launches of gemv_cw.
-        struct {
-            Dims d[kGroupMax];
-            const void *planes[kGroupMax], *books[kGroupMax], *scales[kGroupMax];
-            void *y[kGroupMax], *ws0;
-            int n;
-        } part[2] = {};
-        for (int l = 0; l < n; ++l) {
-            if (ds[l].out == 0) continue;
-            auto& p = part[gemv_uses_ts(ds[l], m, batch, x_dt) ? 1 : 0];
-            if (p.n == 0) p.ws0 = ws[l];
-            p.d[p.n] = ds[l];
-            p.planes[p.n] = planes[l];
-            p.books[p.n] = books[l];
-            p.scales[p.n] = scales[l];
-            p.y[p.n++] = y[l];
-        }
-        if (part[1].n > 0)
-            if (aq_status e = launch_gemv_ts(part[1].d, part[1].n, m, part[1].planes, part[1].books, part[1].scales, x,
-                                             x_dt, batch, part[1].y, y_dt, part[1].ws0, ws[0], st);
-                e != AQ_OK)
-                return e;
-        if (part[0].n > 0)
-            return launch_cw(part[0].d, part[0].n, m, part[0].planes, part[0].books, part[0].scales, x, x_dt, batch,
-                             part[0].y, y_dt, nullptr, st);
-        return AQ_OK;
-    }
-    for (int l = 0; l < n; ++l)
-        if (aq_status e = launch_gemv(ds[l], m, planes[l], books[l], scales[l], x, x_dt, batch, y[l],
-                                      y_dt, ws[l], st, nullptr);
+    if (const Part& p = parts[kTs]; p.n > 0)
+        if (aq_status e = launch_gemv_ts(p.d, p.n, m, p.planes, p.books, p.scales, x, x_dt, batch, p.y, y_dt, p.ws[0],
+                                         ws[0], st);
             e != AQ_OK)
             return e;
+    if (const Part& p = parts[kCw]; p.n > 0)
+        if (aq_status e = launch_cw(p.d, p.n, m, p.planes, p.books, p.scales, x, x_dt, batch, p.y, y_dt, nullptr, st);
+            e != AQ_OK)
+            return e;
+    Part& t = parts[kTables];
+    if (t.n > 1) {
+        GemvArgs as[kGroupMax];
+        int flags = AQ_LAYOUT_STATIC_WEIGHTS;
+        for (int l = 0; l < t.n; ++l) {
+            flags &= t.d[l].flags;
+            as[l] = GemvArgs{t.planes[l], t.books[l], t.scales[l], x, x_dt, batch, t.y[l], y_dt,
+                             (float*)((char*)t.ws[l] + ws_partial_offset(t.d[l])), (unsigned int*)ws[0]};
+        }
+        const int own = t.d[0].flags;
+        t.d[0].flags = flags;   // prefetch before the grid wait only if every layer's weights are static
+        const int bb = t.d[0].book_dt == AQ_BF16, xb = x_dt == AQ_BF16;
+        aq_status e;
+        switch (bb * 2 + xb) {
+            case 0: e = run_lut_layers<AQ_F16, AQ_F16, 1>(t.d, as, t.n, m, st); break;
+            case 1: e = run_lut_layers<AQ_F16, AQ_BF16, 1>(t.d, as, t.n, m, st); break;
+            case 2: e = run_lut_layers<AQ_BF16, AQ_F16, 1>(t.d, as, t.n, m, st); break;
+            default: e = run_lut_layers<AQ_BF16, AQ_BF16, 1>(t.d, as, t.n, m, st); break;
+        }
+        if (e == AQ_OK) {
+            const int P = t.d[0].S * m, sw = flags ? 1 : 0;
+            e = t.d[0].scale_dt == AQ_BF16 ? launch_reduce_layers<AQ_BF16>(t.d, as, t.n, P, nullptr, sw, st)
+                                           : launch_reduce_layers<AQ_F16>(t.d, as, t.n, P, nullptr, sw, st);
+            if (e != AQ_OK) return e;
+            t.n = 0;
+        } else if (e != AQ_ERR_UNSUPPORTED) {
+            return e;           // nothing was launched for UNSUPPORTED
+        }
+        t.d[0].flags = own;
+    }
+    for (int form = kTables; form < kForms; ++form)
+        for (int l = 0; l < parts[form].n; ++l) {
+            const Part& p = parts[form];
+            if (aq_status e = launch_gemv(p.d[l], m, p.planes[l], p.books[l], p.scales[l], x, x_dt, batch, p.y[l], y_dt,
+                                          p.ws[l], st, nullptr, ws[0]);
+                e != AQ_OK)
+                return e;
+        }
     return AQ_OK;
 }
 
