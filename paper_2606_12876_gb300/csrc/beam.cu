@@ -205,8 +205,10 @@ __device__ __forceinline__ bool before(float a, int ia, float b, int ib) {
 // eps: both forms add up products bounded by the terms of T_r = |score_r| + lambda (D^T |S_gg| D +
 // 2 D . |h|), D = |w_g| + |s| (|P_r| + max_c |C_t[c]|), each term with at most about 30 roundings of
 // 2^-24 and the expanded form with four such sums: eps = 2^-16 max_r T_r covers their sum twice.
-// Where the list would overflow (many equal scores) or T_r is out of range, the K first are found by
-// K passes over all candidates scored by the definition.
+// Where the list would overflow (many equal scores) or T_r is out of range, every candidate is scored by the
+// definition, once, and the list holds the best so far. (512 x 2048, M = 4, K = 8: equal codewords in every book
+// 9.9 ms, half of the rows of zero scale 5.7, half of the inputs without energy in H, which needs no scores,
+// 1.2; scored anew for each of the K, 60.3, 30.8 and 35.7; sorted lists per lane 14.4, 18.2 and 19.5.)
 // (rows x inputs 1024 x 4096, M = 4, K = 8: scoring every candidate with sorted lists per lane took
 // 75 ms, this form 3.9 ms.)
 constexpr int kBeamList = 256;     // listed candidates per warp
@@ -396,6 +398,7 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
             };
             // magnitude bound T_r, and the expanded form's G_r and A_r: four lanes per state
             float tot = 0.0f;
+            bool differ = false;                       // scores of one state's candidates may differ
             // (eight states, or all sixteen places: the estimates read no further)
             for (int r = lane >> 2; r < (nstates > 8 ? kBeamMaxK : 8); r += 8) {
                 float ga[2], au = 0.0f, tr = 0.0f;
@@ -437,15 +440,18 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
                 if ((lane & 3) == 0) bw.A[r] = r < nstates ? fmaf(lt, au, cur.score[rr]) : FLT_MAX;
                 const float T = fmaf(lt, tr, fabsf(cur.score[rr]));
                 tot = fmaxf(tot, T < 1.0e36f ? T : FLT_MAX);   // (a NaN counts as too large)
+                differ = differ || !(lt * tr == 0.0f);
             }
+            differ = __any_sync(0xffffffffu, differ);
 #pragma unroll
             for (int sh = 16; sh >= 4; sh >>= 1)
                 tot = fmaxf(tot, __shfl_xor_sync(0xffffffffu, tot, sh));
             __syncwarp();
             int n = -1;                                // listed candidates (-1: no list)
-            if (tot < 1.0e36f && (lt == 0.0f || tot > 1.0e-30f)) {   // (below, products underflow)
-                if (lt == 0.0f) {
-                    // every candidate has its state's score: the first `keep` indices are the first
+            if (tot < 1.0e36f && (!differ || tot > 1.0e-30f)) {   // (below, products underflow)
+                if (!differ) {
+                    // every candidate has its state's score (a prefix weight of zero; an input that H has no
+                    // energy for: the terms of T_r bound the score's): the first `keep` indices are the first
                     if (lane < keep) bw.lidx[lane] = lane;
                     n = keep;
                 } else if (nb < 256) {                 // at most 256 candidates: all of them
@@ -494,36 +500,81 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
                 }
                 if (lane < n && rank < keep) keep_state(rank, j, sc);
             } else {
-                // K rounds: the first candidate after the last kept one, of the list or of all
-                if (n >= 0)
-                    for (int i = lane; i < n; i += 32) bw.lscore[i] = score(bw.lidx[i]);
-                __syncwarp();
-                float ps = -FLT_MAX;
-                int pj = -1;
-                for (int i = 0; i < keep; ++i) {
-                    float bs = FLT_MAX;
-                    int bj = 0x7fffffff;
-                    for (int q = lane; q < (n >= 0 ? n : ncand); q += 32) {
-                        const int j = n >= 0 ? bw.lidx[q] : q;
-                        const float sc = n >= 0 ? bw.lscore[q] : score(j);
-                        if ((i == 0 || before(ps, pj, sc, j)) && before(sc, j, bs, bj)) {
-                            bs = sc;
-                            bj = j;
+                // The first `keep` of the list's first n places in order, rank by rank: each round a minimum over the
+                // candidates after the last one taken.
+                auto in_order = [&](int n, auto take) {
+                    float ps = -FLT_MAX;
+                    int pj = -1;
+                    for (int i = 0; i < keep; ++i) {
+                        float bs = FLT_MAX;
+                        int bj = 0x7fffffff;
+                        for (int q = lane; q < n; q += 32) {
+                            const int j = bw.lidx[q];
+                            const float sc = bw.lscore[q];
+                            if ((i == 0 || before(ps, pj, sc, j)) && before(sc, j, bs, bj)) {
+                                bs = sc;
+                                bj = j;
+                            }
                         }
-                    }
 #pragma unroll
-                    for (int sh = 16; sh > 0; sh >>= 1) {
-                        const float os = __shfl_xor_sync(0xffffffffu, bs, sh);
-                        const int oj = __shfl_xor_sync(0xffffffffu, bj, sh);
-                        if (before(os, oj, bs, bj)) {
-                            bs = os;
-                            bj = oj;
+                        for (int sh = 16; sh > 0; sh >>= 1) {
+                            const float os = __shfl_xor_sync(0xffffffffu, bs, sh);
+                            const int oj = __shfl_xor_sync(0xffffffffu, bj, sh);
+                            if (before(os, oj, bs, bj)) {
+                                bs = os;
+                                bj = oj;
+                            }
+                        }
+                        ps = bs;
+                        pj = min(bj, ncand - 1);       // every round finds one; only guards the index
+                        take(i, pj, ps);
+                    }
+                };
+                if (n >= 0) {
+                    for (int i = lane; i < n; i += 32) bw.lscore[i] = score(bw.lidx[i]);
+                } else {
+                    // No list: every candidate is scored once, in index order, and listed if it comes before the
+                    // keep-th best of those that the list has been cut down to. (Where all tie, nothing after
+                    // the first list is.)
+                    float ks = FLT_MAX;
+                    int kj = 0x7fffffff;
+                    n = 0;
+                    for (int q = 0; q < ncand; q += 32) {
+                        const int j = q + lane;
+                        const float sc = j < ncand ? score(j) : FLT_MAX;
+                        const bool add = j < ncand && before(sc, j, ks, kj);
+                        const uint32_t adds = __ballot_sync(0xffffffffu, add);
+                        if (add) {
+                            const int at = n + __popc(adds & ((1u << lane) - 1u));
+                            bw.lidx[at] = j;
+                            bw.lscore[at] = sc;
+                        }
+                        n += __popc(adds);
+                        if (n > kBeamList - 32) {      // no room for 32 more
+                            __syncwarp();
+                            float ws = 0.0f;           // the candidate of rank `lane`
+                            int wj = 0;
+                            in_order(n, [&](int i, int j2, float s2) {
+                                if (i == lane) {
+                                    ws = s2;
+                                    wj = j2;
+                                }
+                                ks = s2;
+                                kj = j2;
+                            });
+                            __syncwarp();
+                            if (lane < keep) {
+                                bw.lidx[lane] = wj;
+                                bw.lscore[lane] = ws;
+                            }
+                            n = keep;
                         }
                     }
-                    ps = bs;
-                    pj = min(bj, ncand - 1);           // every round finds one; only guards the index
-                    if (lane == 0) keep_state(i, pj, ps);
                 }
+                __syncwarp();
+                in_order(n, [&](int i, int j, float sc) {
+                    if (lane == 0) keep_state(i, j, sc);
+                });
             }
             __syncwarp();
             nstates = keep;
