@@ -204,7 +204,11 @@ __device__ __forceinline__ bool before(float a, int ia, float b, int ib) {
 //     the K first of them are the K first of all: the result is the full search's, bit for bit.
 // eps: both forms add up products bounded by the terms of T_r = |score_r| + lambda (D^T |S_gg| D +
 // 2 D . |h|), D = |w_g| + |s| (|P_r| + max_c |C_t[c]|), each term with at most about 30 roundings of
-// 2^-24 and the expanded form with four such sums: eps = 2^-16 max_r T_r covers their sum twice.
+// 2^-24 and the expanded form with four such sums: eps = 2^-16 max_r T_r covers their sum twice. What products
+// lose below fp32's normal range (2^-149 each, times the factors that follow) is at most about
+// 2^-140 lambda (1 + |s|)^2 (2 + max |C_t| + max D), and is kept below eps / 4; the estimates are not used where
+// that, C_t[c]^T S_gg C_t[c] or lambda s^2 is out of range (codebooks of 2^62 and scales of 2^-68 overflowed the
+// table, and only the smallest codewords were found).
 // Where the list would overflow (many equal scores) or T_r is out of range, every candidate is scored by the
 // definition, once, and the list holds the best so far. (512 x 2048, M = 4, K = 8: equal codewords in every book
 // 9.9 ms, half of the rows of zero scale 5.7, half of the inputs without energy in H, which needs no scores,
@@ -308,7 +312,9 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
     float* Q = (float*)(hi + (size_t)M * nb);          // [M][nb] C^T S_gg C
     float* Sgg = Q + (size_t)M * nb;                   // [8][8]
     unsigned int* cmax = (unsigned int*)(Sgg + 64);    // [M][8] max |C_t[c]_e| (float bits)
-    BeamWarp& bw = ((BeamWarp*)(cmax + 64))[threadIdx.x >> 5];
+    unsigned int* qmax = cmax + 64;                    // max |Q| (infinities and NaN are the largest)
+    float* csum = (float*)(qmax + 1);                  // sum of all of cmax; infinity if Q is out of range
+    BeamWarp& bw = ((BeamWarp*)(qmax + 4))[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     pdl_wait();
     pdl_launch_dependents();
@@ -316,6 +322,7 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
     for (int i = threadIdx.x; i < 64; i += blockDim.x) {
         Sgg[i] = S[(size_t)(g * 8 + i / 8) * in + g * 8 + i % 8];
         cmax[i] = 0u;
+        if (i == 0) *qmax = 0u;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < M * nb; i += blockDim.x) {
@@ -333,6 +340,13 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
             atomicMax(&cmax[(i >> B) * 8 + e], __float_as_uint(fabsf(cv[e])));
         }
         Q[i] = q;
+        atomicMax(qmax, __float_as_uint(fabsf(q)));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float sum = 0.0f;
+        for (int i = 0; i < M * 8; ++i) sum += __uint_as_float(cmax[i]);
+        *csum = __uint_as_float(*qmax) < 1.0e37f ? sum : INFINITY;
     }
     __syncthreads();
 
@@ -357,6 +371,11 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
             bw.st[0].codes[0] = 0ull;
         }
         __syncwarp();
+        // What the estimates lose by underflow, over lambda, and eps / 4 of it as a bound of T (2^-122)
+        float wmax = 0.0f;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) wmax = fmaxf(wmax, fabsf(wg[e]));
+        const float s1 = 1.0f + fabsf(s), tmin = 1.8807909e-37f * s1 * s1 * (2.0f + wmax + s1 * *csum);
         int nstates = 1;
         for (int t = 0; t < M; ++t) {
             const BeamWarp::States& cur = bw.st[t & 1];
@@ -447,8 +466,10 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
             for (int sh = 16; sh >= 4; sh >>= 1)
                 tot = fmaxf(tot, __shfl_xor_sync(0xffffffffu, tot, sh));
             __syncwarp();
+            const float F = lt * s * s;
+            const bool fine = tot > fmaxf(1.0e-30f, lt * tmin) && F >= FLT_MIN && lt >= FLT_MIN;
             int n = -1;                                // listed candidates (-1: no list)
-            if (tot < 1.0e36f && (!differ || tot > 1.0e-30f)) {   // (below, products underflow)
+            if (tot < 1.0e36f && (!differ || nb < 256 || fine)) {
                 if (!differ) {
                     // every candidate has its state's score (a prefix weight of zero; an input that H has no
                     // energy for: the terms of T_r bound the score's): the first `keep` indices are the first
@@ -458,7 +479,7 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
                     for (int j = lane; j < ncand; j += 32) bw.lidx[j] = j;
                     n = ncand;
                 } else {
-                    const float F = lt * s * s, slack = 3.0517578125e-5f * tot;   // 2 eps
+                    const float slack = 3.0517578125e-5f * tot;   // 2 eps
                     const float* Qt = Q + (size_t)t * nb;
                     uint32_t rmask, cmask;
                     if (nstates <= 2)
@@ -586,7 +607,7 @@ beam_kernel(const uint16_t* __restrict__ w, const uint16_t* __restrict__ books,
 }
 
 inline size_t beam_smem(int M, int B) {
-    return ((size_t)M << B) * 9 * 4 + 64 * 4 + 64 * 4 + kBeamWarps * sizeof(BeamWarp);
+    return ((size_t)M << B) * 9 * 4 + (64 + 64 + 4) * 4 + kBeamWarps * sizeof(BeamWarp);
 }
 
 template <int BDT, int SDT>
