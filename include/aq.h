@@ -125,13 +125,14 @@ aq_status aq_decode(const aq_layout* layout, int m, const void* planes, const vo
  * y[t, o] = sum_i x[t, i] * W_m[o, i] for t < batch (Sec. 2.2 Y = W X, with W_m the prefix-m
  * reconstruction of Sec. 3.2 / Sec. 5), accumulated in fp32. The kernel reads the first m
  * planes once (HBM-bound at batch 1); 4- and 8-bit codebooks are staged on chip. Up to batch 8,
- * and wherever that is estimated to be faster, no weight is rounded on the way: the products are
- * taken from tables of fp32 values (batch 1..2 with 8-bit codes, batch 1 with 4-bit codes) or by
- * 16-bit tensor-core multiplies of the stored codewords themselves (batch above, and small layers
- * at batch 1; where the books and the activations differ in type, the bf16 side is scaled by
- * powers of two into fp16, which is exact for values within 2^29 of the largest of their book
- * set, or of their token and slice). Larger layers with 8-bit codes at batch 9..16 run
- * the tensor-memory kernel of aq_gemm, whose decoded weights are rounded once to fp16.
+ * with one book or 4-bit codes, and wherever that is estimated to be faster, no weight is rounded on
+ * the way: the products are taken from tables of fp32 values (8-bit codes at batch 1..2 and, on some
+ * larger layers, 3..4; 4-bit codes at batch 1) or by 16-bit tensor-core multiplies of the stored
+ * codewords themselves (batch above, and small layers at batch 1; where the books and the
+ * activations differ in type, the bf16 side is scaled by powers of two into fp16, over all of bf16's
+ * range, which is exact for values within 2^29 of the largest finite one of their book set, or of their
+ * token and slice). Larger layers with two or more 8-bit books at batch 9..16 run the tensor-memory
+ * kernel of aq_gemm: decoded weights rounded once to fp16, bf16 activations scaled by token.
  *   x         : device, [batch][d_in] of x_dtype (AQ_F16 or AQ_BF16), row-major
  *   y         : device, [batch][d_out] of y_dtype (AQ_F16, AQ_BF16 or AQ_F32), row-major
  *   workspace : device scratch of at least aq_gemv_workspace_bytes(layout, batch) bytes:
@@ -141,17 +142,22 @@ aq_status aq_decode(const aq_layout* layout, int m, const void* planes, const vo
  *               before its first use (aq_workspace_init); every call leaves it ready for the next
  *               one.
  *               Calls that may overlap on the GPU must not share a workspace.
- * Enqueued with programmatic dependent launch: with 8-bit codes at batch 1..2 (but for small
- * layers at batch 1) and 16-bit codes the product (fp32 partial sums per slice, and per codebook with 8-bit codes, into the
- * workspace) and a split-K reduction that sums each row's partials, scales it and writes y;
- * otherwise one kernel that writes y itself. Each waits for the preceding grid before reading
- * activations. The sums are added in a fixed order, so the result does not depend on scheduling.
+ * Enqueued with programmatic dependent launch: in the table form for 8-bit codes and with 16-bit
+ * codes the product (fp32 partial sums per slice, and per codebook with 8-bit codes, into the
+ * workspace) and a split-K reduction that sums each row's partials, scales it and writes y; in the
+ * tensor-memory form with bf16 activations the copy of x and the product; otherwise one kernel. Each
+ * waits for the preceding grid before reading activations. The sums are added in a fixed order, so the
+ * result does not depend on scheduling.
  * Accuracy: relative Frobenius error <= 2e-3 and |y - y_exact| <= 1e-2*(1+|y_exact|) per
  * element, with y_exact the fp64 product of the exactly widened stored values, on unit-scale
  * inputs (activations of order 1, codebook entries of the order of N(0, 0.02^2), as in the
- * benchmark layers); in terms of the inputs, fp32 accumulation of exact products: about
- * 2^-15 * |s[o]| * sum_i |x_i| sum_k |C_k[b_k]_i| at most (2^-11 where weights are rounded), and
- * one rounding to a 16-bit y. */
+ * benchmark layers). In terms of A = |s[o]| * sum_i |x_i| sum_k |C_k[b_k]_i|, apart from one rounding
+ * to a 16-bit y: up to batch 4, with one book and with 4-bit codes, exact products in sums of at most
+ * 64 and fp32 additions of those (relative Frobenius error 0.7e-7 to 2e-7 on the benchmark layers); with
+ * two or more 8-bit books at batch 5..16, exact products accumulated by the tensor cores, which
+ * truncate after every 16 of them, over at most S * m / 16 + 1 units of 16 steps (S = ceil(d_in / 256)): at
+ * most (S * m + 16) * 2^-23 A; in the tensor-memory form 2^-11 A for the weights and at most
+ * d_in / 16 * 2^-23 A for the sums. */
 size_t aq_gemv_workspace_bytes(const aq_layout* layout, int batch);
 aq_status aq_gemv(const aq_layout* layout, int m, const void* planes, const void* books,
                   const void* scales, const void* x, int x_dtype, int batch, void* y,

@@ -1056,18 +1056,20 @@ aq_status run_gemm_dense(const Dims& d, int m, const void* planes, const void* b
 // of the pair kernel with decoding in its loop, below the length at which W_m is decoded once. The
 // pair kernel's waves (76 pairs or 36 clusters of four on 152 SMs) times 64-input stages, measured:
 // 1110 / 1850 / 2200 clocks a stage for m = 1 / 3 / 4 with one pair, 1250 / 1690 for m = 2 / 4 with
-// two. (14336 x 4096, m = 4: 31.7 against 79.4 us at 100 tokens, 73.1 against 81.8 at 512; m = 1:
-// 54.0 against 45.3 at 512, where the pair kernel stays; 4096 x 14336, m = 3, 100 tokens: 27.5
-// against 211.) 4-bit layouts have no in-loop form; their other way, decoding W_m first, costs about
-// 15000 clocks and 2 bytes per weight of HBM more than its product. Five and more books leave too
-// little shared memory for the activation stages of more than a few tokens.
+// two. (14336 x 4096, m = 4: 30.8 against 79.4 us at 100 tokens, 74.3 against 82.9 at 512; m = 1:
+// 54.0 against 45.3 at 512, where the pair kernel stays; 4096 x 14336, m = 3, 100 tokens: 26.9
+// against 213.) 4-bit layouts have no in-loop form; their other way, decoding W_m first, costs about
+// 15000 clocks and 2 bytes per weight of HBM more than its product. Five and more books stay with the
+// pair kernel: above 16 tokens neither estimate has been measured for them.
 bool gemm_uses_ts(const Dims& d, int m, int tokens) {
-    if (tokens >= kGemmDenseTokens || m > 4) return false;
+    DeviceInfo di;
+    if (tokens >= kGemmDenseTokens || m > 4 || device_info(&di) != AQ_OK) return false;
     const double ts = ts_clocks(d, m, tokens);
     if (ts < 0.0) return false;
     const int np = d.B == 4 ? 1 : gemm_pairs_per_cluster(m, tokens);
     const long long clusters = (long long)((d.out + kBN - 1) / kBN) * ((tokens + np * kPairTokens - 1) / (np * kPairTokens));
-    const long long waves = np == 1 ? (clusters + 75) / 76 : (clusters + 35) / 36;
+    const long long at_once = np == 1 ? di.sms / 2 : di.sms * 9 / 38;
+    const long long waves = (clusters + at_once - 1) / at_once;
     const double loop = np == 1 ? (m == 1 ? 1110.0 : 740.0 + 365.0 * m) : 810.0 + 220.0 * m;
     const double stage = d.B == 4 ? 1100.0 : loop, extra = d.B == 4 ? 15000.0 + (double)d.out * d.in / 1500.0 : 0.0;
     return ts < waves * (((d.in + kBK - 1) / kBK) * stage + 12000.0) + extra;

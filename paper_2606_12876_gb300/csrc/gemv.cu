@@ -1043,10 +1043,13 @@ static bool gemv_uses_lut4(const Dims& d, int m, int batch, int x_dt) {
 }
 
 // Whether a call runs in one kernel (gemv_cw, or gemm_ts for 9..16 tokens): 4-bit codes at two and more
-// tokens, 8-bit codes at three and more (but see gemv_uses_lut4), and at one token on small layers, with at most half a unit (slice,
-// book) per warp of a CTA and 64 row blocks. There the table kernel and its reduction take 4.0 us and two
-// launches, this one 3.75 us and one launch (1024 x 1024, m = 2: an eager call 9.3 against 12.9 us); with
-// 128 row blocks it is 4.3 against 3.95 us.
+// tokens, 8-bit codes at three and more (but see gemv_uses_lut4), and at one token on small layers, of at most
+// eight units (slice, book) and 64 row blocks. Table kernel and reduction against this one, one token, in a graph,
+// fp16 / bf16 x, and eager: 1024 x 1024, m = 2 (8 units) 4.0 / 4.0 us and 13.0 against 3.2 / 4.0 and 10.2; m = 4 (16)
+// 4.0 / 4.1 against 3.5 / 4.1; 1024 x 2048, m = 3 (24) 4.1 / 4.1 against 4.4 / 5.1; 4096 x 1024 (128 row blocks),
+// m = 2 4.2 / 4.1 against 4.0 / 4.7. Units end at eight, not at sixteen: with sixteen the key and value projections
+// of a 4096-input block (one book) would leave the launch that the tables share with the query projection
+// (4096, 1024 and 1024 rows, 2048 inputs, m = 1: 5.8 us shared, 7.9 parted).
 static bool gemv_uses_cw(const Dims& d, int m, int batch, int x_dt) {
     if (d.B == 4) return batch >= 2;
     if (d.B != 8) return false;
