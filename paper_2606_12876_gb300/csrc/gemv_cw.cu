@@ -180,8 +180,8 @@ struct RowCodes {
 
 // CHAIN: multiplies (of 16 inputs) that the tensor pipe accumulates before an fp32 addition takes them over. The
 // pipe truncates as it accumulates, so the longer the chain, the larger the error of an fp32 y:
-//   1: the two multiplies of a step are added, then the steps of a unit, then the units of a warp: as accurate as
-//      the table kernel's fp32 sums (1.0 times its error at 1024 x 1024, 0.7 to 0.9 on longer rows);
+//   1: the two multiplies of a step are added, then the steps of a unit, the units of a warp, and the warps in
+//      pairs: as accurate as the table kernel's fp32 sums (0.7 to 1.05 times its error);
 //   4: two steps: 0.5 to 0.95 times the error of fp32 sums in input order;
 //   0: all units of a warp (4096 x 14336, m = 1 / 4: 1.1e-6 / 4.3e-6).
 template <int B, int BDT, int XDT, int CHAIN>
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     int pass = 0;
     for (int rb = cid; rb < L.RBc; rb += L.nclusters, ++pass) {
         float acc[2][4];
-        // The warps' sums of a pass, added in warp order. Two buffers: a pass's writes meet the sums
+        // The warps' sums of a pass, added in warp order or (CHAIN) in pairs. Two buffers: a pass's writes meet the sums
         // that are read two passes earlier, which every thread finished before the last barrier.
         float* rp = red + (pass & 1) * kCwRedFloats;
         float* mine = rp + (size_t)warp * kCwTokens * kCwPitch;
@@ -394,14 +394,20 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
         float* cs = csum + (pass & 1) * 32 * kCwTokens;
         float v = 0.0f;
         if (tid < 32 * kCwTokens) {
-            float t[kCwWarps];
+            const float* p = rp + (tid >> 5) * kCwPitch + (tid & 31);
+            if constexpr (CHAIN == 0) {
 #pragma unroll
-            for (int w = 0; w < kCwWarps; ++w) t[w] = rp[((size_t)w * kCwTokens + (tid >> 5)) * kCwPitch + (tid & 31)];
+                for (int w = 0; w < kCwWarps; ++w) v += p[w * kCwTokens * kCwPitch];
+            } else {
+                float t[kCwWarps];
 #pragma unroll
-            for (int n = kCwWarps / 2; n > 0; n /= 2)
+                for (int w = 0; w < kCwWarps; ++w) t[w] = p[w * kCwTokens * kCwPitch];
 #pragma unroll
-                for (int w = 0; w < n; ++w) t[w] = t[2 * w] + t[2 * w + 1];
-            v = t[0];
+                for (int n = kCwWarps / 2; n > 0; n /= 2)
+#pragma unroll
+                    for (int w = 0; w < n; ++w) t[w] = t[2 * w] + t[2 * w + 1];
+                v = t[0];
+            }
             if (a.kc > 1) cs[tid] = v;
         }
         if (a.kc > 1) {
