@@ -131,8 +131,9 @@ aq_status aq_decode(const aq_layout* layout, int m, const void* planes, const vo
  * codewords themselves (batch above, and small layers at batch 1; where the books and the
  * activations differ in type, the bf16 side is scaled by powers of two into fp16, over all of bf16's
  * range, which is exact for values within 2^29 of the largest finite one of their book set, or of their
- * token and slice). Larger layers with two or more 8-bit books at batch 9..16 run the tensor-memory
- * kernel of aq_gemm: decoded weights rounded once to fp16, bf16 activations scaled by token.
+ * token and slice). Larger layers with 8-bit codes at batch 9..16 run the tensor-memory kernel of
+ * aq_gemm (one book only with a 16-bit y): sums of two or more codewords rounded once to fp16, bf16
+ * activations scaled by token.
  *   x         : device, [batch][d_in] of x_dtype (AQ_F16 or AQ_BF16), row-major
  *   y         : device, [batch][d_out] of y_dtype (AQ_F16, AQ_BF16 or AQ_F32), row-major
  *   workspace : device scratch of at least aq_gemv_workspace_bytes(layout, batch) bytes:
@@ -152,7 +153,7 @@ aq_status aq_decode(const aq_layout* layout, int m, const void* planes, const vo
  * element, with y_exact the fp64 product of the exactly widened stored values, on unit-scale
  * inputs (activations of order 1, codebook entries of the order of N(0, 0.02^2), as in the
  * benchmark layers). In terms of A = |s[o]| * sum_i |x_i| sum_k |C_k[b_k]_i|, apart from one rounding
- * to a 16-bit y: up to batch 4, with one book and with 4-bit codes, exact products in sums of at most
+ * to a 16-bit y: up to batch 4, with one book (fp32 y) and with 4-bit codes, exact products in sums of at most
  * 64 and fp32 additions of those (relative Frobenius error 0.7e-7 to 2e-7 on the benchmark layers); with
  * two or more 8-bit books at batch 5..16, exact products accumulated by the tensor cores, which
  * truncate after every 16 of them, over at most S * m / 16 + 1 units of 16 steps (S = ceil(d_in / 256)): at

@@ -1062,10 +1062,11 @@ static bool gemv_uses_cw(const Dims& d, int m, int batch, int x_dt) {
 // clocks), which has room unless the layer has few rows. Over 256 to 14336 rows, 1024 to 14336 inputs and two to
 // five books the choice costs at most 11 % of the faster one. 16 tokens, fp16 x: 14336 x 4096, m = 4 24.8 us (gemv_cw
 // 41.3); 4096 x 4096, m = 4 11.5 (15.6); but 1024 x 4096, m = 2 8.2 against gemv_cw's 5.4, 1024 x 8192, m = 4
-// 19.2 against 10.6. 8-bit codes and several books only: with 4-bit codes or one book every intermediate of a
-// GEMV is fp32 or exact, and stays so.
-static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt) {
-    if (batch <= 8 || d.B != 8 || m == 1) return false;
+// 19.2 against 10.6. 8-bit codes only, and an fp32 y only with several books: with 4-bit codes or one book every
+// intermediate of the other forms is fp32 or exact (one book: the tensor cores' chain over all of K leaves 4.9e-6 in an
+// fp32 y, 0.03 % of the rounding of a 16-bit one; 4096 x 14336, 16 tokens, bf16 15.3 us, gemv_cw 24.1).
+static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt, int y_dt) {
+    if (batch <= 8 || d.B != 8 || (m == 1 && y_dt == AQ_F32)) return false;
     const size_t room = gemv_ws_planes(d, batch) * (size_t)d.rows_pad * 4;
     if (x_dt == AQ_BF16 && room < kWsStatusBytes + (size_t)batch * d.in * 2) return false;
     const double ts = ts_clocks(d, m, batch);
@@ -1098,7 +1099,7 @@ aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* book
     if (d.B == 4 && batch == 1)
         return launch_lut4(d, m, planes, books, scales, x, x_dt, y, y_dt, y_prev, st);
     if (gemv_uses_cw(d, m, batch, x_dt)) {
-        if (!y_prev && gemv_uses_ts(d, m, batch, x_dt))
+        if (!y_prev && gemv_uses_ts(d, m, batch, x_dt, y_dt))
             return launch_gemv_ts(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, ws, status, st);
         return launch_cw(&d, 1, m, &planes, &books, &scales, x, x_dt, batch, &y, y_dt, y_prev, st);
     }
@@ -1136,7 +1137,7 @@ aq_status launch_gemv_group(const Dims* ds, int n, int m, const void* const* pla
     } parts[kForms] = {};
     for (int l = 0; l < n; ++l) {
         if (ds[l].out == 0) continue;
-        const int form = gemv_uses_cw(ds[l], m, batch, x_dt) ? (gemv_uses_ts(ds[l], m, batch, x_dt) ? kTs : kCw)
+        const int form = gemv_uses_cw(ds[l], m, batch, x_dt) ? (gemv_uses_ts(ds[l], m, batch, x_dt, y_dt) ? kTs : kCw)
                          : ds[l].B == 8 && batch == 1        ? kTables
                                                              : kOther;
         Part& p = parts[form];

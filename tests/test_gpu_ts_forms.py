@@ -59,7 +59,8 @@ def test_form(quarters, cluster, out, inp, m, tokens):
     (1024, 1024, 2, 8, 3, ["gemv_cw_kernel"]),
     (4096, 4096, 4, 8, 8, ["gemv_cw_kernel"]),
     (4096, 4096, 4, 8, 9, ["gemm_ts_kernel"]),
-    (4096, 4096, 1, 8, 9, ["gemv_cw_kernel"]),                            # one book: exact weights
+    (4096, 4096, 1, 8, 9, ["gemv_cw_kernel"]),                            # one book, fp32 y: exact weights, fp32 sums
+    (14336, 2048, 1, 8, 16, ["gemm_ts_kernel"]),                          # one book, 16-bit y
     (1024, 1024, 4, 8, 16, ["gemv_cw_kernel"]),
     (1024, 1024, 4, 4, 1, ["gemv_lut4_kernel"]),
     (4096, 4096, 4, 4, 16, ["gemv_cw_kernel"]),                           # 4-bit codes: no rounded weights
@@ -67,10 +68,11 @@ def test_form(quarters, cluster, out, inp, m, tokens):
 def test_gemv_kernel(out, inp, m, B, batch, names):
     lin = AQLinear.from_layer(workloads.make_layer(out, inp, G=8, M=4, B=B, book_dtype="f16", scale_dtype="f16", seed=1))
     x = x_to_device(workloads.make_x(batch, inp, "f16", seed=2), "f16")
-    y = torch.empty(batch, out, dtype=torch.float16, device="cuda")
+    yd = aq.AQ_F32 if m == 1 and names == ["gemv_cw_kernel"] else aq.AQ_F16
+    y = torch.empty(batch, out, dtype=torch.float32 if yd == aq.AQ_F32 else torch.float16, device="cuda")
     if all_sms():
-        assert [k[0] for k in kernels(lambda: lin.gemv(x, m, y=y))] == names
-    lin.gemv(x, m, y=y)
+        assert [k[0] for k in kernels(lambda: lin.gemv(x, m, y=y, y_dtype=yd))] == names
+    lin.gemv(x, m, y=y, y_dtype=yd)
     W = lin.decode(m).double()                # one rounding of a weight to fp16, one of y, fp32 sums
     ref, bound = x.double() @ W.t(), 2.0 ** -9 * (x.double().abs() @ W.abs().t())
     assert bool(((y.double() - ref).abs() <= bound + 1e-6).all())
