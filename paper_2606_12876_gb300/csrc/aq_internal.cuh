@@ -102,7 +102,7 @@ aq_status launch_gemv(const Dims& d, int m, const void* planes, const void* book
 aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, const void* const* books,
                     const void* const* scales, const void* x, int x_dt, int batch, void* const* y, int y_dt,
                     const void* y_prev, cudaStream_t st);
-double cw_clocks(const Dims& d, int m, int batch);   // its estimated time in clocks, without the launch
+double cw_clocks(const Dims& d, int m, int batch, int x_dt);   // its estimated time in clocks, without the launch
 // The product with the decoded weights in tensor memory (gemm_ts.cu): its estimated time in clocks
 // (below 0: not served), and the launch, of n (<= 4) layers as above (x: fp16; xfac: per-token factors
 // or null; ws: its first word is the status word).

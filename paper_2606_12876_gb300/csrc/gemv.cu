@@ -1038,8 +1038,7 @@ static bool gemv_uses_lut4(const Dims& d, int m, int batch, int x_dt) {
     if (d.B != 8 || m > 4 || batch < 3 || batch > 4 || d.S * m < 48 || device_info(&di) != AQ_OK || d.RBc <= di.sms)
         return false;
     const double lut = 11200.0 + 185.0 * d.S * m * d.RBc / di.sms;
-    const double mixed = d.book_dt == AQ_F16 && x_dt == AQ_BF16 ? 500.0 * ((d.RBc - 1) / di.sms + 1) * ((d.S + 15) / 16) : 0.0;
-    return lut < cw_clocks(d, m, batch) + 2850.0 + mixed;
+    return lut < cw_clocks(d, m, batch, x_dt) + 2850.0;
 }
 
 // Whether a call runs in one kernel (gemv_cw, or gemm_ts for 9..16 tokens): 4-bit codes at two and more
@@ -1058,7 +1057,7 @@ static bool gemv_uses_cw(const Dims& d, int m, int batch, int x_dt) {
 
 // Whether 9..16 tokens run the tensor-memory kernel (gemm_ts.cu): where its estimated time is below that of
 // gemv_cw with two token tiles, which gathers every codeword twice. Both estimates leave out the launch; gemm_ts's
-// is about 1500 clocks high at 16 tokens, and bf16 activations are copied to the workspace first (about 3000
+// is about 2000 clocks high at 16 tokens, and bf16 activations are copied to the workspace first (about 3000
 // clocks), which has room unless the layer has few rows. Over 256 to 14336 rows, 1024 to 14336 inputs and two to
 // five books the choice costs at most 11 % of the faster one. 16 tokens, fp16 x: 14336 x 4096, m = 4 24.8 us (gemv_cw
 // 41.3); 4096 x 4096, m = 4 11.5 (15.6); but 1024 x 4096, m = 2 8.2 against gemv_cw's 5.4, 1024 x 8192, m = 4
@@ -1071,7 +1070,7 @@ static bool gemv_uses_ts(const Dims& d, int m, int batch, int x_dt, int y_dt) {
     if (x_dt == AQ_BF16 && room < kWsStatusBytes + (size_t)batch * d.in * 2) return false;
     const double ts = ts_clocks(d, m, batch);
     if (ts < 0.0) return false;
-    return ts + (x_dt == AQ_BF16 ? 3000.0 : 0.0) < cw_clocks(d, m, batch) + 1500.0;
+    return ts + (x_dt == AQ_BF16 ? 3000.0 : 0.0) < cw_clocks(d, m, batch, x_dt) + 2000.0;
 }
 
 // The tensor-memory kernel for n layers that share x; ws0: the first layer's workspace, whose partial-sum

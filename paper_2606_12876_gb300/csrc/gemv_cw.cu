@@ -438,16 +438,19 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
 // Copies of a codebook (log2): eight while they fit next to the sums, else four.
 inline int cw_cshift(int B, int m) { return B == 4 || m <= 5 ? 3 : 2; }
 
-// CTAs per cluster: the split with the smallest estimated time of the busiest cluster, in clocks:
-// passes over its row blocks times the units of a warp (a unit's gathers are 128 wavefronts, about
-// twice that with four copies of a book, plus staging, conversions and sums, shared by the SM's
-// active warps, or about 2000 clocks of latencies where few are) and 1500 to 2200 clocks of reduction and
-// start-up a pass, plus what a cluster launch and its barriers cost over a plain one: 600, 1000 and 2000 clocks
-// for 2, 4 and 8 CTAs, and 2400 and 2000 more for 2 and 4 where the call's CTAs exceed half of the SMs (its
-// clusters then wait for those of the preceding kernel). Measured with the cluster size given, 8-bit
-// codes, 3 tokens, fp16 x, clusters of 1 / 2 / 4 / 8: 256 x 8192, m = 1 5.5 / 4.6 / 4.4 / 4.7 us, m = 4
-// 15.1 / 9.5 / 6.4 / 5.3; 1024 x 4096, m = 1 3.6 / 4.4 / 5.2 / 11.3, m = 4 8.6 / 6.4 / 6.1 / 14.9; 32 x 32768,
-// m = 1 16.7 / 10.2 / 6.5 / 4.5.
+// CTAs per cluster: the split with the smallest estimated time of the busiest cluster, in clocks: passes over its
+// row blocks times
+//  * the gathers of a CTA's units: 185 clocks each with 8-bit codes (128 wavefronts, staging, sums), 160 with 4-bit
+//    codes, 300 with four copies of a book, at least 2500 for each unit of a warp; where no warp has a second unit
+//    1700 and about half of the gathers;
+//  * 1500 to 2200 clocks of reduction and start-up (1000 less where one pass and one unit are all);
+//  * the activations of a warp's further slices (64 bytes a clock and SM), and 800 clocks a slice if they are scaled;
+// plus what a cluster launch and its barriers cost over a plain one: 600, 1000 and 1900 clocks for 2, 4 and 8 CTAs,
+// 3000 and 2600 for 2 and 4 where the call's CTAs exceed half of the SMs (its clusters then wait for those of
+// the preceding kernel). Within 6 % of most calls measured with the cluster size given; clusters of 1 / 2 / 4 / 8,
+// 8-bit codes, 3 tokens, fp16 x: 256 x 8192, m = 1 5.5 / 4.6 / 4.4 / 4.7 us, m = 4 15.1 / 9.5 / 6.4 / 5.3; 1024 x 4096,
+// m = 1 3.6 / 4.4 / 5.2 / 11.3, m = 4 8.6 / 6.4 / 6.1 / 14.9; 32 x 32768, m = 1 16.7 / 10.2 / 6.5 / 4.5; 256 x 1024, m = 5
+// 5.0 / 4.3 / 3.6 / 4.4.
 // Clusters of 2, 4 and 8 that are resident at once: 76, 36 and (beside the preceding call's) 8 on 152 SMs;
 // sixteen clusters of eight took twice the time of eight (512 x 8192, m = 1: 8.8 us). With several token tiles
 // each tile has its share of the SMs.
@@ -456,7 +459,9 @@ inline int cw_clusters(int kc, int tiles, int sms) {
     const int n = (kc == 1 ? sms : kc == 2 ? sms / 2 : kc == 4 ? sms * 9 / 38 : sms / 19) / tiles;
     return n < 1 ? 1 : n;
 }
-inline int cw_cluster(const Dims& d, int m, int tiles, int sms, int* nclusters, double* clocks) {
+inline int cw_cluster(const Dims& d, int m, int batch, int x_dt, int sms, int* nclusters, double* clocks) {
+    const int tiles = cw_tiles(batch);
+    const bool scaled = d.book_dt == AQ_F16 && x_dt == AQ_BF16;
     int best = 1;
     double best_t = -1.0;
     for (int kc = 1; kc <= 8; kc *= 2) {
@@ -464,12 +469,16 @@ inline int cw_cluster(const Dims& d, int m, int tiles, int sms, int* nclusters, 
         if (nc > d.RBc) nc = d.RBc;
         const long long U = (long long)d.S * m;
         const long long units = (U + 16 * kc - 1) / (16 * kc);
-        const long long active = U < 16 * kc ? (U + kc - 1) / kc : 16;
         const double gather = cw_cshift(d.B, m) != 3 ? 300.0 : d.B == 8 ? 185.0 : 160.0;
-        const double unit_clk = active * gather > 2000.0 ? active * gather : 2000.0;
+        const double all = (double)((U + kc - 1) / kc) * gather, least = units * 2500.0;
+        const double work = units == 1 ? 1700.0 + 0.55 * all : all > least ? all : least;
         const bool wide = 2 * nc * kc * tiles > sms;
-        const double cluster = kc == 1 ? 0.0 : kc == 2 ? (wide ? 3000.0 : 600.0) : kc == 4 ? (wide ? 3000.0 : 1000.0) : 2000.0;
-        const double t = (double)((d.RBc + nc - 1) / nc) * (units * unit_clk + (kc > 1 ? 2200.0 : 1500.0)) + cluster;
+        const double cluster = kc == 1 ? (units == 1 ? -1000.0 : 0.0) : kc == 2 ? (wide ? 3000.0 : 600.0)
+                               : kc == 4 ? (wide ? 2600.0 : 1000.0) : 1900.0;
+        const double slices = units > m ? (double)units / m : 1.0;    // of a warp
+        const double x_clk = d.in * 2.0 * (batch < kCwTokens ? batch : kCwTokens) / kc / 64.0 * (1.0 - 1.0 / slices) +
+                             (scaled ? 800.0 * slices : 0.0);
+        const double t = (double)((d.RBc + nc - 1) / nc) * (work + x_clk + (kc > 1 ? 2200.0 : 1500.0)) + cluster;
         if (best_t < 0.0 || t < best_t) {
             best_t = t;
             best = kc;
@@ -510,11 +519,11 @@ aq_status run_cw_types(const CwArgs& a, int book_dt, int x_dt, cudaStream_t st) 
 
 }  // namespace
 
-double cw_clocks(const Dims& d, int m, int batch) {
+double cw_clocks(const Dims& d, int m, int batch, int x_dt) {
     DeviceInfo di;
     int nc;
     double t = -1.0;
-    if (device_info(&di) == AQ_OK) cw_cluster(d, m, cw_tiles(batch), di.sms, &nc, &t);
+    if (device_info(&di) == AQ_OK) cw_cluster(d, m, batch, x_dt, di.sms, &nc, &t);
     return t;
 }
 
@@ -527,7 +536,7 @@ aq_status launch_cw(const Dims* ds, int n, int m, const void* const* planes, con
     int kcs[4], own[4];
     const int tiles = cw_tiles(batch);
     double clocks;
-    for (int l = 0; l < n; ++l) kcs[l] = cw_cluster(ds[l], m, tiles, di.sms, &own[l], &clocks);
+    for (int l = 0; l < n; ++l) kcs[l] = cw_cluster(ds[l], m, batch, x_dt, di.sms, &own[l], &clocks);
     bool done[4] = {};
     for (int f = 0; f < n; ++f) {
         if (done[f]) continue;
