@@ -421,8 +421,9 @@ def measure_beam(lin, layer, dev, stream, sm_mhz, K=8, reps=3):
     groups = out * (inp // 8)
     nb = 1 << B
     cands = nb + (M - 1) * K * nb                      # candidates scored per group
-    # per candidate: d (8 FMA), S_gg d (64 FMA), d.(S_gg d) and d.h (16 FMA), score (2)
-    cand_flops = 2 * (8 + 64 + 16) + 2
+    # per candidate what ranking it cannot do without: its eight elements against a vector of the state (8 FMA);
+    # the definition (d, S_gg d, d.(S_gg d), d.h: 90 FMA) is evaluated for the few that the estimate leaves
+    cand_flops = 2 * 8
     gemm_flops = 2.0 * M * out * inp * inp             # E_k S for every prefix
     flops = groups * cands * cand_flops + gemm_flops
     changed = float((new != codes).any(dim=2).float().mean())

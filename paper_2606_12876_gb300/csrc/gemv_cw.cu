@@ -451,6 +451,9 @@ inline int cw_cshift(int B, int m) { return B == 4 || m <= 5 ? 3 : 2; }
 // 8-bit codes, 3 tokens, fp16 x: 256 x 8192, m = 1 5.5 / 4.6 / 4.4 / 4.7 us, m = 4 15.1 / 9.5 / 6.4 / 5.3; 1024 x 4096,
 // m = 1 3.6 / 4.4 / 5.2 / 11.3, m = 4 8.6 / 6.4 / 6.1 / 14.9; 32 x 32768, m = 1 16.7 / 10.2 / 6.5 / 4.5; 256 x 1024, m = 5
 // 5.0 / 4.3 / 3.6 / 4.4.
+// Clusters are taken for a gain of 1050 clocks or more only: layers of a group share a launch where their sizes
+// agree, and one more launch costs about 3 us (hidden 2800, m = 2, 4-bit codes, 5 tokens, block: 29.0 us with
+// the key and value projections in clusters of two, 25.4 without; but 256 x 1024, m = 5 gains 1.3 us in fours).
 // Clusters of 2, 4 and 8 that are resident at once: 76, 36 and (beside the preceding call's) 8 on 152 SMs;
 // sixteen clusters of eight took twice the time of eight (512 x 8192, m = 1: 8.8 us). With several token tiles
 // each tile has its share of the SMs.
@@ -479,7 +482,7 @@ inline int cw_cluster(const Dims& d, int m, int batch, int x_dt, int sms, int* n
         const double x_clk = d.in * 2.0 * (batch < kCwTokens ? batch : kCwTokens) / kc / 64.0 * (1.0 - 1.0 / slices) +
                              (scaled ? 800.0 * slices : 0.0);
         const double t = (double)((d.RBc + nc - 1) / nc) * (work + x_clk + (kc > 1 ? 2200.0 : 1500.0)) + cluster;
-        if (best_t < 0.0 || t < best_t) {
+        if (best_t < 0.0 || t + (best == 1 ? 1050.0 : 0.0) < best_t) {
             best_t = t;
             best = kc;
             *nclusters = nc;
@@ -500,13 +503,14 @@ aq_status run_cw(CwArgs a, cudaStream_t st) {
     return launch_pdl_cluster(a.kc, kern, dim3((last.c0 + last.nclusters) * a.kc, cw_tiles(a.batch)), dim3(kCwThreads), smem, st, a);
 }
 
-// The chain by what the other forms of the product give: 8-bit codes have fp32 tables up to two tokens, and one
-// book's codewords are exact everywhere; sums of several books from five tokens are otherwise rounded to 11 bits
-// (2e-4), where any chain will do. 4-bit codes: fp32 sums over the inputs in order (2 to 3e-7).
+// The chain by what the other forms of the product give. 8-bit codes have fp32 tables up to four tokens. From five,
+// sums of several books are rounded to 11 bits in the other forms (2e-4), where any chain will do; one book's
+// codewords are exact there, in sums with errors of 3.0e-7 to 6.4e-7: the pipe's chain over one unit stays below that
+// (2.4e-7 to 3.5e-7), but not over two. 4-bit codes: fp32 sums over the inputs in order (2 to 3e-7).
 template <int B, int BDT, int XDT>
 aq_status run_cw_chain(const CwArgs& a, cudaStream_t st) {
     if constexpr (B == 4) return run_cw<B, BDT, XDT, 4>(a, st);
-    else if (a.batch <= 4 || a.m == 1) return run_cw<B, BDT, XDT, 1>(a, st);
+    else if (a.batch <= 4 || (a.m == 1 && a.S > kCwWarps * a.kc)) return run_cw<B, BDT, XDT, 1>(a, st);
     else return run_cw<B, BDT, XDT, 0>(a, st);
 }
 
