@@ -209,12 +209,15 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
     const long long U = (long long)a.S * a.m;
     const int nwarps = kCwWarps * a.kc, gw = rank * kCwWarps + warp;
     const int u0 = (int)(U * gw / nwarps), u1 = (int)(U * (gw + 1) / nwarps);
+    const int sk0 = (u0 / a.m) << 3 | (u0 % a.m);             // slice and book of u0 (m <= 8)
     struct Item {
         int rb, u, s, k;
     };
     auto next_item = [&](Item& it) {
         if (++it.u == u1) {
-            it = Item{it.rb + L.nclusters, u0, u0 / a.m, u0 % a.m};
+            // (a division per pass costs 1 % of a call; where the sums take registers, one for it costs as much)
+            if constexpr (CHAIN == 0) it = Item{it.rb + L.nclusters, u0, sk0 >> 3, sk0 & 7};
+            else it = Item{it.rb + L.nclusters, u0, u0 / a.m, u0 % a.m};
         } else if (++it.k == a.m) {
             it.k = 0;
             ++it.s;
@@ -229,7 +232,7 @@ __global__ void __launch_bounds__(kCwThreads, 1) gemv_cw_kernel(const __grid_con
             if constexpr (B == 8) raw[1] = ld_stream_v4(src + 16);
         }
     };
-    Item nxt{cid, u0, u0 / a.m, u0 % a.m};
+    Item nxt{cid, u0, sk0 >> 3, sk0 & 7};
     float bfac = 1.0f;                                   // 2^f of the staged books (kScaleB)
     auto stage_books = [&]() {
         if constexpr (kScaleB) {
