@@ -454,9 +454,10 @@ inline int cw_cshift(int B, int m) { return B == 4 || m <= 5 ? 3 : 2; }
 // 8-bit codes, 3 tokens, fp16 x: 256 x 8192, m = 1 5.5 / 4.6 / 4.4 / 4.7 us, m = 4 15.1 / 9.5 / 6.4 / 5.3; 1024 x 4096,
 // m = 1 3.6 / 4.4 / 5.2 / 11.3, m = 4 8.6 / 6.4 / 6.1 / 14.9; 32 x 32768, m = 1 16.7 / 10.2 / 6.5 / 4.5; 256 x 1024, m = 5
 // 5.0 / 4.3 / 3.6 / 4.4.
-// Clusters are taken for a gain of 1050 clocks or more only: layers of a group share a launch where their sizes
-// agree, and one more launch costs about 3 us (hidden 2800, m = 2, 4-bit codes, 5 tokens, block: 29.0 us with
-// the key and value projections in clusters of two, 25.4 without; but 256 x 1024, m = 5 gains 1.3 us in fours).
+// Clusters are taken for a gain of 1400 clocks or more only: layers of a group share a launch where their sizes
+// agree, and one more launch costs about 3 us (block of hidden 2800, m = 2, 4-bit codes, 5 tokens: 29.0 us with
+// the key and value projections in clusters of two, 25.4 without; but 256 x 1024, m = 5 by itself takes 4.9 us
+// where clusters of four take 3.6).
 // Clusters of 2, 4 and 8 that are resident at once: 76, 36 and (beside the preceding call's) 8 on 152 SMs;
 // sixteen clusters of eight took twice the time of eight (512 x 8192, m = 1: 8.8 us). With several token tiles
 // each tile has its share of the SMs.
@@ -485,7 +486,7 @@ inline int cw_cluster(const Dims& d, int m, int batch, int x_dt, int sms, int* n
         const double x_clk = d.in * 2.0 * (batch < kCwTokens ? batch : kCwTokens) / kc / 64.0 * (1.0 - 1.0 / slices) +
                              (scaled ? 800.0 * slices : 0.0);
         const double t = (double)((d.RBc + nc - 1) / nc) * (work + x_clk + (kc > 1 ? 2200.0 : 1500.0)) + cluster;
-        if (best_t < 0.0 || t + (best == 1 ? 1050.0 : 0.0) < best_t) {
+        if (best_t < 0.0 || t + (best == 1 ? 1400.0 : 0.0) < best_t) {
             best_t = t;
             best = kc;
             *nclusters = nc;
