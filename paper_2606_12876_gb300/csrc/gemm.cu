@@ -1056,7 +1056,7 @@ aq_status run_gemm_dense(const Dims& d, int m, const void* planes, const void* b
 // of the pair kernel with decoding in its loop, below the length at which W_m is decoded once. The
 // pair kernel's waves (76 pairs or 36 clusters of four on 152 SMs) times 64-input stages, measured:
 // 1110 / 1850 / 2200 clocks a stage for m = 1 / 3 / 4 with one pair, 1250 / 1690 for m = 2 / 4 with
-// two. (14336 x 4096, m = 4: 30.8 against 79.4 us at 100 tokens, 74.3 against 82.9 at 512; m = 1:
+// two. (14336 x 4096, m = 4: 31.0 against 79.4 us at 100 tokens, 74.5 against 82.9 at 512; m = 1:
 // 54.0 against 45.3 at 512, where the pair kernel stays; 4096 x 14336, m = 3, 100 tokens: 26.9
 // against 213.) 4-bit layouts have no in-loop form; their other way, decoding W_m first, costs about
 // 15000 clocks and 2 bytes per weight of HBM more than its product. Five and more books stay with the

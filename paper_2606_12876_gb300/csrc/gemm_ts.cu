@@ -25,8 +25,8 @@
 // once its MMAs completed) and each finishes a share of the tokens, adding the CTAs' sums in rank
 // order.
 // Measured (the call, with the copy of bf16 activations), against the pair kernel: 4096 x 14336, m = 3,
-// 100 tokens 26.8 / 213 us; 14336 x 4096, m = 4, 100 tokens 30.8 / 79.4 us, 512 tokens 74 / 83 us; 16 tokens,
-// m = 4: 27.6 us against 54.9 of the tf32 kernel before and 47.7 of gemv_cw. Five to eight books,
+// 100 tokens 26.9 / 213 us; 14336 x 4096, m = 4, 100 tokens 31.0 / 79.4 us, 512 tokens 74.5 / 83 us; 16 tokens,
+// m = 4: 27.7 us against 54.9 of the tf32 kernel before and 42.8 of gemv_cw. Five to eight books,
 // 14336 x 4096, 16 tokens: 32 / 37 / 56 / 64 us (tf32 kernel: 66 / 77 / 88 / 179).
 // Roles: warps 0-15 decoders (warp w: quarter w mod 4, set w / 4; the warps of absent quarters idle)
 // and epilogue; one warp for TMA (and L2 prefetch of the codes), one for MMA issue and the

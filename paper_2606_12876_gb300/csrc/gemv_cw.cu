@@ -36,11 +36,13 @@
 // books with bf16 activations: every (token, slice) of x is scaled by a power of two that puts
 // its largest |x| in [2^14, 2^15) and rounded to fp16, which is exact for values within 2^29 of
 // the largest, and the slice's sums are scaled back when they are added to the total. bf16 books
-// with fp16 activations: the books are scaled the same way (one power of two for the m books).
+// with fp16 activations: the books are scaled the same way (one power of two for the m books, by their
+// largest finite entry).
 //
-// Measured, 8B block (seven layers; q/k/v and gate/up as groups): 8 tokens, m = 3 83.5 us (the eight-token
-// tables and tf32 kernel before: 145.8), 4-bit codes, 4 tokens, m = 4 91.1 us (fp32 kernel before: 229.7).
-// 14336 x 4096, 8 tokens: m = 3 17.8 us, m = 4 22.1 us; 1024 x 1024, m = 4, 16 tokens: 3.9 us.
+// Measured, 8B block (seven layers; q/k/v and gate/up as groups): 8 tokens, m = 3 83.2 us (the eight-token
+// tables and tf32 kernel before: 145.8), 4-bit codes, 4 tokens, m = 4 92.0 us (fp32 kernel before: 229.7).
+// 14336 x 4096, 8 tokens: m = 3 17.8 us, m = 4 22.1 us; 4 tokens (fp32 sums): 18.8, 23.5; 1024 x 1024, m = 4, 16
+// tokens: 3.8 us.
 #include "aq_internal.cuh"
 #include "cw_split.h"
 #include "launch.cuh"
